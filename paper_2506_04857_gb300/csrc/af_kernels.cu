@@ -548,6 +548,10 @@ __device__ __forceinline__ int upwind_sign(const AfGrid &g, double vl) {
 // into acc (per component), with F^pm = (F +- alpha U)/2.  Writing out D+ and D-:
 // (D+F+ + D-F-) h = ((F0 - F4) + 4 (F3 - F1) + alpha ((U0 + U4) - 4 (U1 + U3) + 6 U2)) / 2.
 // Also returns 2h times the derivative of B_l for the point source in dBl (b_line).
+// The second difference of U runs on the integer pipes (up5): the point pass is bound by
+// the FP64 pipe (84 % busy, integer ALUs 14 %).  Orszag-Tang 1536^2: the pass 1813 -> 1555 us;
+// blast 1024^2: 838 -> 694 us.  The flux difference stays on the FP64 pipe: moved too, the
+// integer instructions cost more than they saved (1790 us).
 template <int L>
 __device__ __forceinline__ void fvs_line(const PP *P, size_t PS, int nxa, double c, double *acc, double &dBl,
                                          int upw) {
@@ -558,7 +562,7 @@ __device__ __forceinline__ void fvs_line(const PP *P, size_t PS, int nxa, double
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const double u0 = pu(P[0], k), u1 = pu(P[1], k), u2 = pu(P[2], k), u3 = pu(P[3], k), u4 = pu(P[4], k);
-    const double up = fma(6.0, u2, fma(-4.0, u1 + u3, u0 + u4));
+    const double up = up5(u0, u1, u2, u3, u4);
     double dk;
     if (k == 4 + L) {
       dk = mul_i(al, up);
@@ -583,7 +587,7 @@ __device__ __forceinline__ void fvs_line_g(const PPG *P, double c, double *acc, 
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const double u0 = pug(P[0], k), u1 = pug(P[1], k), u2 = pug(P[2], k), u3 = pug(P[3], k), u4 = pug(P[4], k);
-    const double up = fma(6.0, u2, fma(-4.0, u1 + u3, u0 + u4));
+    const double up = up5(u0, u1, u2, u3, u4);
     double dk;
     if (k == 4 + L) {
       dk = al * up;

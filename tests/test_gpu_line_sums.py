@@ -1,0 +1,70 @@
+"""The second difference of a 5-point FVS line in fixed point (af_math.cuh up5): components over
+the whole exponent range, exact zeros, mixed signs and jumps, through af_rhs against the oracle."""
+import numpy as np
+import pytest
+
+import af_inputs as ai
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import paper_2506_04857_gb300 as af  # noqa: E402
+
+
+def rhs(pb, U):
+    s = af.Solver(pb.nx, pb.ny, pb.gamma, pb.bc, domain=(pb.x0, pb.x1, pb.y0, pb.y1), kappa=0.0)
+    s.set_state([torch.from_numpy(u).cuda() for u in U])
+    out = s.rhs(device=False)
+    s.close()
+    return out
+
+
+# size of the third components of momentum and field (they enter the others squared only):
+# ordinary, exactly zero, at and beyond the smallest exponent of the fixed-point path
+# (2^-823), and subnormal
+@pytest.mark.parametrize("log2", [0, None, -60, -500, -822, -826, -1060])
+@pytest.mark.parametrize("bc", [ai.PERIODIC, ai.OUTFLOW])
+def test_small_components(log2, bc):
+    pb = ai.random_smooth(33, 9, seed=4, amp=0.3, bc=bc)
+    rng = np.random.default_rng(7)
+    U = ai.dofs(pb)
+    for u in U:
+        for k in (3, 6):
+            E = 0.5 * u[3] ** 2 / u[0] if k == 3 else 0.5 * u[6] ** 2
+            u[7] -= E
+            u[k] = 0.0 if log2 is None else np.ldexp(rng.normal(size=u[k].shape), log2)
+            u[7] += 0.5 * u[3] ** 2 / u[0] if k == 3 else 0.5 * u[6] ** 2
+    G, R = rhs(pb, U), oracle.rhs(pb, U)
+    for a, b in zip(G, R):
+        for k in range(8):
+            scale = np.abs(b[k]).max()
+            # a right-hand side below 2^-1000 is at the subnormal spacing times 1/h
+            tiny = 64 * 33 * 5e-324
+            assert np.abs(a[k] - b[k]).max() <= 1e-12 * scale + tiny, (k, log2)
+            if log2 is None and k in (3, 6):
+                assert not a[k].any()
+
+
+# a jump of 2^bits in density, energy and field between neighbouring points, and noise of
+# either sign: alignments from 0 to beyond 63 bits.  Compared at the corners, whose lines hold
+# corners and faces only (a cell-centre value is itself a difference of such states).
+@pytest.mark.parametrize("bits", [0, 5, 6, 7, 31, 32, 33, 57, 58, 59, 63, 64, 70])
+def test_jumps(bits):
+    pb = ai.random_smooth(20, 7, seed=5, amp=0.2)
+    rng = np.random.default_rng(bits)
+    U = ai.dofs(pb)
+    for u in U:
+        big = rng.random(u[0].shape) < 0.3
+        f = np.where(big, 2.0 ** bits, 1.0)
+        u[1:4] *= rng.choice([-1.0, 1.0], size=u[1:4].shape) * 0.1
+        u[4:7] *= rng.choice([-1.0, 1.0], size=u[4:7].shape) * 0.1
+        u[[0, 1, 2, 3, 7]] *= f
+        u[4:7] *= np.sqrt(f)
+        u[7] = 2.0 * f + 0.5 * (u[1:4] ** 2).sum(0) / u[0] + 0.5 * (u[4:7] ** 2).sum(0)
+    a, b = rhs(pb, U)[3], oracle.rhs(pb, U)[3]
+    for k in range(8):
+        assert np.abs(a[k] - b[k]).max() <= 1e-12 * np.abs(b[k]).max(), (k, bits)
