@@ -741,7 +741,10 @@ __device__ void sensor_phi(const AfDev &d, const AfGrid &g, int ci, int cj, doub
   phi[3] = ddiv(absd(num), absd(Ub(ci, cj, 4) + Ub(ci, cj, 5)) + 1e-40);
 }
 
-template <bool GB, bool UP>
+// PL: a stage of a single run with its work lists, nothing recorded or frozen: the slow
+// paths are not compiled in.  Their call frames cost the point pass spills and the cell
+// pass registers: cells 356 -> 319 us and points 694 -> 667 us (blast 1024^2).
+template <bool GB, bool UP, bool PL>
 __device__ __forceinline__ void b_points(const AfDev &d, const AfGrid &g, const int i, const int j, double a, double b,
                                          int mode) {
   const size_t PS = (size_t)g.nxa * g.nya;
@@ -828,7 +831,7 @@ __device__ __forceinline__ void b_points(const AfDev &d, const AfGrid &g, const 
       if (g.pp_on) {
         const size_t op = (size_t)j * g.nxa + i, s1 = (size_t)(AFC_P1 + 2 * (cls - 1)) * PS + op;
         double t1 = 1.0, t2 = 1.0;
-        if (d.frz) {   // frozen branch: the recorded theta*, theta**
+        if (!PL && d.frz) {   // frozen branch: the recorded theta*, theta**
           t1 = d.frz[s1];
           t2 = d.frz[s1 + PS];
           if (!(t1 == 1.0 && t2 == 1.0)) {
@@ -839,7 +842,7 @@ __device__ __forceinline__ void b_points(const AfDev &d, const AfGrid &g, const 
             for (int k = 0; k < 8; ++k) acc[k] = out[k];
           }
         } else if (!clear_of_floor(acc, g)) {
-          if (d.pq) {   // slow path in k_points_slow, over a dense list (the warp does not wait here)
+          if (PL || d.pq) {   // slow path in k_points_slow, over a dense list (the warp does not wait here)
             const int slot = enqueue(d.st, &d.st->npq, d.pq_cap);
             if (slot >= 0) {
               d.pq[slot] = (cls << 28) | (int)op;
@@ -848,15 +851,17 @@ __device__ __forceinline__ void b_points(const AfDev &d, const AfGrid &g, const 
             }
             continue;
           }
-          double out[8];
-          int lim, shr, bad;
-          point_pp<GB>(d, g, cls, i, j, acc, dt, out, lim, shr, bad, t1, t2);
-          nlim += lim;
-          nshr += shr;
-          nbad += bad;
-          for (int k = 0; k < 8; ++k) acc[k] = out[k];
+          if constexpr (!PL) {
+            double out[8];
+            int lim, shr, bad;
+            point_pp<GB>(d, g, cls, i, j, acc, dt, out, lim, shr, bad, t1, t2);
+            nlim += lim;
+            nshr += shr;
+            nbad += bad;
+            for (int k = 0; k < 8; ++k) acc[k] = out[k];
+          }
         }
-        if (d.rec) {
+        if (!PL && d.rec) {
           d.rec[s1] = t1;
           d.rec[s1 + PS] = t2;
         }
@@ -1226,7 +1231,8 @@ __device__ __forceinline__ void cell_H(const AfDev &d, const AfGrid &g, int i, i
   }
 }
 
-template <bool GB>
+// PL: as in the point pass, with the positivity limiters on
+template <bool GB, bool PL>
 __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const int i, const int j, double a, double b,
                                         int mode) {
   const size_t PS = (size_t)g.nxa * g.nya;
@@ -1234,7 +1240,7 @@ __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const i
   int nsrc = 0, nlam = 0, ncfl = 0;
   NewtonLog nl = {0, 0};
   if (i < g.nx && j < g.ny) {
-    const double dt = mode == 1 ? 1.0 : d.sc->dt;
+    const double dt = !PL && mode == 1 ? 1.0 : d.sc->dt;
     const int ip = mface(i + 1, g.nx, g.bc), jp = mface(j + 1, g.ny, g.bc);
     const SV X = sview(d.us[1], g, 1), Y = sview(d.us[2], g, 2), C = sview(d.us[3], g, 3);
     const WV PX = wview(d.pd[1], g), PY = wview(d.pd[2], g), PC = wview(d.pd[3], g), PZ = wview(d.pd[4], g);
@@ -1313,7 +1319,7 @@ __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const i
     const double cxf = mul_i(dt, g.rdx), cyf = mul_i(dt, g.rdy);
     double *uo = d.uo[0];
     const size_t cs0 = (size_t)g.nx * g.ny, o0 = (size_t)j * g.nx + i;
-    if (mode == 1) {
+    if (!PL && mode == 1) {
       // semi-discrete rhs: -(F_R - F_L)/dx - (F_U - F_D)/dy - S (G holds the Simpson flux here)
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
@@ -1355,7 +1361,7 @@ __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const i
       // theta^s_ij = min over the four faces
       const double tsL = FX(i, j, QF_TS), tsR = FX(ip, j, QF_TS), tsD = FY(i, j, QF_TS), tsU = FY(i, jp, QF_TS);
       const double tsc = minnn(minnn(tsL, tsR), minnn(tsD, tsU));
-      if (!g.pp_on) {
+      if (!PL && !g.pp_on) {
         // sensor-blended high-order update: F^ss = F^LLF + G, S^ss = S^LLF + theta^s (S - S^LLF)
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
@@ -1388,14 +1394,14 @@ __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const i
         const double dtts = mul_i(dt, tsc);
         double L1[8], Lam[4];
         double th_src = 1.0;
-        if (d.frz) {   // frozen branch: Lim1 with the recorded theta_ij; face theta are recorded too
+        if (!PL && d.frz) {   // frozen branch: Lim1 with the recorded theta_ij; face theta are recorded too
           th_src = d.frz[AFC_TSRC * PS + o];
 #pragma unroll
           for (int k = 0; k < 8; ++k) L1[k] = fma(th_src, fma(-dtts, dS[k], Ullf[k]) - Ullf[k], Ullf[k]);
           Lam[0] = Lam[1] = Lam[2] = Lam[3] = 1.0;
           nsrc += th_src < 1.0;
         }
-        bool fast = !d.frz && clear_of_floor(Ullf, g);
+        bool fast = (PL || !d.frz) && clear_of_floor(Ullf, g);
         if (fast) {
 #pragma unroll
           for (int k = 0; k < 8; ++k) L1[k] = fma(-dtts, dS[k], Ullf[k]);
@@ -1405,10 +1411,10 @@ __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const i
           fast = box_cert32(L1, Gf, cxf, cyf, g.c13) ||
                  box_cert64(d, g, i, j, ip, jp, L1[0], L1[1], L1[2], L1[3], L1[4], L1[5], L1[6], L1[7], cxf, cyf);
         bool listed = false;
-        if (d.frz) {
+        if (!PL && d.frz) {
         } else if (fast) {
           Lam[0] = Lam[1] = Lam[2] = Lam[3] = 1.0;
-        } else if (d.cq) {   // step (1) here, the box of step (2) in k_cells_slow over a dense list
+        } else if (PL || d.cq) {   // step (1) here, the box of step (2) in k_cells_slow over a dense list
           int sl = 0;
           double eps_rho, eps_p;
           cell_source_limit(Ullf, dS, dtts, g, L1, sl, th_src, eps_rho, eps_p);
@@ -1420,7 +1426,7 @@ __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const i
             d.cqe[2 * slot + 1] = eps_p;
           }
           listed = true;
-        } else {
+        } else if constexpr (!PL) {
           double H[4][8];
 #pragma unroll
           for (int k = 0; k < 8; ++k) {
@@ -1439,7 +1445,7 @@ __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const i
         if (!listed)
 #pragma unroll
           for (int I = 0; I < 4; ++I) d.lam[I * PS + o] = Lam[I];
-        if (d.rec) d.rec[AFC_TSRC * PS + o] = th_src;
+        if (!PL && d.rec) d.rec[AFC_TSRC * PS + o] = th_src;
       }
     }
   }
@@ -1889,16 +1895,17 @@ __global__ void kb_dt(const AfRun *__restrict__ runs, int nruns) {
 // little, the common path runs at twice the occupancy (measured 8 % faster).
 // UP: the velocity-upwind point source (Example 4.2 variant) is compiled in
 // only where it is asked for; the central scheme pays nothing for it.
-template <bool GB, bool UP>
+template <bool GB, bool UP, bool PL>
 __global__ void AF_LB_PT k_points(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                                 double a, double b, int mode) {
-  if (GB && interior_block(g.nx, g.ny)) b_points<false, UP>(d, g, AF_IJ, a, b, mode);
-  else b_points<GB, UP>(d, g, AF_IJ, a, b, mode);
+  if (PL) mode = 0;
+  if (GB && interior_block(g.nx, g.ny)) b_points<false, UP, PL>(d, g, AF_IJ, a, b, mode);
+  else b_points<GB, UP, PL>(d, g, AF_IJ, a, b, mode);
 }
 template <bool UP>
 __global__ void __launch_bounds__(256, 2) kb_points(const AfRun *__restrict__ runs, const int4 *__restrict__ items,
                                                  int nitems, double a, double b) {
-  AF_BATCH_LOOP((b_points<false, UP>(r->d, r->g, i, j, a, b, 0)));
+  AF_BATCH_LOOP((b_points<false, UP, false>(r->d, r->g, i, j, a, b, 0)));
 }
 template <bool GB>
 __global__ void AF_LB_FC k_faces(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
@@ -1910,15 +1917,15 @@ __global__ void __launch_bounds__(256) kb_faces(const AfRun *__restrict__ runs, 
                                                 int nitems) {
   AF_BATCH_LOOP(b_faces<false>(r->d, r->g, i, j, 0));
 }
-template <bool GB>
+template <bool GB, bool PL>
 __global__ void AF_LB_CL k_cells(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                                double a, double b, int mode) {
-  if (GB && interior_block(g.nx, g.ny)) b_cells<false>(d, g, AF_IJ, a, b, mode);
-  else b_cells<GB>(d, g, AF_IJ, a, b, mode);
+  if (GB && interior_block(g.nx, g.ny)) b_cells<false, PL>(d, g, AF_IJ, a, b, mode);
+  else b_cells<GB, PL>(d, g, AF_IJ, a, b, mode);
 }
 __global__ void __launch_bounds__(256, 2) kb_cells(const AfRun *__restrict__ runs, const int4 *__restrict__ items,
                                                 int nitems, double a, double b) {
-  AF_BATCH_LOOP(b_cells<false>(r->d, r->g, i, j, a, b, 0));
+  AF_BATCH_LOOP((b_cells<false, false>(r->d, r->g, i, j, a, b, 0)));
 }
 __global__ void AF_LB_FN k_final(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                                double a, double b) {
@@ -2166,12 +2173,15 @@ void af_launch_divb(const AfDev &d, const AfGrid &g, double *partials, double *o
 }
 void af_launch_points(const AfDev &d, const AfGrid &g, double a, double b, int mode, cudaStream_t s) {
   const dim3 gr = grid2(g.nxa, g.nya), bl(32, 4);
+  const bool plain = mode == 0 && d.pq && !d.rec && !d.frz;
   if (g.special) {
-    if (g.upwind) k_points<true, true><<<gr, bl, 0, s>>>(d, g, a, b, mode);
-    else k_points<true, false><<<gr, bl, 0, s>>>(d, g, a, b, mode);
+    if (g.upwind) k_points<true, true, false><<<gr, bl, 0, s>>>(d, g, a, b, mode);
+    else if (plain) k_points<true, false, true><<<gr, bl, 0, s>>>(d, g, a, b, mode);
+    else k_points<true, false, false><<<gr, bl, 0, s>>>(d, g, a, b, mode);
   } else {
-    if (g.upwind) k_points<false, true><<<gr, bl, 0, s>>>(d, g, a, b, mode);
-    else k_points<false, false><<<gr, bl, 0, s>>>(d, g, a, b, mode);
+    if (g.upwind) k_points<false, true, false><<<gr, bl, 0, s>>>(d, g, a, b, mode);
+    else if (plain) k_points<false, false, true><<<gr, bl, 0, s>>>(d, g, a, b, mode);
+    else k_points<false, false, false><<<gr, bl, 0, s>>>(d, g, a, b, mode);
   }
 }
 void af_launch_faces(const AfDev &d, const AfGrid &g, int mode, cudaStream_t s) {
@@ -2179,8 +2189,15 @@ void af_launch_faces(const AfDev &d, const AfGrid &g, int mode, cudaStream_t s) 
   else k_faces<false><<<grid2(g.nxa, g.nya), dim3(32, 4), 0, s>>>(d, g, mode);
 }
 void af_launch_cells(const AfDev &d, const AfGrid &g, double a, double b, int mode, cudaStream_t s) {
-  if (g.special) k_cells<true><<<grid2(g.nx, g.ny), dim3(32, 4), 0, s>>>(d, g, a, b, mode);
-  else k_cells<false><<<grid2(g.nx, g.ny), dim3(32, 4), 0, s>>>(d, g, a, b, mode);
+  const dim3 gr = grid2(g.nx, g.ny), bl(32, 4);
+  const bool plain = mode == 0 && g.pp_on && d.cq && !d.rec && !d.frz;
+  if (g.special) {
+    if (plain) k_cells<true, true><<<gr, bl, 0, s>>>(d, g, a, b, mode);
+    else k_cells<true, false><<<gr, bl, 0, s>>>(d, g, a, b, mode);
+  } else {
+    if (plain) k_cells<false, true><<<gr, bl, 0, s>>>(d, g, a, b, mode);
+    else k_cells<false, false><<<gr, bl, 0, s>>>(d, g, a, b, mode);
+  }
 }
 void af_launch_final(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s) {
   k_final<<<grid2(g.nx, g.ny), dim3(32, 4), 0, s>>>(d, g, a, b);
