@@ -13,9 +13,12 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libaf.so")
-SOURCES = ["af_kernels.cu", "af_adjoint.cu", "af_api.cu", "af_batch.cu", "af_noalloc.cu", "af_api1d.cu"]
-HEADERS = ["af_internal.h", "af_math.cuh", "af_device.cuh", "af_kernels1d.cuh"]
+SOURCES = ["af_kernels.cu", "af_kernels_lat.cu", "af_adjoint.cu", "af_api.cu", "af_batch.cu", "af_noalloc.cu", "af_api1d.cu"]
+HEADERS = ["af_internal.h", "af_math.cuh", "af_stage.cuh", "af_device.cuh", "af_kernels1d.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
+# The stage kernels are compiled twice (af_kernels.cu, af_kernels_lat.cu) and their results must not
+# depend on which build runs: no contraction of products and sums beyond the fma the source writes.
+SOURCE_FLAGS = {"af_kernels.cu": ["-fmad=false"], "af_kernels_lat.cu": ["-fmad=false"]}
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 
 
@@ -43,7 +46,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         o = os.path.join(BUILD, src.replace(".cu", ".o"))
         objs.append(o)
         if force or _stale(o, [s] + hdrs):
-            cmd = [nvcc(), *ARCH, *FLAGS, "-c", s, "-o", o + ".tmp"]
+            cmd = [nvcc(), *ARCH, *FLAGS, *SOURCE_FLAGS.get(src, []), "-c", s, "-o", o + ".tmp"]
             if verbose:
                 cmd.insert(1, "-Xptxas=-v")
             procs.append((subprocess.Popen(cmd), o))

@@ -163,10 +163,9 @@ void bind_ptrs(af_ctx *c, const double *n, const double *st, double *o) {
 // One stage: P1..P5 on the bound buffers.
 void run_stage(af_ctx *c, double a, double b, int reduce_dt) {
   TIMED(AF_K_POINTDATA, af_launch_pointdata(c->dev, c->g, reduce_dt, c->stream));
-  if (reduce_dt) TIMED(AF_K_DT, af_launch_dt(c->dev, c->g, c->stream));
   TIMED(AF_K_POINTS, af_launch_points(c->dev, c->g, a, b, 0, c->stream));
-  const bool lists = c->g.pp_on && !c->dev.frz;
-  if (lists) {
+  const bool lists = c->g.pp_on && !c->dev.frz, small = af_small_grid(c->g);
+  if (lists && !small) {
     // the point list: only the next stage reads what it writes, so it runs on the
     // second stream beside the face and cell passes and joins at the end of the stage
     // (a short list would otherwise cost the latency of one thread's slow path)
@@ -177,12 +176,10 @@ void run_stage(af_ctx *c, double a, double b, int reduce_dt) {
   }
   TIMED(AF_K_FACES, af_launch_faces(c->dev, c->g, 0, c->stream));
   TIMED(AF_K_CELLS, af_launch_cells(c->dev, c->g, a, b, 0, c->stream));
-  if (lists) TIMED(AF_K_CELLS_SLOW, af_launch_cells_slow(c->dev, c->g, c->stream));
-  if (c->g.pp_on) {
-    TIMED(AF_K_FINAL, af_launch_final(c->dev, c->g, a, b, c->stream));
-    TIMED(AF_K_REPAIR, af_launch_repair(c->dev, c->g, a, b, c->stream));
-  }
-  if (lists) cudaStreamWaitEvent(c->stream, c->ev_join, 0);
+  if (lists && small) TIMED(AF_K_CELLS_SLOW, af_lat_lists(c->dev, c->g, a, b, c->stream));
+  else if (lists) TIMED(AF_K_CELLS_SLOW, af_launch_cells_slow(c->dev, c->g, c->stream));
+  if (c->g.pp_on) TIMED(AF_K_FINAL, af_launch_final(c->dev, c->g, a, b, c->stream));
+  if (lists && !small) cudaStreamWaitEvent(c->stream, c->ev_join, 0);
 }
 
 const double RK_A[3] = {0.0, 3.0 / 4.0, 1.0 / 3.0};
@@ -257,9 +254,7 @@ int af_create(int nx, int ny, double gamma, int bc, af_ctx **out) {
   const size_t PS = (size_t)c->g.nxa * c->g.nya;
   // stage work arrays, then the limiter work lists: points (3 PS entries: an int and 8
   // doubles each), cells (PS entries: an int and 2 doubles each)
-  // and the vertex list (16 PS entries, an unsigned each) with Lambda^rho of the listed cells (4 PS)
-  const size_t nwork = PS * (AF_NQA + 4 * AF_NQP + 8 + 4 + 2 * AF_NQF + 4 + 8 + 2) + PS * (24 + 2) + 2 * PS + 1 +
-                       PS * (8 + 4);
+  const size_t nwork = PS * (AF_NQA + 4 * AF_NQP + 8 + 4 + 2 * AF_NQF + 4 + 8 + 2) + PS * (24 + 2) + 2 * PS + 1;
   int rc = AF_OK;
   for (int b = 0; b < 3; ++b) {
     if (cudaMalloc(&c->state[b], off * sizeof(double)) != cudaSuccess) rc = AF_ENOMEM;
@@ -297,9 +292,6 @@ int af_create(int nx, int ny, double gamma, int bc, af_ctx **out) {
   c->dev.cqe = w; w += 2 * PS;
   c->dev.pq = reinterpret_cast<int *>(w); w += (3 * PS + 1) / 2;
   c->dev.cq = reinterpret_cast<int *>(w); w += (PS + 1) / 2;
-  c->dev.cql = w; w += 4 * PS;
-  c->dev.vq_cap = (int)(16 * PS);
-  c->dev.vq = reinterpret_cast<unsigned *>(w); w += 8 * PS;
   c->dev.sc = c->sc;
   c->dev.st = c->st;
   c->cur = 0;
@@ -428,7 +420,6 @@ int af_dt(af_ctx *c, double *dt_out, int on_device) {
   CK(cudaSetDevice(c->device), "set device");
   bind_states(c, c->cur, c->cur, (c->cur + 1) % 3);
   af_launch_pointdata(c->dev, c->g, 1, c->stream);
-  af_launch_dt(c->dev, c->g, c->stream);
   CK(cudaGetLastError(), "dt launch");
   if (dt_out) {
     CK(cudaMemcpyAsync(dt_out, &c->sc->dt, sizeof(double), on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,

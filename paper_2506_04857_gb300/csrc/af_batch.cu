@@ -179,7 +179,8 @@ void launch_pass(af_batch *b, int pass, const AfRun *tab, double a, double bb, i
   int bps = b->blocks_per_sm[pass];
   if (bps_cap > 0 && bps > bps_cap) bps = bps_cap;
   int nblocks = b->sms * bps;
-  if (nblocks > b->nitems) nblocks = b->nitems;
+  const int n = b->nitems * af_batch_parts(pass);
+  if (nblocks > n) nblocks = n;
   af_launch_batch(pass, tab, b->nruns, b->items, b->nitems, b->block, nblocks, a, bb, reduce_dt, b->stream);
 }
 

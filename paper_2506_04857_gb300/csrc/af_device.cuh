@@ -5,6 +5,14 @@
 
 #include "af_internal.h"
 
+// Loads of the stage's arrays.  The small-grid build runs several passes in one kernel
+// (k1_step), where the read-only path must not be used for what the kernel itself wrote.
+#ifdef AF_LAT
+#define AF_LD(p) (*(p))
+#else
+#define AF_LD(p) __ldg(p)
+#endif
+
 namespace {
 
 __device__ __forceinline__ int wrapi(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
@@ -24,7 +32,7 @@ struct SV {   // one DoF class of a state: component k at (i,j) is p[k*cs + j*ex
   size_t cs;
   int ex;
   __device__ __forceinline__ double operator()(int i, int j, int k) const {
-    return __ldg(p + (size_t)k * cs + (size_t)j * ex + i);
+    return AF_LD(p + (size_t)k * cs + (size_t)j * ex + i);
   }
 };
 __device__ __forceinline__ SV sview(const double *p, const AfGrid &g, int c) {
@@ -39,7 +47,7 @@ struct WV {   // a work array [q][nya][nxa]
   size_t PS;
   int nxa;
   __device__ __forceinline__ double operator()(int i, int j, int q) const {
-    return __ldg(p + (size_t)q * PS + (size_t)j * nxa + i);
+    return AF_LD(p + (size_t)q * PS + (size_t)j * nxa + i);
   }
 };
 __device__ __forceinline__ WV wview(const double *p, const AfGrid &g) {

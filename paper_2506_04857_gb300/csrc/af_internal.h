@@ -66,7 +66,8 @@ struct AfGrid {
 struct AfScalars {
   double dt;
   unsigned long long smax[2];   // running max of varrho_1, varrho_2 (bit patterns of non-negative doubles)
-  int pad[4];
+  int ticket[2];   // blocks of the point-data and final passes that have finished
+  int pad[2];
 };
 
 struct AfStatus {
@@ -75,7 +76,6 @@ struct AfStatus {
   int nrepair;
   int repair[AF_MAX_REPAIR];
   int npq, ncq;   // entries of the point and cell work lists of the current stage
-  int nvq;        // entries of the vertex list (vertices of listed cells that need the Newton solve)
 };
 
 struct AfDev {
@@ -100,11 +100,6 @@ struct AfDev {
   int *pq, *cq;
   double *pqu, *cqe;
   int pq_cap, cq_cap;
-  // vertices of R_rho (listed cell << 4 | vertex) whose pressure falls below eps_p, and
-  // Lambda^rho of each listed cell
-  unsigned *vq;
-  double *cql;
-  int vq_cap;
 };
 
 // one member of a batch (af_batch.cu): its work pointers and grid
@@ -113,17 +108,24 @@ struct AfRun {
   AfGrid g;
 };
 
-// kernel launchers (af_kernels.cu)
+// kernel launchers (af_kernels.cu).  The point-data pass forms dt too when reduce_dt is set;
+// the final pass also runs the repair list.
 void af_launch_pointdata(const AfDev &d, const AfGrid &g, int reduce_dt, cudaStream_t s);
-void af_launch_dt(const AfDev &d, const AfGrid &g, cudaStream_t s);
 void af_launch_points(const AfDev &d, const AfGrid &g, double a, double b, int mode, cudaStream_t s);
 void af_launch_faces(const AfDev &d, const AfGrid &g, int mode, cudaStream_t s);
 void af_launch_cells(const AfDev &d, const AfGrid &g, double a, double b, int mode, cudaStream_t s);
 void af_launch_final(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s);
+// the same passes compiled for small grids (af_kernels_lat.cu)
+void af_lat_pointdata(const AfDev &d, const AfGrid &g, int reduce_dt, cudaStream_t s);
+void af_lat_points(const AfDev &d, const AfGrid &g, double a, double b, int mode, cudaStream_t s);
+void af_lat_faces(const AfDev &d, const AfGrid &g, int mode, cudaStream_t s);
+void af_lat_cells(const AfDev &d, const AfGrid &g, double a, double b, int mode, cudaStream_t s);
+void af_lat_final(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s);
+void af_lat_lists(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s);   // both work lists
+bool af_small_grid(const AfGrid &g);   // which build the launchers below take
 // the limiter slow paths over the work lists the point and cell passes filled
 void af_launch_points_slow(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s);
 void af_launch_cells_slow(const AfDev &d, const AfGrid &g, cudaStream_t s);
-void af_launch_repair(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s);
 float af_run_fp64_probe(cudaStream_t s, double *flops);
 // point data of the inflow state U (device, 8 doubles) into out (8 + AF_NQP + AF_NQA doubles)
 void af_launch_inflow_pd(const AfGrid &g, const double *U, double *out, cudaStream_t s);
@@ -229,6 +231,7 @@ void af_launch_divb(const AfDev &d, const AfGrid &g, double *partials, double *o
 // point source" for the point pass
 void af_launch_batch(int pass, const AfRun *runs, int nruns, const int4 *items, int nitems, dim3 block, int nblocks,
                      double a, double b, int flag, cudaStream_t s);
+int af_batch_parts(int pass);                   // items of the pass per tile
 int af_batch_occupancy(int pass, dim3 block);   // resident blocks per SM
 // adjoint (af_adjoint.cu).  With T = (dL/dU)^T v at the state bound in d (after
 // the point-data pass on it), the last kernel writes

@@ -39,7 +39,7 @@ __device__ __forceinline__ void b1_pointdata(const AfDev &d, const AfGrid &g, in
     const SV P = sview(d.us[1], g, 1);
     const int ip = mface(i + 1, g.nx, g.bc);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) uc[k] = (6.0 * A[k] - P(i, 0, k) - P(ip, 0, k)) * 0.25;
+    for (int k = 0; k < 8; ++k) uc[k] = (fma(6.0, A[k], -P(i, 0, k)) - P(ip, 0, k)) * 0.25;
     if (!clear_of_floor(uc, g)) {   // Remark 3.2
       double out[8], t1, t2;
       scaling_limiter(uc, A, g.gm1, out, t1, t2);
@@ -80,7 +80,7 @@ __device__ __noinline__ void point_pp1(const AfDev &d, const AfGrid &g, int f, c
   llf_flux_full(0, me, nb, Fr);
   const double cxf = dt * g.rdx;
   double UL[8];
-  for (int k = 0; k < 8; ++k) UL[k] = me.U[k] - cxf * (Fr[k] - Fl[k]);
+  for (int k = 0; k < 8; ++k) UL[k] = fma(-cxf, Fr[k] - Fl[k], me.U[k]);
   double t1, t2;
   scaling_limiter(UH, UL, g.gm1, out, t1, t2);
   limited = (t1 < 1.0 || t2 < 1.0);
@@ -116,7 +116,7 @@ __device__ __forceinline__ void b1_points(const AfDev &d, const AfGrid &g, int f
 #pragma unroll
     for (int k = 0; k < 8; ++k) acc[k] = pu(me, k);
     const PP L[5] = {pref(d, g, 1, fm, 0), pref(d, g, 4, c0, 0), me, pref(d, g, 4, c1, 0), pref(d, g, 1, fp, 0)};
-    fvs_line<0>(L, PS, g.nxa, 0.5 * dt * g.rdx, acc, dB, 0);
+    fvs_line<0, false>(L, PS, g.nxa, 0.5 * dt * g.rdx, acc, dB, 0);
     if (g.pp_on && !clear_of_floor(acc, g)) {
       double out[8];
       int lim, shr, bad;
@@ -132,7 +132,7 @@ __device__ __forceinline__ void b1_points(const AfDev &d, const AfGrid &g, int f
       for (int k = 0; k < 8; ++k) d.uo[1][k * cs + f] = acc[k];
     } else {
 #pragma unroll
-      for (int k = 0; k < 8; ++k) d.uo[1][k * cs + f] = fma(a, __ldg(d.un[1] + k * cs + f), b * acc[k]);
+      for (int k = 0; k < 8; ++k) d.uo[1][k * cs + f] = fma(a, AF_LD(d.un[1] + k * cs + f), b * acc[k]);
     }
   }
   if (f < g.nx && g.kappa != 0.0) {
@@ -229,7 +229,7 @@ __device__ __forceinline__ void b1_cells(const AfDev &d, const AfGrid &g, int i,
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         const double fe = Ullf[k] + H[0][k] + H[1][k];
-        d.uo[0][k * cs0 + i] = a == 0.0 ? fe : fma(a, __ldg(d.un[0] + k * cs0 + i), b * fe);
+        d.uo[0][k * cs0 + i] = a == 0.0 ? fe : fma(a, AF_LD(d.un[0] + k * cs0 + i), b * fe);
       }
     } else {
       if (dt * ((FX(i, 0, QF_AL) + FX(ip, 0, QF_AL)) * g.rdx) > 1.0 + 1e-12) ncfl = 1;   // Lemma 3.1 (count only)
@@ -309,7 +309,7 @@ __device__ __forceinline__ void b1_final(const AfDev &d, const AfGrid &g, int i,
     }
     const size_t cs0 = (size_t)g.nx;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) d.uo[0][k * cs0 + i] = a == 0.0 ? fe[k] : fma(a, __ldg(d.un[0] + k * cs0 + i), b * fe[k]);
+    for (int k = 0; k < 8; ++k) d.uo[0][k * cs0 + i] = a == 0.0 ? fe[k] : fma(a, AF_LD(d.un[0] + k * cs0 + i), b * fe[k]);
   }
   if (nface) atomicAdd(&d.st->cnt[ST_FACE_THETA_LT1], (unsigned long long)nface);
 }

@@ -161,8 +161,15 @@ __device__ __forceinline__ double rcp44(float xh, float xl) {
 
 __device__ __forceinline__ double mul_i(double a, double b);
 
+// AF_LAT (the small-grid build): see the end of this file
+#ifdef AF_LAT
+#define AF_ONCE static __device__ __noinline__
+#else
+#define AF_ONCE __device__ __forceinline__
+#endif
+
 // 1/x: the 44-bit reciprocal and one FP64 Newton step
-__device__ __forceinline__ double rcp(double x) {
+AF_ONCE double rcp(double x) {
   float xh, xl;
   if (!split_f32(x, xh, xl)) return rcp_nr2(x);
   const double y = rcp44(xh, xl);
@@ -172,7 +179,7 @@ __device__ __forceinline__ double rcp(double x) {
 
 // a/b: q = a y with the 44-bit reciprocal y of b (product on the integer pipes),
 // then one residual correction
-__device__ __forceinline__ double ddiv(double a, double b) {
+AF_ONCE double ddiv(double a, double b) {
   float bh, bl;
   if (!split_f32(b, bh, bl)) return ddiv_nr(a, b);
   const double y = rcp44(bh, bl);
@@ -184,7 +191,7 @@ __device__ __forceinline__ double ddiv(double a, double b) {
 // sqrt(x), x > 0 in range: s0 = xh / sqrt(xh) from the rsqrt seed, one Heron step
 // s0 + (x - s0^2) / (2 s0) in FP32 on the split, one FP64 Heron step (1/(2 s) from
 // the seed)
-__device__ __forceinline__ double dsqrt(double x) {
+AF_ONCE double dsqrt(double x) {
   float xh, xl;
   if ((long long)bits(x) <= 0 || !split_f32(x, xh, xl)) return dsqrt_nr2(x);
   const float r0 = rsqrt_approx_f32(xh);
@@ -235,6 +242,9 @@ static __device__ __noinline__ double add_hw(double a, double b) { return __dadd
 
 // a * b.  Fast path: both finite with normal exponent fields and a product
 // exponent field in [1, 2045], or a zero factor times a finite one (+-0).
+#ifdef AF_LAT
+__device__ __forceinline__ double mul_i(double a, double b) { return __dmul_rn(a, b); }
+#else
 __device__ __forceinline__ double mul_i(double a, double b) {
   const unsigned long long ia = bits(a), ib = bits(b);
   const unsigned s = (unsigned)((ia ^ ib) >> 32) & 0x80000000u;
@@ -276,6 +286,7 @@ __device__ __forceinline__ double mul_i(double a, double b) {
   const unsigned long long r = (za || zb) ? ((unsigned long long)s << 32) : (((unsigned long long)hi << 32) | lo);
   return from_bits(r);
 }
+#endif
 
 // IEEE compares on the integer pipe (the same result as the FP64 compare for every
 // input, NaN and +-0 included).
@@ -314,17 +325,24 @@ __device__ __forceinline__ double neg_i(double x) { return from_bits(bits(x) ^ 0
 template <int K>
 __device__ __forceinline__ double ldexp_i(double x) {
   static_assert(K >= -8 && K <= 8, "small scalings only");
+#ifdef AF_LAT
+  return __dmul_rn(x, K >= 0 ? (double)(1 << (K >= 0 ? K : 0)) : 1.0 / (double)(1 << (K < 0 ? -K : 0)));
+#else
   const unsigned long long ix = bits(x);
   const unsigned e = (unsigned)(ix >> 52) & 0x7ffu;
   if ((ix << 1) == 0) return x;
   const bool ok = K >= 0 ? (e - 1u < (unsigned)(2046 - K)) : (e - (unsigned)(1 - K) < (unsigned)(2046 + K));
   if (!ok) return mul_hw(x, K >= 0 ? (double)(1 << (K >= 0 ? K : 0)) : 1.0 / (double)(1 << (K < 0 ? -K : 0)));
   return from_bits(ix + ((unsigned long long)(long long)K << 52));
+#endif
 }
 
 // a + b.  Fast path: the operand of larger magnitude finite and normal with an
 // exponent field <= 2045, the other zero or with an exponent field >= 54 (no
 // result is then subnormal), or both zero.
+#ifdef AF_LAT
+__device__ __forceinline__ double add_i(double a, double b) { return __dadd_rn(a, b); }
+#else
 __device__ __forceinline__ double add_i(double a, double b) {
   const unsigned long long SGN = 0x8000000000000000ULL;
   const unsigned long long ia = bits(a), ib = bits(b);
@@ -355,6 +373,7 @@ __device__ __forceinline__ double add_i(double a, double b) {
   r = (X == 0) ? (ia & ib) : r;           // +-0 + +-0: -0 only for -0 + -0
   return from_bits(r);
 }
+#endif
 
 // a - b on the integer pipes
 __device__ __forceinline__ double sub_i(double a, double b) { return add_i(a, neg_i(b)); }
@@ -370,9 +389,10 @@ __device__ __forceinline__ double sub_i(double a, double b) { return add_i(a, ne
 // equal terms whose coefficients cancel give exactly 0.  An alignment costs about 12
 // integer instructions and the normalisation 18: the 5-point sum keeps the integer ALUs
 // (16 lanes per scheduler) busy for about 180 cycles where its four FP64 instructions
-// kept the FP64 pipe busy for 300, and both run at once.  Zero lines return at once;
-// terms below 2^-823, infinite, NaN or close to overflow take the FP64 sums, in a
-// function that is not inlined.
+// kept the FP64 pipe busy for 300, and both run at once.  The sum is that of magnitudes
+// truncated to the guard bits, so it changes sign exactly with its terms (mirrored data
+// give mirrored results).  Zero lines return at once; terms below 2^-823, infinite, NaN or
+// close to overflow take the FP64 sums, in a function that is not inlined.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ unsigned fx_exp(double x) { return hi32(x) & 0x7ff00000u; }
 __device__ __forceinline__ bool fx_ok(unsigned emax) { return emax - (200u << 20) <= (1800u << 20); }
@@ -381,24 +401,29 @@ __device__ __forceinline__ unsigned long long fx_shr(unsigned long long m, unsig
   asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"(s));
   return r;
 }
-// the signed significand of x, aligned to the exponent field emax (in place in the high word)
+// the significand of x with its sign, aligned to the exponent field emax (in place in the high
+// word), in ones' complement: the value minus one for a negative x.  neg: -1 for a negative x
+// (the caller adds the ones of its sum at once)
 template <int G>
-__device__ __forceinline__ long long fx_term(double x, unsigned emax) {
+__device__ __forceinline__ long long fx_term(double x, unsigned emax, int &neg) {
   const unsigned long long b = bits(x);
   const unsigned hi = (unsigned)(b >> 32);
   const unsigned s = (emax - (hi & 0x7ff00000u)) >> 20;
   const unsigned long long m = (((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | (unsigned)b) << G;
-  return (long long)fx_shr(m, s) ^ (long long)((int)hi >> 31);
+  neg = (int)hi >> 31;
+  return (long long)fx_shr(m, s) ^ (long long)neg;
 }
 // the double nearest to acc 2^(e - G), in units of the last place, e the exponent of the field emax
 template <int G>
 __device__ __forceinline__ double fx_round(long long acc, unsigned emax) {
   const long long sg = acc >> 63;
-  unsigned long long a = (unsigned long long)(acc ^ sg);
+  unsigned long long a = (unsigned long long)((acc ^ sg) - sg);
   const int lz = __clzll((long long)a);
   a <<= (lz & 63);
   const unsigned e = (emax >> 20) + (unsigned)(10 - G) - (unsigned)lz;   // exponent field minus one
-  const unsigned long long q = (a >> 11) + ((a >> 10) & 1ULL);
+  // to nearest, ties to even: one less than half a unit, or half a unit above an odd place, carries
+  // into the kept bits exactly when the sum is rounded up
+  const unsigned long long q = (a >> 11) + (((a & 0x7ffULL) + 0x3ffULL + ((a >> 11) & 1ULL)) >> 11);
   const unsigned long long r = ((unsigned long long)((e << 20) | ((unsigned)(sg >> 32) & 0x80000000u)) << 32) + q;
   return from_bits(a == 0 ? 0ULL : r);
 }
@@ -406,16 +431,18 @@ static __device__ __noinline__ double up5_hw(double u0, double u1, double u2, do
   return fma(6.0, u2, fma(-4.0, u1 + u3, u0 + u4));
 }
 // (u0 + u4) - 4 (u1 + u3) + 6 u2
-__device__ __forceinline__ double up5(double u0, double u1, double u2, double u3, double u4) {
+AF_ONCE double up5(double u0, double u1, double u2, double u3, double u4) {
   const unsigned em = max(max(max(fx_exp(u0), fx_exp(u1)), fx_exp(u2)), max(fx_exp(u3), fx_exp(u4)));
   if (!fx_ok(em)) {
     if (((bits(u0) | bits(u1) | bits(u2) | bits(u3) | bits(u4)) << 1) == 0) return 0.0;
     return up5_hw(u0, u1, u2, u3, u4);
   }
-  const long long v2 = fx_term<6>(u2, em), t13 = fx_term<6>(u1, em) + fx_term<6>(u3, em);
-  const long long t04 = fx_term<6>(u0, em) + fx_term<6>(u4, em);
+  int n0, n1, n2, n3, n4;
+  const long long v2 = fx_term<6>(u2, em, n2), t13 = fx_term<6>(u1, em, n1) + fx_term<6>(u3, em, n3);
+  const long long t04 = fx_term<6>(u0, em, n0) + fx_term<6>(u4, em, n4);
   const long long w = v2 + ((v2 - t13) << 1);   // 3 u2 - 2 (u1 + u3)
-  return fx_round<6>(t04 + (w << 1), em);
+  const int ones = (n0 + n4) - 4 * (n1 + n3) + 6 * n2;
+  return fx_round<6>(t04 + (w << 1) - ones, em);
 }
 
 }  // namespace afm
