@@ -24,6 +24,7 @@ struct af1d_ctx {
   AfScalars *sc;
   AfStatus *st;
   AfDev dev;
+  int cluster;        // CTAs of the one-launch step of a short grid (0: one launch per pass)
   AfEventTimer tm;    // per-kernel event timing (af1d_timing)
   char msg[512];
 };
@@ -114,11 +115,36 @@ int set_dt1(af1d_ctx *c, const double *dt, int on_device) {
 const double RK1_A[3] = {0.0, 3.0 / 4.0, 1.0 / 3.0};
 const double RK1_B[3] = {1.0, 1.0 / 4.0, 2.0 / 3.0};
 
-int stage1(af1d_ctx *c, int s, int reduce_dt) {
+void bind_stage1(af1d_ctx *c, int s) {
   const int n = c->cur, b1 = (c->cur + 1) % 3, b2 = (c->cur + 2) % 3;
   if (s == 0) bind1(c, n, n, b1);
   else if (s == 1) bind1(c, n, b1, b2);
   else bind1(c, n, b2, b1);
+}
+
+// Stages s0..s1 in one launch (short grids)
+#ifndef AF_STEP1D_MAX
+#define AF_STEP1D_MAX 4096
+#endif
+int stages1(af1d_ctx *c, int s0, int s1, int reduce_dt) {
+  AfDev d[3];
+  for (int s = 0; s < 3; ++s) {
+    bind_stage1(c, s);
+    d[s] = c->dev;
+  }
+  af_lat_step1d(d, c->g, s0, s1, reduce_dt, c->cluster, c->stream);
+  CK1(cudaGetLastError(), "step launch");
+  const int b1 = (c->cur + 1) % 3, b2 = (c->cur + 2) % 3;
+  c->last_out = s1 == 1 ? b2 : b1;
+  if (s1 == 2) c->cur = b1;
+  c->next_stage = (s1 + 1) % 3;
+  return AF_OK;
+}
+
+int stage1(af1d_ctx *c, int s, int reduce_dt) {
+  if (c->cluster && !c->tm.on) return stages1(c, s, s, reduce_dt);
+  const int b1 = (c->cur + 1) % 3, b2 = (c->cur + 2) % 3;
+  bind_stage1(c, s);
   af_launch_stage1d(c->dev, c->g, RK1_A[s], RK1_B[s], reduce_dt, c->stream, &c->tm);
   CK1(cudaGetLastError(), "stage launch");
   c->last_out = s == 1 ? b2 : b1;
@@ -188,6 +214,7 @@ int af1d_create(int n, double gamma, int bc, af1d_ctx **out) {
   c->dev.thx = w; w += PS;
   c->dev.sc = c->sc;
   c->dev.st = c->st;
+  c->cluster = c->nf <= AF_STEP1D_MAX ? af_lat_step1d_cluster(c->nf) : 0;
   c->cur = 0;
   c->next_stage = 0;
   *out = c;
@@ -271,9 +298,14 @@ int af1d_step(af1d_ctx *c, double *dt_used, int on_device) {
   if (!c) return AF_EINVAL;
   if (c->next_stage != 0) return fail1(c, AF_EINVAL, "af1d_step called in the middle of a step");
   CK1(cudaSetDevice(c->device), "set device");
-  int rc = stage1(c, 0, 1);
-  if (!rc) rc = stage1(c, 1, 0);
-  if (!rc) rc = stage1(c, 2, 0);
+  int rc;
+  if (c->cluster && !c->tm.on) {
+    rc = stages1(c, 0, 2, 1);
+  } else {
+    rc = stage1(c, 0, 1);
+    if (!rc) rc = stage1(c, 1, 0);
+    if (!rc) rc = stage1(c, 2, 0);
+  }
   if (rc) return rc;
   if (dt_used) {
     CK1(cudaMemcpyAsync(dt_used, &c->sc->dt, sizeof(double), on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,

@@ -217,6 +217,9 @@ struct AfEventTimer {
 // One 1D stage; t (may be NULL) times each launch.
 void af_launch_stage1d(const AfDev &d, const AfGrid &g, double a, double b, int reduce_dt, cudaStream_t s,
                        AfEventTimer *t);
+// Stages s0..s1 of a step of a short 1D grid in one cluster launch (d: the three stages' bindings)
+int af_lat_step1d_cluster(int n);
+void af_lat_step1d(const AfDev *d, const AfGrid &g, int s0, int s1, int reduce_dt, int cluster, cudaStream_t s);
 void af_launch_dt1d(const AfDev &d, const AfGrid &g, cudaStream_t s);
 // divergence measures of Example 4.4 of the state bound in d.us into out[2]
 // (device); partials: 2 * af_divb_nblocks(g) doubles

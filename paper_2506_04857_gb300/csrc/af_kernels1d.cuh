@@ -21,21 +21,26 @@
 namespace {
 
 // P1 (1D): point data of the points, the averages and the centre values; dt maximum
-__device__ __forceinline__ void b1_pointdata(const AfDev &d, const AfGrid &g, int i, int reduce_dt) {
+// parts: 1 the point, 2 the average, 4 the centre of index i
+__device__ __forceinline__ void b1_pointdata(const AfDev &d, const AfGrid &g, int i, int reduce_dt, int parts = 7) {
   const size_t PS = (size_t)g.nxa;
   double m1 = 0.0, s1, s2;
   bool clim = false;
-  if (i < g.ex[1]) {
+  if ((parts & 1) && i < g.ex[1]) {
     double U[8];
     load8(sview(d.us[1], g, 1), i, 0, U);
     point_data(U, g, d.pd[1] + i, PS, false, s1, s2);
     m1 = maxnn(m1, s1);
   }
-  if (i < g.nx) {
-    double A[8], uc[8];
+  if ((parts & 2) && i < g.nx) {
+    double A[8];
     load8(sview(d.us[0], g, 0), i, 0, A);
     point_data(A, g, d.pd[0] + i, PS, true, s1, s2);
     m1 = maxnn(m1, s1);
+  }
+  if ((parts & 4) && i < g.nx) {
+    double A[8], uc[8];
+    load8(sview(d.us[0], g, 0), i, 0, A);
     const SV P = sview(d.us[1], g, 1);
     const int ip = mface(i + 1, g.nx, g.bc);
 #pragma unroll
@@ -104,11 +109,12 @@ __device__ __noinline__ void point_pp1(const AfDev &d, const AfGrid &g, int f, c
 }
 
 // P2 (1D): point update, its limiter and the RK combination; the sensor phi
-__device__ __forceinline__ void b1_points(const AfDev &d, const AfGrid &g, int f, double a, double b) {
+// parts: 1 the point, 2 the sensor values of cell f
+__device__ __forceinline__ void b1_points(const AfDev &d, const AfGrid &g, int f, double a, double b, int parts = 3) {
   const size_t PS = (size_t)g.nxa;
   const double dt = d.sc->dt;
   int nlim = 0, nshr = 0, nbad = 0;
-  if (f < g.ex[1]) {
+  if ((parts & 1) && f < g.ex[1]) {
     const int fm = mface(f - 1, g.nx, g.bc), fp = mface(f + 1, g.nx, g.bc);
     const int c0 = mcell(f - 1, g.nx, g.bc), c1 = mcell(f, g.nx, g.bc);
     const PP me = pref(d, g, 1, f, 0);
@@ -135,7 +141,7 @@ __device__ __forceinline__ void b1_points(const AfDev &d, const AfGrid &g, int f
       for (int k = 0; k < 8; ++k) d.uo[1][k * cs + f] = fma(a, AF_LD(d.un[1] + k * cs + f), b * acc[k]);
     }
   }
-  if (f < g.nx && g.kappa != 0.0) {
+  if ((parts & 2) && f < g.nx && g.kappa != 0.0) {
     double phi[4];
     sensor_phi<false>(d, g, f, 0, phi);
 #pragma unroll
@@ -371,6 +377,60 @@ __device__ void b1_repair(const AfDev &d, const AfGrid &g, double a, double b) {
   }
 }
 
+#ifdef AF_LAT
+// A whole step (or the stages s0..s1 of one) of a short grid in one launch of one thread-block
+// cluster: the passes follow one another across a cluster barrier.  Arrays stay in global
+// memory (L2), written by one CTA of the cluster and read by its neighbours after the barrier,
+// whose arrive releases and whose wait acquires at cluster scope.
+// What bounds it: latency.  At 800 cells a pass is about 50 threads per SM with 40 to 130
+// dependent FP64 instructions of 64 cycles each, and a launch of its own costs more than that.
+// threadIdx.y is a role: the point, the average and the centre of a cell side by side in the
+// point-data pass, the point and the sensor in the point pass; the other passes deal the
+// indices to all threads.
+struct AfStages1d {
+  AfDev d[3];
+};
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+constexpr int kStepThreads = 128;   // of each role, at most
+__global__ void __launch_bounds__(3 * kStepThreads) k1_step(const __grid_constant__ AfStages1d S,
+                                                            const __grid_constant__ AfGrid g, int s0, int s1,
+                                                            int reduce_dt) {
+  const int bx = (int)blockDim.x, cs = (int)gridDim.x, rank = (int)blockIdx.x, role = (int)threadIdx.y;
+  const int n = g.nxa;
+  const bool first = rank == 0 && threadIdx.x == 0 && threadIdx.y == 0;
+  // one index per thread of a role, and one per thread of the cluster; the trip counts are uniform in a block
+  const int base1 = rank * bx, step1 = cs * bx, base3 = (role * cs + rank) * bx, step3 = 3 * cs * bx;
+  for (int s = s0; s <= s1; ++s) {
+    const AfDev &d = S.d[s];
+    const double a = s == 0 ? 0.0 : (s == 1 ? 3.0 / 4.0 : 1.0 / 3.0), b = s == 0 ? 1.0 : (s == 1 ? 1.0 / 4.0 : 2.0 / 3.0);
+    for (int q = base1; q < n; q += step1) b1_pointdata(d, g, q + (int)threadIdx.x, reduce_dt && s == 0, 1 << role);
+    cluster_sync();
+    if (reduce_dt && s == 0) {
+      if (first) b_dt(d, g);
+      cluster_sync();
+    }
+    if (role < 2)
+      for (int q = base1; q < n; q += step1) b1_points(d, g, q + (int)threadIdx.x, a, b, 1 << role);
+    cluster_sync();
+    for (int q = base3; q < n; q += step3) b1_faces(d, g, q + (int)threadIdx.x);
+    cluster_sync();
+    for (int q = base3; q < n; q += step3) b1_cells(d, g, q + (int)threadIdx.x, a, b);
+    cluster_sync();
+    if (g.pp_on) {
+      for (int q = base3; q < n; q += step3) b1_final(d, g, q + (int)threadIdx.x, a, b);
+      cluster_sync();
+      // every thread reads the same count: nothing changes it before the next barrier
+      if (*(volatile int *)&d.st->nrepair > 0) {
+        cluster_sync();
+        if (first) b1_repair(d, g, a, b);
+        cluster_sync();
+      }
+    }
+  }
+}
+#else
 __global__ void __launch_bounds__(128) k1_pointdata(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                                     int reduce_dt) {
   b1_pointdata(d, g, blockIdx.x * blockDim.x + threadIdx.x, reduce_dt);
@@ -390,11 +450,56 @@ __global__ void __launch_bounds__(128) k1_final(const __grid_constant__ AfDev d,
                                                 double a, double b) {
   b1_final(d, g, blockIdx.x * blockDim.x + threadIdx.x, a, b);
 }
+__global__ void k1_dt(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g) {
+  if (threadIdx.x == 0 && blockIdx.x == 0) b_dt(d, g);
+}
 __global__ void k1_repair(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g, double a, double b) {
   if (blockIdx.x == 0 && threadIdx.x == 0) b1_repair(d, g, a, b);
 }
+#endif
 
 }  // namespace
+
+#ifdef AF_LAT
+namespace {
+int step_threads(int n, int cs) {
+  const int t = ((n + cs - 1) / cs + 31) / 32 * 32;
+  return t < kStepThreads ? t : kStepThreads;
+}
+cudaLaunchConfig_t step_config(int n, int cs, cudaLaunchAttribute *at, cudaStream_t s) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(cs);
+  c.blockDim = dim3(step_threads(n, cs), 3);
+  c.stream = s;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = cs;
+  at->val.clusterDim.y = at->val.clusterDim.z = 1;
+  c.attrs = at;
+  c.numAttrs = 1;
+  return c;
+}
+}  // namespace
+
+// The cluster size of k1_step on the current device for n indices: 16, else 8, else 0 (no cluster fits)
+int af_lat_step1d_cluster(int n) {
+  cudaFuncSetAttribute(k1_step, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  for (int cs = 16; cs >= 8; cs /= 2) {
+    cudaLaunchAttribute at;
+    cudaLaunchConfig_t c = step_config(n, cs, &at, nullptr);
+    int k = 0;
+    if (cudaOccupancyMaxActiveClusters(&k, k1_step, &c) == cudaSuccess && k > 0) return cs;
+    cudaGetLastError();
+  }
+  return 0;
+}
+void af_lat_step1d(const AfDev *d, const AfGrid &g, int s0, int s1, int reduce_dt, int cluster, cudaStream_t s) {
+  AfStages1d S;
+  for (int k = 0; k < 3; ++k) S.d[k] = d[k];
+  cudaLaunchAttribute at;
+  cudaLaunchConfig_t c = step_config(g.nxa, cluster, &at, s);
+  cudaLaunchKernelEx(&c, k1_step, S, g, s0, s1, reduce_dt);
+}
+#else
 
 // One 1D stage: P1 (with the dt pass when reduce_dt), P2..P5 and the repair
 // pass; t (may be NULL) brackets each launch with an event pair.
@@ -407,7 +512,7 @@ void af_launch_stage1d(const AfDev &d, const AfGrid &g, double a, double b, int 
     if (t) t->end(on, s);
   };
   timed(AF_K_POINTDATA, [&] { k1_pointdata<<<nb, 128, 0, s>>>(d, g, reduce_dt); });
-  if (reduce_dt) timed(AF_K_DT, [&] { k_dt<<<1, 32, 0, s>>>(d, g); });
+  if (reduce_dt) timed(AF_K_DT, [&] { k1_dt<<<1, 32, 0, s>>>(d, g); });
   timed(AF_K_POINTS, [&] { k1_points<<<nb, 128, 0, s>>>(d, g, a, b); });
   timed(AF_K_FACES, [&] { k1_faces<<<nb, 128, 0, s>>>(d, g); });
   timed(AF_K_CELLS, [&] { k1_cells<<<nb, 128, 0, s>>>(d, g, a, b); });
@@ -419,5 +524,6 @@ void af_launch_stage1d(const AfDev &d, const AfGrid &g, double a, double b, int 
 void af_launch_dt1d(const AfDev &d, const AfGrid &g, cudaStream_t s) {
   const unsigned nb = (unsigned)((g.nxa + 127) / 128);
   k1_pointdata<<<nb, 128, 0, s>>>(d, g, 1);
-  k_dt<<<1, 32, 0, s>>>(d, g);
+  k1_dt<<<1, 32, 0, s>>>(d, g);
 }
+#endif

@@ -12,3 +12,5 @@ void af_lat_cells(const AfDev &d, const AfGrid &g, double a, double b, int mode,
 }
 void af_lat_final(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s) { launch_final(d, g, a, b, s); }
 void af_lat_lists(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s) { launch_lists(d, g, a, b, s); }
+
+#include "af_kernels1d.cuh"
