@@ -160,9 +160,18 @@ void bind_ptrs(af_ctx *c, const double *n, const double *st, double *o) {
   } while (0)
 #define TIMED(kernel, call) TIMED_ON(c->stream, kernel, call)
 
-// One stage: P1..P5 on the bound buffers.
-void run_stage(af_ctx *c, double a, double b, int reduce_dt) {
-  TIMED(AF_K_POINTDATA, af_launch_pointdata(c->dev, c->g, reduce_dt, c->stream));
+// One stage: P1..P5 on the bound buffers.  keep_pd: the point data of every DoF is used after
+// the stage (the adjoint), so no tile is passed over.
+void run_stage(af_ctx *c, double a, double b, int reduce_dt, bool keep_pd = false) {
+  c->dev.lev = nullptr;
+  if (!keep_pd && af_quiet_grid(c->g) && !c->dev.rec && !c->dev.frz) {
+    c->dev.lev = c->dev.quiet + 2 * af_quiet_tiles(c->g);
+    c->dev.ntx = (c->g.nxa + 31) / 32;
+  }
+  TIMED(AF_K_POINTDATA, {
+    if (c->dev.lev) af_launch_quiet(c->dev, c->g, c->stream);
+    af_launch_pointdata(c->dev, c->g, reduce_dt, c->stream);
+  });
   TIMED(AF_K_POINTS, af_launch_points(c->dev, c->g, a, b, 0, c->stream));
   const bool lists = c->g.pp_on && !c->dev.frz, small = af_small_grid(c->g);
   if (lists && !small) {
@@ -180,6 +189,7 @@ void run_stage(af_ctx *c, double a, double b, int reduce_dt) {
   else if (lists) TIMED(AF_K_CELLS_SLOW, af_launch_cells_slow(c->dev, c->g, c->stream));
   if (c->g.pp_on) TIMED(AF_K_FINAL, af_launch_final(c->dev, c->g, a, b, c->stream));
   if (lists && !small) cudaStreamWaitEvent(c->stream, c->ev_join, 0);
+  c->dev.lev = nullptr;   // the levels are those of this stage's input
 }
 
 const double RK_A[3] = {0.0, 3.0 / 4.0, 1.0 / 3.0};
@@ -254,7 +264,8 @@ int af_create(int nx, int ny, double gamma, int bc, af_ctx **out) {
   const size_t PS = (size_t)c->g.nxa * c->g.nya;
   // stage work arrays, then the limiter work lists: points (3 PS entries: an int and 8
   // doubles each), cells (PS entries: an int and 2 doubles each)
-  const size_t nwork = PS * (AF_NQA + 4 * AF_NQP + 8 + 4 + 2 * AF_NQF + 4 + 8 + 2) + PS * (24 + 2) + 2 * PS + 1;
+  const size_t nwork = PS * (AF_NQA + 4 * AF_NQP + 8 + 4 + 2 * AF_NQF + 4 + 8 + 2) + PS * (24 + 2) + 2 * PS + 1 +
+                       (3 * af_quiet_tiles(c->g) + 7) / 8;
   int rc = AF_OK;
   for (int b = 0; b < 3; ++b) {
     if (cudaMalloc(&c->state[b], off * sizeof(double)) != cudaSuccess) rc = AF_ENOMEM;
@@ -292,6 +303,7 @@ int af_create(int nx, int ny, double gamma, int bc, af_ctx **out) {
   c->dev.cqe = w; w += 2 * PS;
   c->dev.pq = reinterpret_cast<int *>(w); w += (3 * PS + 1) / 2;
   c->dev.cq = reinterpret_cast<int *>(w); w += (PS + 1) / 2;
+  c->dev.quiet = reinterpret_cast<unsigned char *>(w);
   c->dev.sc = c->sc;
   c->dev.st = c->st;
   c->cur = 0;
@@ -650,10 +662,10 @@ int af_adjoint_step(af_ctx *c, const double *dt, int dt_on_device, const double 
   const int n = c->cur, b1 = (c->cur + 1) % 3, b2 = (c->cur + 2) % 3;
   bind_pd(c, 0);
   bind_states(c, n, n, b1);
-  run_stage(c, RK_A[0], RK_B[0], 0);
+  run_stage(c, RK_A[0], RK_B[0], 0, true);
   bind_pd(c, 1);
   bind_states(c, n, b1, b2);
-  run_stage(c, RK_A[1], RK_B[1], 0);
+  run_stage(c, RK_A[1], RK_B[1], 0, true);
   bind_pd(c, 2);
   if ((flags & AF_ADJ_RECORDED) && !with_dt) {
     bind_states(c, b2, b2, b2);
@@ -661,7 +673,7 @@ int af_adjoint_step(af_ctx *c, const double *dt, int dt_on_device, const double 
   } else {
     bind_states(c, n, b2, b1);
     for (int cls = 0; cls < 4; ++cls) c->dev.uo[cls] = abuf(c, 5) + c->class_off[cls];
-    run_stage(c, RK_A[2], RK_B[2], 0);
+    run_stage(c, RK_A[2], RK_B[2], 0, true);
   }
   CK(cudaGetLastError(), "stage recompute");
   CK(cudaMemcpyAsync(c->cnt_pin + 16, c->st->cnt, cnt_bytes, cudaMemcpyDeviceToHost, c->stream), "read status");

@@ -123,6 +123,9 @@ void bind_stage1(af1d_ctx *c, int s) {
 }
 
 // Stages s0..s1 in one launch (short grids)
+#ifndef AF_QUIET1_MIN
+#define AF_QUIET1_MIN (1 << 20)
+#endif
 #ifndef AF_STEP1D_MAX
 #define AF_STEP1D_MAX 4096
 #endif
@@ -145,7 +148,10 @@ int stage1(af1d_ctx *c, int s, int reduce_dt) {
   if (c->cluster && !c->tm.on) return stages1(c, s, s, reduce_dt);
   const int b1 = (c->cur + 1) % 3, b2 = (c->cur + 2) % 3;
   bind_stage1(c, s);
+  // quiet tiles: from 2^20 cells on a stage takes about a millisecond, the check about 10 us
+  c->dev.lev = c->prm.pp_on && c->nf >= AF_QUIET1_MIN ? c->dev.quiet + 2 * af_quiet_tiles1d(c->g) : nullptr;
   af_launch_stage1d(c->dev, c->g, RK1_A[s], RK1_B[s], reduce_dt, c->stream, &c->tm);
+  c->dev.lev = nullptr;
   CK1(cudaGetLastError(), "stage launch");
   c->last_out = s == 1 ? b2 : b1;
   if (s == 2) c->cur = b1;
@@ -182,7 +188,7 @@ int af1d_create(int n, double gamma, int bc, af1d_ctx **out) {
   c->off1 = (size_t)8 * n;
   c->state_len = c->off1 + (size_t)8 * c->nf;
   const size_t PS = (size_t)c->nf;
-  const size_t nwork = PS * (AF_NQA + 2 * AF_NQP + 8 + 4 + AF_NQF + 4 + 8 + 1);
+  const size_t nwork = PS * (AF_NQA + 2 * AF_NQP + 8 + 4 + AF_NQF + 4 + 8 + 1) + (3 * af_quiet_tiles1d(c->g) + 7) / 8;
   int rc = AF_OK;
   for (int b = 0; b < 3 && !rc; ++b)
     if (cudaMalloc(&c->state[b], c->state_len * sizeof(double)) != cudaSuccess ||
@@ -212,6 +218,7 @@ int af1d_create(int n, double gamma, int bc, af1d_ctx **out) {
   c->dev.lam = w; w += 4 * PS;
   c->dev.lim1 = w; w += 8 * PS;
   c->dev.thx = w; w += PS;
+  c->dev.quiet = reinterpret_cast<unsigned char *>(w);
   c->dev.sc = c->sc;
   c->dev.st = c->st;
   c->cluster = c->nf <= AF_STEP1D_MAX ? af_lat_step1d_cluster(c->nf) : 0;

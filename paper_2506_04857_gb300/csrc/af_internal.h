@@ -100,6 +100,11 @@ struct AfDev {
   int *pq, *cq;
   double *pqu, *cqe;
   int pq_cap, cq_cap;
+  // quiet tiles (large grids): flags, deep flags and levels, a byte per tile of 32 x 4 index
+  // points each; lev is set for the stages that use the levels
+  unsigned char *quiet;
+  const unsigned char *lev;
+  int ntx;
 };
 
 // one member of a batch (af_batch.cu): its work pointers and grid
@@ -123,6 +128,10 @@ void af_lat_cells(const AfDev &d, const AfGrid &g, double a, double b, int mode,
 void af_lat_final(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s);
 void af_lat_lists(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s);   // both work lists
 bool af_small_grid(const AfGrid &g);   // which build the launchers below take
+// levels of the quiet tiles of the stage input; af_quiet_grid: whether a grid's stages use them
+void af_launch_quiet(const AfDev &d, const AfGrid &g, cudaStream_t s);
+bool af_quiet_grid(const AfGrid &g);
+inline size_t af_quiet_tiles(const AfGrid &g) { return (size_t)((g.nxa + 31) / 32) * ((g.nya + 3) / 4); }
 // the limiter slow paths over the work lists the point and cell passes filled
 void af_launch_points_slow(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s);
 void af_launch_cells_slow(const AfDev &d, const AfGrid &g, cudaStream_t s);
@@ -220,6 +229,7 @@ void af_launch_stage1d(const AfDev &d, const AfGrid &g, double a, double b, int 
 // Stages s0..s1 of a step of a short 1D grid in one cluster launch (d: the three stages' bindings)
 int af_lat_step1d_cluster(int n);
 void af_lat_step1d(const AfDev *d, const AfGrid &g, int s0, int s1, int reduce_dt, int cluster, cudaStream_t s);
+size_t af_quiet_tiles1d(const AfGrid &g);
 void af_launch_dt1d(const AfDev &d, const AfGrid &g, cudaStream_t s);
 // divergence measures of Example 4.4 of the state bound in d.us into out[2]
 // (device); partials: 2 * af_divb_nblocks(g) doubles

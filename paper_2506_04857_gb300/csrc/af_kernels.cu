@@ -31,10 +31,10 @@
 namespace {
 
 #ifndef AF_KBPT
-#define AF_KBPT 2
+#define AF_KBPT 4
 #endif
 #ifndef AF_KBPD
-#define AF_KBPD 1
+#define AF_KBPD 3
 #endif
 #ifndef AF_KBCL
 #define AF_KBCL 2
@@ -285,6 +285,13 @@ inline dim3 grid2(int nx, int ny) { return dim3((nx + 31) / 32, (ny + 3) / 4); }
 #endif
 // small grids
 bool af_small_grid(const AfGrid &g) { return (long long)((g.nxa + 31) / 32) * g.nya <= AF_SMALL; }
+
+#ifndef AF_QUIET_MIN
+#define AF_QUIET_MIN (1 << 19)
+#endif
+// From 2^19 index points on: a stage then takes over a millisecond, the check about 10 us.
+bool af_quiet_grid(const AfGrid &g) { return !g.special && g.pp_on && !g.upwind && (long long)g.nxa * g.nya >= AF_QUIET_MIN; }
+void af_launch_quiet(const AfDev &d, const AfGrid &g, cudaStream_t s) { launch_quiet(d, g, s); }
 
 void af_launch_pointdata(const AfDev &d, const AfGrid &g, int reduce_dt, cudaStream_t s) {
   if (af_small_grid(g)) af_lat_pointdata(d, g, reduce_dt, s);

@@ -44,7 +44,11 @@ __device__ __forceinline__ void b1_pointdata(const AfDev &d, const AfGrid &g, in
     const SV P = sview(d.us[1], g, 1);
     const int ip = mface(i + 1, g.nx, g.bc);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) uc[k] = (fma(6.0, A[k], -P(i, 0, k)) - P(ip, 0, k)) * 0.25;
+    for (int k = 0; k < 8; ++k) {
+      const double pl = P(i, 0, k), pr = P(ip, 0, k), v = (fma(6.0, A[k], -pl) - pr) * 0.25;
+      // equal values give exactly that value (uniform data stay uniform bit for bit)
+      uc[k] = ((bits(pl) ^ bits(A[k])) | (bits(pr) ^ bits(A[k]))) == 0 ? A[k] : v;
+    }
     if (!clear_of_floor(uc, g)) {   // Remark 3.2
       double out[8], t1, t2;
       scaling_limiter(uc, A, g.gm1, out, t1, t2);
@@ -431,29 +435,117 @@ __global__ void __launch_bounds__(3 * kStepThreads) k1_step(const __grid_constan
   }
 }
 #else
+// Quiet tiles of 128 indices, as in 2D (levels d.lev, one per block)
+constexpr int kTile1 = 128;
+__device__ __forceinline__ int level1(const AfDev &d) { return d.lev ? AF_LD(d.lev + blockIdx.x) : 0; }
+__global__ void __launch_bounds__(kTile1) k1_quiet1(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g) {
+  pass_begin();
+  const int i0 = blockIdx.x * kTile1, i = i0 + threadIdx.x;
+  const SV P = sview(d.us[1], g, 1), A = sview(d.us[0], g, 0);
+  bool ok = true;
+  for (int s = 0; s < 8 && ok; ++s) {
+    const int k = 7 - s;
+    const double v = P(i0, 0, k);
+    const bool eq = (i >= g.ex[1] || same_value(P(i, 0, k), v)) && (i >= g.nx || same_value(A(i, 0, k), v));
+    ok = __all_sync(0xffffffffu, eq);
+  }
+  ok = __syncthreads_and(ok);
+  if (threadIdx.x == 0) {
+    if (ok) {
+      double V[8];
+      load8(P, i0, 0, V);
+      ok = ge_pos(V[0], 1e-13) && qform_cert32(V, g.c13);
+    }
+    d.quiet[blockIdx.x] = ok;
+  }
+}
+__global__ void __launch_bounds__(128) k1_quiet23(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
+                                                  int pass) {
+  pass_begin();
+  b_quiet23<kTile1, 1, 1>(d, g, pass);
+}
+// As quiet_cfl, one dimension
+__device__ __noinline__ bool quiet_cfl1(const AfDev &d, const AfGrid &g, int i) {
+  double V[8];
+  load8(sview(d.us[0], g, 0), i, 0, V);
+  const double dt = d.sc->dt;
+  const float rho = (float)V[0], bb = (float)(V[4]) * (float)(V[4]) + (float)(V[5]) * (float)(V[5]) + (float)(V[6]) * (float)(V[6]);
+  const float cf = sqrtf((1.0001f * (float)(g.gamma * g.gm1) * (float)V[7] + bb) / rho);
+  if (2.0f * (float)dt * (fabsf((float)V[1]) / rho + cf) * (float)g.rdx < 0.999f) return false;
+  Full f;
+  full_data(V, g, f);
+  const double al = alpha_llf(f.v[0], f.v[0], f.cf[0], f.cf[0], f.srho, f.srho, f.B, f.B);
+  return dt * ((al + al) * g.rdx) > 1.0 + 1e-12;
+}
+
+// blockIdx.y: the point, the average or the centre of a cell (one body at a time in the
+// instruction cache, as in 2D)
 __global__ void __launch_bounds__(128) k1_pointdata(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                                     int reduce_dt) {
-  b1_pointdata(d, g, blockIdx.x * blockDim.x + threadIdx.x, reduce_dt);
+  pass_begin();
+  if (level1(d) > 4 && !(reduce_dt && blockIdx.y == 0 && threadIdx.x < 32)) return;
+  b1_pointdata(d, g, blockIdx.x * blockDim.x + threadIdx.x, reduce_dt, 1 << blockIdx.y);
 }
+// blockIdx.y: the point, the sensor
 __global__ void __launch_bounds__(128) k1_points(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                                  double a, double b) {
-  b1_points(d, g, blockIdx.x * blockDim.x + threadIdx.x, a, b);
+  pass_begin();
+  const int lev = level1(d), i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (blockIdx.y == 0 && lev > 0) {
+    const SV P = sview(d.us[1], g, 1);
+    const size_t cs = (size_t)g.ex[1];
+    if (i < g.ex[1])
+#pragma unroll
+      for (int k = 0; k < 8; ++k) rk_store(d.uo[1] + k * cs + i, d.un[1] + k * cs + i, a, b, P(i, 0, k));
+    return;
+  }
+  if (blockIdx.y == 0 || lev <= 3) b1_points(d, g, i, a, b, 1 << blockIdx.y);
 }
 __global__ void __launch_bounds__(128) k1_faces(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g) {
-  b1_faces(d, g, blockIdx.x * blockDim.x + threadIdx.x);
+  pass_begin();
+  if (level1(d) <= 2) b1_faces(d, g, blockIdx.x * blockDim.x + threadIdx.x);
 }
 __global__ void __launch_bounds__(128) k1_cells(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                                 double a, double b) {
-  b1_cells(d, g, blockIdx.x * blockDim.x + threadIdx.x, a, b);
+  pass_begin();
+  const int lev = level1(d), i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (lev > 0) {
+    if (i < g.nx && threadIdx.x % 32 == 0 && quiet_cfl1(d, g, i))
+      atomicAdd(&d.st->cnt[ST_CFL_VIOLATIONS], (unsigned long long)min(32, g.nx - i));
+    if (i < g.nx && lev == 1) {
+      const SV A = sview(d.us[0], g, 0);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) d.lim1[(size_t)k * g.nxa + i] = A(i, 0, k);
+      d.lam[i] = d.lam[(size_t)g.nxa + i] = 1.0;
+    }
+    return;
+  }
+  b1_cells(d, g, i, a, b);
 }
 __global__ void __launch_bounds__(128) k1_final(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                                 double a, double b) {
-  b1_final(d, g, blockIdx.x * blockDim.x + threadIdx.x, a, b);
+  pass_begin();
+  const int lev = level1(d), i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (lev > 0) {
+    if (i >= g.nx) return;
+    const SV A = sview(d.us[0], g, 0);
+    const size_t cs0 = (size_t)g.nx;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) rk_store(d.uo[0] + k * cs0 + i, d.un[0] + k * cs0 + i, a, b, A(i, 0, k));
+    if (lev == 1) {
+      d.thx[i] = 1.0;
+      if (g.bc == 1 && i == g.nx - 1) d.thx[i + 1] = 1.0;
+    }
+    return;
+  }
+  b1_final(d, g, i, a, b);
 }
 __global__ void k1_dt(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g) {
+  pass_begin();
   if (threadIdx.x == 0 && blockIdx.x == 0) b_dt(d, g);
 }
 __global__ void k1_repair(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g, double a, double b) {
+  pass_begin();
   if (blockIdx.x == 0 && threadIdx.x == 0) b1_repair(d, g, a, b);
 }
 #endif
@@ -501,29 +593,40 @@ void af_lat_step1d(const AfDev *d, const AfGrid &g, int s0, int s1, int reduce_d
 }
 #else
 
+// threads per block: a warp until every SM has four of them, which is when the FP64 pipe is full
+static unsigned threads1d(const AfGrid &g) { return g.nxa <= 152 * kTile1 ? 32 : kTile1; }
+
 // One 1D stage: P1 (with the dt pass when reduce_dt), P2..P5 and the repair
 // pass; t (may be NULL) brackets each launch with an event pair.
 void af_launch_stage1d(const AfDev &d, const AfGrid &g, double a, double b, int reduce_dt, cudaStream_t s,
                        AfEventTimer *t) {
-  const unsigned nb = (unsigned)((g.nxa + 127) / 128);
+  const unsigned nt = threads1d(g), nb = (unsigned)((g.nxa + nt - 1) / nt);
   auto timed = [&](int k, auto launch) {
     const bool on = t && t->begin(k, s);
     launch();
     if (t) t->end(on, s);
   };
-  timed(AF_K_POINTDATA, [&] { k1_pointdata<<<nb, 128, 0, s>>>(d, g, reduce_dt); });
-  if (reduce_dt) timed(AF_K_DT, [&] { k1_dt<<<1, 32, 0, s>>>(d, g); });
-  timed(AF_K_POINTS, [&] { k1_points<<<nb, 128, 0, s>>>(d, g, a, b); });
-  timed(AF_K_FACES, [&] { k1_faces<<<nb, 128, 0, s>>>(d, g); });
-  timed(AF_K_CELLS, [&] { k1_cells<<<nb, 128, 0, s>>>(d, g, a, b); });
+  timed(AF_K_POINTDATA, [&] {
+    if (d.lev) {
+      pass(k1_quiet1, nb, nt, s, d, g);
+      pass(k1_quiet23, (nb + 127) / 128, 128, s, d, g, 0);
+      pass(k1_quiet23, (nb + 127) / 128, 128, s, d, g, 1);
+    }
+    pass(k1_pointdata, dim3(nb, 3), nt, s, d, g, reduce_dt);
+  });
+  if (reduce_dt) timed(AF_K_DT, [&] { pass(k1_dt, 1, 32, s, d, g); });
+  timed(AF_K_POINTS, [&] { pass(k1_points, dim3(nb, g.kappa != 0.0 ? 2 : 1), nt, s, d, g, a, b); });
+  timed(AF_K_FACES, [&] { pass(k1_faces, nb, nt, s, d, g); });
+  timed(AF_K_CELLS, [&] { pass(k1_cells, nb, nt, s, d, g, a, b); });
   if (g.pp_on) {
-    timed(AF_K_FINAL, [&] { k1_final<<<nb, 128, 0, s>>>(d, g, a, b); });
-    timed(AF_K_REPAIR, [&] { k1_repair<<<1, 32, 0, s>>>(d, g, a, b); });
+    timed(AF_K_FINAL, [&] { pass(k1_final, nb, nt, s, d, g, a, b); });
+    timed(AF_K_REPAIR, [&] { pass(k1_repair, 1, 32, s, d, g, a, b); });
   }
 }
+size_t af_quiet_tiles1d(const AfGrid &g) { return (size_t)((g.nxa + kTile1 - 1) / kTile1); }
 void af_launch_dt1d(const AfDev &d, const AfGrid &g, cudaStream_t s) {
-  const unsigned nb = (unsigned)((g.nxa + 127) / 128);
-  k1_pointdata<<<nb, 128, 0, s>>>(d, g, 1);
-  k1_dt<<<1, 32, 0, s>>>(d, g);
+  const unsigned nt = threads1d(g), nb = (unsigned)((g.nxa + nt - 1) / nt);
+  pass(k1_pointdata, dim3(nb, 3), nt, s, d, g, 1);
+  pass(k1_dt, 1, 32, s, d, g);
 }
 #endif

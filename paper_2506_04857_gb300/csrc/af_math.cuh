@@ -401,17 +401,15 @@ __device__ __forceinline__ unsigned long long fx_shr(unsigned long long m, unsig
   asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"(s));
   return r;
 }
-// the significand of x with its sign, aligned to the exponent field emax (in place in the high
-// word), in ones' complement: the value minus one for a negative x.  neg: -1 for a negative x
-// (the caller adds the ones of its sum at once)
+// the signed significand of x, aligned to the exponent field emax (in place in the high word)
 template <int G>
-__device__ __forceinline__ long long fx_term(double x, unsigned emax, int &neg) {
+__device__ __forceinline__ long long fx_term(double x, unsigned emax) {
   const unsigned long long b = bits(x);
   const unsigned hi = (unsigned)(b >> 32);
   const unsigned s = (emax - (hi & 0x7ff00000u)) >> 20;
   const unsigned long long m = (((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | (unsigned)b) << G;
-  neg = (int)hi >> 31;
-  return (long long)fx_shr(m, s) ^ (long long)neg;
+  const long long neg = (int)hi >> 31;
+  return ((long long)fx_shr(m, s) ^ neg) - neg;
 }
 // the double nearest to acc 2^(e - G), in units of the last place, e the exponent of the field emax
 template <int G>
@@ -437,12 +435,10 @@ AF_ONCE double up5(double u0, double u1, double u2, double u3, double u4) {
     if (((bits(u0) | bits(u1) | bits(u2) | bits(u3) | bits(u4)) << 1) == 0) return 0.0;
     return up5_hw(u0, u1, u2, u3, u4);
   }
-  int n0, n1, n2, n3, n4;
-  const long long v2 = fx_term<6>(u2, em, n2), t13 = fx_term<6>(u1, em, n1) + fx_term<6>(u3, em, n3);
-  const long long t04 = fx_term<6>(u0, em, n0) + fx_term<6>(u4, em, n4);
+  const long long v2 = fx_term<6>(u2, em), t13 = fx_term<6>(u1, em) + fx_term<6>(u3, em);
+  const long long t04 = fx_term<6>(u0, em) + fx_term<6>(u4, em);
   const long long w = v2 + ((v2 - t13) << 1);   // 3 u2 - 2 (u1 + u3)
-  const int ones = (n0 + n4) - 4 * (n1 + n3) + 6 * n2;
-  return fx_round<6>(t04 + (w << 1) - ones, em);
+  return fx_round<6>(t04 + (w << 1), em);
 }
 
 }  // namespace afm

@@ -280,6 +280,23 @@ __device__ __forceinline__ void load8(const SV &v, int i, int j, double *U) {
   for (int k = 0; k < 8; ++k) U[k] = v(i, j, k);
 }
 
+// Whether component k of the eight points of cell (i, j) equals a bit for bit
+__device__ __forceinline__ bool same_nine(const SV &X, const SV &Y, const SV &C, int i, int ip, int j, int jp, int k,
+                                          double a) {
+  const unsigned long long b = bits(a);
+  return ((bits(X(i, j, k)) ^ b) | (bits(X(ip, j, k)) ^ b) | (bits(Y(i, j, k)) ^ b) | (bits(Y(i, jp, k)) ^ b) |
+          (bits(C(i, j, k)) ^ b) | (bits(C(ip, j, k)) ^ b) | (bits(C(i, jp, k)) ^ b) | (bits(C(ip, jp, k)) ^ b)) == 0;
+}
+// Whether all nine states of cell (i, j) are equal: its centre value is then that state exactly, not
+// within rounding, and uniform gas stays uniform bit for bit (quiet tiles).  Not inlined: the rare
+// case, and its loads would cost the point-data pass spills.
+__device__ __noinline__ bool uniform_cell(const AfDev &d, const AfGrid &g, int i, int ip, int j, int jp) {
+  const SV A = sview(d.us[0], g, 0), X = sview(d.us[1], g, 1), Y = sview(d.us[2], g, 2), C = sview(d.us[3], g, 3);
+  for (int k = 0; k < 8; ++k)
+    if (!same_nine(X, Y, C, i, ip, j, jp, k, A(i, j, k))) return false;
+  return true;
+}
+
 // Sec. 2.1 centre value [36 Ubar - 4 (faces) - (corners)] / 16 of cell (i, j),
 // limited toward the cell average A by Remark 3.2; true when the limiter acted.
 __device__ __forceinline__ bool centre_value(const AfDev &d, const AfGrid &g, int i, int j, const double *A,
@@ -292,6 +309,11 @@ __device__ __forceinline__ bool centre_value(const AfDev &d, const AfGrid &g, in
     const double corners = (C(i, j, k) + C(ip, j, k)) + (C(i, jp, k) + C(ip, jp, k));
     uc[k] = fma(2.25, A[k], fma(-0.25, faces, ldexp_i<-4>(neg_i(corners))));
   }
+  // a cell whose nine states are equal has that state at its centre (the energies end the test
+  // almost everywhere else)
+  if (same_nine(X, Y, C, i, ip, j, jp, 7, A[7]) && uniform_cell(d, g, i, ip, j, jp))
+#pragma unroll
+    for (int k = 0; k < 8; ++k) uc[k] = A[k];
   const size_t PS = (size_t)g.nxa * g.nya, o = (size_t)j * g.nxa + i;
   double t1 = 1.0, t2 = 1.0;
   if (d.frz) {   // frozen branch: the recorded theta*, theta**
@@ -744,6 +766,11 @@ __device__ void sensor_phi(const AfDev &d, const AfGrid &g, int ci, int cj, doub
   phi[3] = ddiv(absd(num), absd(Ub(ci, cj, 4) + Ub(ci, cj, 5)) + 1e-40);
 }
 
+// out = a U^n + b v of the Runge-Kutta stage (a = 0: v itself)
+__device__ __forceinline__ void rk_store(double *out, const double *un, double a, double b, double v) {
+  *out = is_zero(a) ? v : fma(a, AF_LD(un), mul_i(b, v));
+}
+
 struct PointCount {
   int lim, shr, bad;
 };
@@ -753,12 +780,20 @@ struct PointCount {
 //   kPlain: a stage of a single run with its work lists, nothing recorded or frozen: the slow
 //   paths are not compiled in.  Their call frames cost the point pass spills and the cell
 //   pass registers: cells 356 -> 319 us and points 694 -> 667 us (blast 1024^2).
+//   kQuiet: a plain stage with the levels of the quiet tiles.
 //   kStage: any stage.  kRhs: the semi-discrete right-hand side.
-enum { kStage = 0, kPlain = 1, kRhs = 2 };
+enum { kStage = 0, kPlain = 1, kRhs = 2, kQuiet = 3 };
 template <int cls, bool GB, bool UP, int K>
 __device__ __forceinline__ void b_point(const AfDev &d, const AfGrid &g, const int i, const int j, double a, double b,
-                                        PointCount &n) {
-  constexpr bool PL = K == kPlain, RHS = K == kRhs;
+                                        PointCount &n, bool quiet) {
+  constexpr bool PL = K == kPlain || K == kQuiet, RHS = K == kRhs;
+  if (K == kQuiet && quiet) {   // L(U) = 0: the RK combination of the state itself
+    const SV v = sview(d.us[cls], g, cls);
+    const size_t cs = (size_t)g.ex[cls] * g.ey[cls], oo = (size_t)j * g.ex[cls] + i;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) rk_store(d.uo[cls] + k * cs + oo, d.un[cls] + k * cs + oo, a, b, v(i, j, k));
+    return;
+  }
   const size_t PS = (size_t)g.nxa * g.nya;
   const double dt = RHS ? 1.0 : d.sc->dt;
   const double cxc = mul_i(dt, g.rdx), cyc = mul_i(dt, g.rdy);   // central differences
@@ -899,14 +934,14 @@ __device__ __forceinline__ void b_sensor(const AfDev &d, const AfGrid &g, const 
 // slowest grid index): the code of one class at a time stays in the SM's instruction cache.
 template <bool GB, bool UP, int K>
 __device__ __forceinline__ void b_points(const AfDev &d, const AfGrid &g, const int i, const int j, double a, double b,
-                                         int mode, int z) {
+                                         int mode, int z, int lev = 0) {
   PointCount n = {0, 0, 0};
   if (z == 3) {
-    if (K != kRhs) b_sensor<GB>(d, g, i, j);
+    if (K != kRhs && lev <= 3) b_sensor<GB>(d, g, i, j);
   } else if (mode != 2 && i < g.ex[z + 1] && j < g.ey[z + 1]) {
-    if (z == 0) b_point<1, GB, UP, K>(d, g, i, j, a, b, n);
-    else if (z == 1) b_point<2, GB, UP, K>(d, g, i, j, a, b, n);
-    else b_point<3, GB, UP, K>(d, g, i, j, a, b, n);
+    if (z == 0) b_point<1, GB, UP, K>(d, g, i, j, a, b, n, lev > 0);
+    else if (z == 1) b_point<2, GB, UP, K>(d, g, i, j, a, b, n, lev > 0);
+    else b_point<3, GB, UP, K>(d, g, i, j, a, b, n, lev > 0);
   }
   if (K != kStage) return;
   if (n.lim) atomicAdd(&d.st->cnt[ST_POINT_LIMITED], (unsigned long long)n.lim);
@@ -1907,6 +1942,145 @@ __device__ __forceinline__ void b_cells_lists(const AfDev &d, const AfGrid &g, c
   }
 }
 
+// ---------------------------------------------------------------------------
+// Quiet tiles.  Much of a blast, cloud or jet run is gas that nothing has reached yet.  Where
+// every DoF within the reach of a stage (3 indices) holds the same state V bit for bit, and V
+// is admissible with room to spare (the FP32 certificate), FE(V) = V exactly: every difference
+// of the scheme cancels to 0, no limiter acts, and the passes have nothing to form.
+//   k_quiet1: per tile (32 x 4 index points, the tiles of the passes) whether all its DoFs
+//     equal the corner value of its first point and that state is certified;
+//   k_quiet2: whether the tiles two to every side are so too, with the same state;
+//   k_quiet3: the level of each tile: its distance, in tiles, to one that is not (0), at most 5.
+// Level 0 runs everything.  What a level-0 tile reads of its neighbours is formed there as
+// usual: Lambda, Lim1 and theta at level 1 (the values 1, V and 1), faces up to level 2,
+// sensor values up to 3, point data up to 4; each pass reaches one index, so one tile per pass
+// (a last tile may hold a single row or column).  The rest is not touched, but for the
+// Runge-Kutta combination.  Grids with reflective or inflow sides, recorded or frozen stages
+// and small grids (whose passes are as short as a launch) do not take it.  Without quiet
+// tiles the check costs one load per point and class and three launches (Orszag-Tang 1536 x 1536:
+// 14.12 -> 14.3 ms for a step with its copies); the 2048 x 2048 blast, 1/6 of it disturbed, takes
+// 19.7 ms for two steps instead of 45.4.
+// ---------------------------------------------------------------------------
+// equal bit for bit, or zeros of either sign
+__device__ __forceinline__ bool same_value(double x, double y) {
+  return bits(x) == bits(y) || ((bits(x) | bits(y)) << 1) == 0;
+}
+__device__ __forceinline__ bool same_state(const AfDev &d, const AfGrid &g, int cls, int ia, int ja, int ib, int jb) {
+  const SV C = sview(d.us[cls], g, cls);
+  for (int k = 0; k < 8; ++k)
+    if (!same_value(C(ia, ja, k), C(ib, jb, k))) return false;
+  return true;
+}
+__device__ __forceinline__ void b_quiet1(const AfDev &d, const AfGrid &g) {
+  const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 4, i = i0 + threadIdx.x, j = j0 + threadIdx.y;
+  const SV C = sview(d.us[3], g, 3);
+  bool ok = true;
+  // the energy at the corners first: it ends most tiles of a flow without quiet gas
+  for (int s = 0; s < 8 && ok; ++s) {
+    const int k = 7 - s;
+    const double v = C(i0, j0, k);
+    bool eq = true;
+#pragma unroll
+    for (int c = 3; c >= 0; --c)
+      if (i < g.ex[c] && j < g.ey[c]) eq = eq && same_value(sview(d.us[c], g, c)(i, j, k), v);
+    ok = __all_sync(0xffffffffu, eq);
+  }
+  ok = __syncthreads_and(ok);
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
+    if (ok) {
+      double V[8];
+      load8(C, i0, j0, V);
+      ok = ge_pos(V[0], 1e-13) && qform_cert32(V, g.c13);
+    }
+    d.quiet[blockIdx.y * gridDim.x + blockIdx.x] = ok;
+  }
+}
+// tile index shifted by q, wrapped (periodic) or -1 outside
+__device__ __forceinline__ int shift_tile(int t, int q, int n, int bc) {
+  t += q;
+  if (t >= 0 && t < n) return t;
+  if (bc != 0) return -1;
+  t %= n;
+  return t < 0 ? t + n : t;
+}
+// pass 0: flags -> deep flags (radius 2); pass 1: deep flags -> levels (radius 4).  Tiles of W x H
+// index points, compared by the first point of class cls.
+template <int W, int H, int cls>
+__device__ __forceinline__ void b_quiet23(const AfDev &d, const AfGrid &g, int pass) {
+  const int ntx = (g.nxa + W - 1) / W, nty = (g.nya + H - 1) / H, nt = ntx * nty;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= nt) return;
+  const int tx = t % ntx, ty = t / ntx;
+  const unsigned char *in = d.quiet + (size_t)pass * nt;
+  int res = pass == 0 ? in[t] : (in[t] ? 5 : 0);
+  const int R = pass == 0 ? 2 : 4;
+  for (int q = -R; q <= R && res; ++q) {
+    const int y = nty == 1 ? (q == 0 ? 0 : -1) : shift_tile(ty, q, nty, g.bc);
+    if (y < 0) continue;
+    for (int p = -R; p <= R && res; ++p) {
+      const int x = shift_tile(tx, p, ntx, g.bc);
+      if (x < 0) continue;
+      const unsigned char f = in[y * ntx + x];
+      if (pass == 0) res = f && same_state(d, g, cls, tx * W, ty * H, x * W, y * H);
+      else if (!f) res = min(res, max(abs(p), abs(q)));
+    }
+  }
+  d.quiet[(size_t)(pass + 1) * nt + t] = (unsigned char)res;
+}
+__global__ void __launch_bounds__(128) k_quiet1(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g) {
+  pass_begin();
+  b_quiet1(d, g);
+}
+__global__ void __launch_bounds__(128) k_quiet23(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
+                                                 int pass) {
+  pass_begin();
+  b_quiet23<32, 4, 3>(d, g, pass);
+}
+// level of the block's tile (0 where no levels are kept)
+__device__ __forceinline__ int tile_level(const AfDev &d) {
+  return d.lev ? AF_LD(d.lev + (size_t)blockIdx.y * d.ntx + blockIdx.x) : 0;
+}
+// The Lemma 3.1 CFL count of the cells of a quiet tile, all alike: the cell pass's expression with
+// both states V.  An FP32 upper bound of it decides first (cf^2 <= (gamma (gamma - 1) E + |B|^2) / rho).
+__device__ __noinline__ bool quiet_cfl(const AfDev &d, const AfGrid &g, int i, int j) {
+  double V[8];
+  load8(sview(d.us[0], g, 0), i, j, V);
+  const double dt = d.sc->dt;
+  const float rho = (float)V[0], bb = (float)(V[4]) * (float)(V[4]) + (float)(V[5]) * (float)(V[5]) + (float)(V[6]) * (float)(V[6]);
+  const float cf = sqrtf((1.0001f * (float)(g.gamma * g.gm1) * (float)V[7] + bb) / rho);
+  const float lhs = 2.0f * (float)dt * ((fabsf((float)V[1]) / rho + cf) * (float)g.rdx + (fabsf((float)V[2]) / rho + cf) * (float)g.rdy);
+  if (lhs < 0.999f) return false;   // an overflow or NaN goes on
+  Full f;
+  full_data(V, g, f);
+  const double a1 = alpha_llf(f.v[0], f.v[0], f.cf[0], f.cf[0], f.srho, f.srho, f.B, f.B);
+  const double a2 = alpha_llf(f.v[1], f.v[1], f.cf[1], f.cf[1], f.srho, f.srho, f.B, f.B);
+  return gt_pos(mul_i(dt, (a1 + a1) * g.rdx + (a2 + a2) * g.rdy), 1.0 + 1e-12);
+}
+__device__ __forceinline__ void quiet_cells(const AfDev &d, const AfGrid &g, const Tile &t, int lev) {
+  const bool in = t.i < g.nx && t.j < g.ny;
+  if (in && threadIdx.x == 0 && quiet_cfl(d, g, t.i, t.j))
+    atomicAdd(&d.st->cnt[ST_CFL_VIOLATIONS], (unsigned long long)min(32, g.nx - t.i));
+  if (!in || lev > 1) return;
+  const size_t PS = (size_t)g.nxa * g.nya, o = (size_t)t.j * g.nxa + t.i;
+  const SV U = sview(d.us[0], g, 0);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) d.lim1[k * PS + o] = U(t.i, t.j, k);
+#pragma unroll
+  for (int I = 0; I < 4; ++I) d.lam[I * PS + o] = 1.0;
+}
+__device__ __forceinline__ void quiet_final(const AfDev &d, const AfGrid &g, const int i, const int j, double a, double b,
+                                            int lev) {
+  if (!(i < g.nx && j < g.ny)) return;
+  const SV U = sview(d.us[0], g, 0);
+  const size_t cs0 = (size_t)g.nx * g.ny, o0 = (size_t)j * g.nx + i, o = (size_t)j * g.nxa + i;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) rk_store(d.uo[0] + k * cs0 + o0, d.un[0] + k * cs0 + o0, a, b, U(i, j, k));
+  if (lev > 1) return;
+  d.thx[o] = d.thy[o] = 1.0;
+  if (g.bc == 1 && i == g.nx - 1) d.thx[o + 1] = 1.0;
+  if (g.bc == 1 && j == g.ny - 1) d.thy[o + g.nxa] = 1.0;
+}
+
 // Launch bounds of the stage kernels (128 threads): a kernel given AF_MINB_x
 // resident blocks per SM is capped at 65536 / (128 x blocks) registers; without
 // it ptxas picks the count.  The kernels keep the FP64 pipe and the integer
@@ -1922,7 +2096,7 @@ __device__ __forceinline__ void b_cells_lists(const AfDev &d, const AfGrid &g, c
 #else
 #define AF_LB(minb) __launch_bounds__(128, minb)
 #ifndef AF_MINB_PD
-#define AF_MINB_PD 5
+#define AF_MINB_PD 8
 #endif
 #define AF_LB_PD AF_LB(AF_MINB_PD)
 #ifndef AF_MINB_PT
@@ -1953,6 +2127,8 @@ __global__ void AF_LB_PD k_pointdata(const __grid_constant__ AfDev d, const __gr
     d.st->ncq = 0;
   }
   const Tile t = tile();
+  // of a quiet tile nothing is read; its one state enters the time-step bound through one warp
+  if (tile_level(d) > 4 && !(reduce_dt && t.z == 0 && threadIdx.y == 0)) return;
   b_pointdata(d, g, t.i, t.j, reduce_dt, t.z + 1);
 #ifdef AF_LAT
   if (reduce_dt && last_block(&d.sc->ticket[0]) && threadIdx.x == 0) b_dt(d, g);
@@ -1972,14 +2148,16 @@ __global__ void AF_LB_PT k_points(const __grid_constant__ AfDev d, const __grid_
   pass_begin();
   if (K != kStage) mode = 0;
   const Tile t = tile();
-  if (GB && interior_block(g.nx, g.ny, t)) b_points<false, UP, K>(d, g, t.i, t.j, a, b, mode, t.z);
-  else b_points<GB, UP, K>(d, g, t.i, t.j, a, b, mode, t.z);
+  const int lev = K == kQuiet ? tile_level(d) : 0;
+  if (GB && interior_block(g.nx, g.ny, t)) b_points<false, UP, K>(d, g, t.i, t.j, a, b, mode, t.z, lev);
+  else b_points<GB, UP, K>(d, g, t.i, t.j, a, b, mode, t.z, lev);
 }
 template <bool GB>
 __global__ void AF_LB_FC k_faces(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                                int mode) {
   pass_begin();
   const Tile t = tile();
+  if (!GB && tile_level(d) > 2) return;
   if (GB && interior_block(g.nx, g.ny, t)) b_faces<false>(d, g, t.i, t.j, mode, t.z);
   else b_faces<GB>(d, g, t.i, t.j, mode, t.z);
 }
@@ -1988,13 +2166,22 @@ __global__ void AF_LB_CL k_cells(const __grid_constant__ AfDev d, const __grid_c
                                                double a, double b, int mode) {
   pass_begin();
   const Tile t = tile();
+  if (PL && !GB) {
+    const int lev = tile_level(d);
+    if (lev > 0) {
+      quiet_cells(d, g, t, lev);
+      return;
+    }
+  }
   if (GB && interior_block(g.nx, g.ny, t)) b_cells<false, PL>(d, g, t.i, t.j, a, b, mode);
   else b_cells<GB, PL>(d, g, t.i, t.j, a, b, mode);
 }
 __global__ void AF_LB_FN k_final(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                                double a, double b) {
   pass_begin();
-  b_final(d, g, AF_IJ, a, b);
+  const int lev = tile_level(d);
+  if (lev > 0) quiet_final(d, g, AF_IJ, a, b, lev);
+  else b_final(d, g, AF_IJ, a, b);
 #ifdef AF_LAT
   if (last_block(&d.sc->ticket[1]) && threadIdx.x == 0) b_repair(d, g, a, b);
 #endif
@@ -2058,6 +2245,14 @@ inline Shape shape(int nx, int ny, int nz) {
   return {dim3((nx + 31) / 32, (ny + kRows - 1) / kRows, nz), dim3(32, kRows)};
 }
 
+// levels of the quiet tiles of the stage input (d.quiet: three bytes per tile; the last is d.lev)
+void launch_quiet(const AfDev &d, const AfGrid &g, cudaStream_t s) {
+  const dim3 gr((g.nxa + 31) / 32, (g.nya + 3) / 4);
+  const int nb = (int)((gr.x * gr.y + 127) / 128);
+  pass(k_quiet1, gr, dim3(32, 4), s, d, g);
+  pass(k_quiet23, nb, 128, s, d, g, 0);
+  pass(k_quiet23, nb, 128, s, d, g, 1);
+}
 void launch_pointdata(const AfDev &d, const AfGrid &g, int reduce_dt, cudaStream_t s) {
   const Shape h = shape(g.nxa, g.nya, 5);
   pass(k_pointdata, h.g, h.b, s, d, g, reduce_dt);
@@ -2074,7 +2269,8 @@ void launch_points(const AfDev &d, const AfGrid &g, double a, double b, int mode
     else if (kind == kRhs) g.upwind ? go(k_points<true, true, kRhs>) : go(k_points<true, false, kRhs>);
     else g.upwind ? go(k_points<true, true, kStage>) : go(k_points<true, false, kStage>);
   } else {
-    if (kind == kPlain) go(k_points<false, false, kPlain>);
+    if (kind == kPlain && d.lev) go(k_points<false, false, kQuiet>);
+    else if (kind == kPlain) go(k_points<false, false, kPlain>);
     else if (kind == kRhs) g.upwind ? go(k_points<false, true, kRhs>) : go(k_points<false, false, kRhs>);
     else g.upwind ? go(k_points<false, true, kStage>) : go(k_points<false, false, kStage>);
   }
