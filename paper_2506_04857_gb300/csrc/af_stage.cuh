@@ -1763,14 +1763,64 @@ __device__ __forceinline__ Tile tile() {
   return {(int)(blockIdx.x * blockDim.x + threadIdx.x), (int)(blockIdx.y * blockDim.y + threadIdx.y), (int)blockIdx.z};
 }
 
-// On grids with reflective or inflow sides, a thread block whose whole tile
-// lies at least kFrame indices inside [0, nx) x [0, ny) touches no ghost (the
-// stencils of the point, face and cell passes reach 2 indices), so it runs the
-// plain code; only the blocks of the boundary frame resolve ghosts.
+// On grids with reflective or inflow sides, an index point at least kFrame indices inside
+// [0, nx) x [0, ny) touches no ghost (the stencils of the point, face and cell passes reach 2
+// indices) and runs the plain code.  The points of the frame resolve ghosts: the first rows of
+// blocks of such a launch walk the frame point by point, the others skip it.  (Deciding by whole
+// tiles put 2/7 of a 200-cell wide grid on the ghost code, several times slower than the plain
+// one; the frame itself is 1/20.)
 constexpr int kFrame = 4;
-__device__ __forceinline__ bool interior_block(int nx, int ny, const Tile &t) {
-  const int i0 = t.i - (int)threadIdx.x, j0 = t.j - (int)threadIdx.y;
-  return i0 >= kFrame && j0 >= kFrame && i0 + (int)blockDim.x + kFrame <= nx && j0 + (int)blockDim.y + kFrame <= ny;
+struct Frame {
+  int wi, hi, sc;   // inner extents, columns of the frame in an inner row
+  __host__ __device__ Frame(const AfGrid &g) : wi(g.nx - 2 * kFrame), hi(g.ny - 2 * kFrame), sc(g.nxa - wi) {}
+  __host__ __device__ bool all() const { return wi <= 0 || hi <= 0; }
+  __host__ __device__ long long count(const AfGrid &g) const {
+    return all() ? (long long)g.nxa * g.nya : (long long)g.nxa * (g.nya - hi) + (long long)sc * hi;
+  }
+};
+__device__ __forceinline__ bool in_frame(const AfGrid &g, int i, int j) {
+  return i < kFrame || j < kFrame || i >= g.nx - kFrame || j >= g.ny - kFrame;
+}
+// point t of the frame: the rows below and above the inner ones, then the columns beside them
+__device__ __forceinline__ void frame_point(const AfGrid &g, const Frame &f, int t, int &i, int &j) {
+  const int rows = f.all() ? g.nya : g.nya - f.hi;
+  if (t < rows * g.nxa) {
+    j = t / g.nxa;
+    i = t - j * g.nxa;
+    if (!f.all() && j >= kFrame) j += f.hi;
+  } else {
+    t -= rows * g.nxa;
+    j = t / f.sc;
+    i = t - j * f.sc;
+    j += kFrame;
+    if (i >= kFrame) i += f.wi;
+  }
+}
+// rows of blocks that walk the frame (0: no special sides) in a launch ntx blocks wide
+inline __host__ __device__ int frame_rows(const AfGrid &g, int ntx, int threads) {
+  if (!g.special) return 0;
+  const long long n = Frame(g).count(g);
+  return (int)((n + (long long)threads * ntx - 1) / ((long long)threads * ntx));
+}
+// The thread's tile in a launch on a grid with special sides (rows of ntx blocks, all in blockIdx.x:
+// blockIdx.y could not hold the frame's rows of a very tall grid): a frame point (true), a point of
+// the inner tiles (false), or nothing to do (t.i < 0)
+__device__ __forceinline__ bool frame_tile(const AfGrid &g, int nx, Tile &t) {
+  const int threads = blockDim.x * blockDim.y, ntx = (nx + 31) / 32, rows = frame_rows(g, ntx, threads);
+  const int by = blockIdx.x / ntx, bx = blockIdx.x - by * ntx;
+  t = {-1, 0, (int)blockIdx.z};
+  if (by < rows) {
+    const Frame f(g);
+    const long long p = (long long)blockIdx.x * threads + threadIdx.y * blockDim.x + threadIdx.x;
+    if (p < f.count(g)) frame_point(g, f, (int)p, t.i, t.j);
+    return true;
+  }
+  const int i = bx * blockDim.x + threadIdx.x, j = (by - rows) * blockDim.y + threadIdx.y;
+  if (!in_frame(g, i, j)) {
+    t.i = i;
+    t.j = j;
+  }
+  return false;
 }
 // ---- limiter slow paths over the work lists (single runs) -------------------
 // Points whose high-order update left the floors: Sec. 3.3 LLF state, scaling
@@ -2147,34 +2197,49 @@ __global__ void AF_LB_PT k_points(const __grid_constant__ AfDev d, const __grid_
                                                 double a, double b, int mode) {
   pass_begin();
   if (K != kStage) mode = 0;
-  const Tile t = tile();
-  const int lev = K == kQuiet ? tile_level(d) : 0;
-  if (GB && interior_block(g.nx, g.ny, t)) b_points<false, UP, K>(d, g, t.i, t.j, a, b, mode, t.z, lev);
-  else b_points<GB, UP, K>(d, g, t.i, t.j, a, b, mode, t.z, lev);
+  if constexpr (GB) {
+    Tile t;
+    const bool fr = frame_tile(g, g.nxa, t);
+    if (t.i < 0) return;
+    if (fr) b_points<true, UP, K>(d, g, t.i, t.j, a, b, mode, t.z);
+    else b_points<false, UP, K>(d, g, t.i, t.j, a, b, mode, t.z);
+  } else {
+    const Tile t = tile();
+    b_points<false, UP, K>(d, g, t.i, t.j, a, b, mode, t.z, K == kQuiet ? tile_level(d) : 0);
+  }
 }
 template <bool GB>
 __global__ void AF_LB_FC k_faces(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                                int mode) {
   pass_begin();
-  const Tile t = tile();
-  if (!GB && tile_level(d) > 2) return;
-  if (GB && interior_block(g.nx, g.ny, t)) b_faces<false>(d, g, t.i, t.j, mode, t.z);
-  else b_faces<GB>(d, g, t.i, t.j, mode, t.z);
+  if constexpr (GB) {
+    Tile t;
+    const bool fr = frame_tile(g, g.nxa, t);
+    if (t.i < 0) return;
+    if (fr) b_faces<true>(d, g, t.i, t.j, mode, t.z);
+    else b_faces<false>(d, g, t.i, t.j, mode, t.z);
+  } else {
+    const Tile t = tile();
+    if (tile_level(d) > 2) return;
+    b_faces<false>(d, g, t.i, t.j, mode, t.z);
+  }
 }
 template <bool GB, bool PL>
 __global__ void AF_LB_CL k_cells(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                                double a, double b, int mode) {
   pass_begin();
-  const Tile t = tile();
-  if (PL && !GB) {
-    const int lev = tile_level(d);
-    if (lev > 0) {
-      quiet_cells(d, g, t, lev);
-      return;
-    }
+  if constexpr (GB) {
+    Tile t;
+    const bool fr = frame_tile(g, g.nx, t);
+    if (t.i < 0) return;
+    if (fr) b_cells<true, PL>(d, g, t.i, t.j, a, b, mode);
+    else b_cells<false, PL>(d, g, t.i, t.j, a, b, mode);
+  } else {
+    const Tile t = tile();
+    const int lev = PL ? tile_level(d) : 0;
+    if (lev > 0) quiet_cells(d, g, t, lev);
+    else b_cells<false, PL>(d, g, t.i, t.j, a, b, mode);
   }
-  if (GB && interior_block(g.nx, g.ny, t)) b_cells<false, PL>(d, g, t.i, t.j, a, b, mode);
-  else b_cells<GB, PL>(d, g, t.i, t.j, a, b, mode);
 }
 __global__ void AF_LB_FN k_final(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                                double a, double b) {
@@ -2244,6 +2309,12 @@ void pass(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t s, A... args) {
 inline Shape shape(int nx, int ny, int nz) {
   return {dim3((nx + 31) / 32, (ny + kRows - 1) / kRows, nz), dim3(32, kRows)};
 }
+// of a pass that resolves ghosts: with the rows of blocks of the frame
+inline Shape shape(const AfGrid &g, int nx, int ny, int nz) {
+  Shape h = shape(nx, ny, nz);
+  if (g.special) h.g = dim3(h.g.x * (h.g.y + frame_rows(g, (int)h.g.x, 32 * kRows)), 1, nz);
+  return h;
+}
 
 // levels of the quiet tiles of the stage input (d.quiet: three bytes per tile; the last is d.lev)
 void launch_quiet(const AfDev &d, const AfGrid &g, cudaStream_t s) {
@@ -2261,7 +2332,7 @@ void launch_pointdata(const AfDev &d, const AfGrid &g, int reduce_dt, cudaStream
 #endif
 }
 void launch_points(const AfDev &d, const AfGrid &g, double a, double b, int mode, cudaStream_t s) {
-  const Shape h = shape(g.nxa, g.nya, mode != 1 && g.kappa != 0.0 ? 4 : 3);
+  const Shape h = shape(g, g.nxa, g.nya, mode != 1 && g.kappa != 0.0 ? 4 : 3);
   const int kind = mode == 1 ? kRhs : (mode == 0 && d.pq && !d.rec && !d.frz && !g.upwind ? kPlain : kStage);
   auto go = [&](auto k) { pass(k, h.g, h.b, s, d, g, a, b, mode); };
   if (g.special) {
@@ -2276,12 +2347,12 @@ void launch_points(const AfDev &d, const AfGrid &g, double a, double b, int mode
   }
 }
 void launch_faces(const AfDev &d, const AfGrid &g, int mode, cudaStream_t s) {
-  const Shape h = shape(g.nxa, g.nya, 2);
+  const Shape h = shape(g, g.nxa, g.nya, 2);
   if (g.special) pass(k_faces<true>, h.g, h.b, s, d, g, mode);
   else pass(k_faces<false>, h.g, h.b, s, d, g, mode);
 }
 void launch_cells(const AfDev &d, const AfGrid &g, double a, double b, int mode, cudaStream_t s) {
-  const Shape h = shape(g.nx, g.ny, 1);
+  const Shape h = shape(g, g.nx, g.ny, 1);
   const bool plain = mode == 0 && g.pp_on && d.cq && !d.rec && !d.frz;
   if (g.special) {
     if (plain) pass(k_cells<true, true>, h.g, h.b, s, d, g, a, b, mode);
