@@ -66,10 +66,23 @@ struct PI {
 };
 __device__ __forceinline__ bool same(const PI &a, const PI &b) { return a.c == b.c && a.i == b.i && a.j == b.j; }
 
-__constant__ double kCoefF[5] = {1.0, -4.0, 0.0, 4.0, -1.0};   // (F0 - F4) + 4 (F3 - F1)
-__constant__ double kCoefU[5] = {1.0, -4.0, 6.0, -4.0, 1.0};   // (U0 + U4) - 4 (U1 + U3) + 6 U2
-// coefficient of the node value at position l (0,1,2) in the derivative at node lp
-__constant__ double kD1[3][3] = {{-3.0, 4.0, -1.0}, {-1.0, 0.0, 1.0}, {1.0, -4.0, 3.0}};
+// Stencil coefficients are small integers: they are added up as integers and widened once
+// (a predicated FP64 sum per point of a line, and the FP64 products with 0 and 1, took as many
+// issue slots of the FP64 pipe as the gathered products themselves).  With the line coefficients
+// multiplied once per line instead of once per component: A2 207 -> 159 us, A1 (whose second
+// differences are now up5) 65 -> 46 us per transpose at 256 x 256.
+__device__ __forceinline__ int coef_f(int p) { return p == 0 ? 1 : (p == 1 ? -4 : (p == 2 ? 0 : (p == 3 ? 4 : -1))); }   // (F0 - F4) + 4 (F3 - F1)
+__device__ __forceinline__ int coef_u(int p) { return p == 2 ? 6 : ((p & 1) ? -4 : 1); }   // (U0 + U4) - 4 (U1 + U3) + 6 U2
+// a non-zero small integer as a double, without the FP64 pipe
+__device__ __forceinline__ double small_int(int i) { return widen_f32(__int2float_rn(i)); }
+// the derivative D-, D, D+ (position l = 0, 1, 2) of three node values (Sec. 2.1), times h
+__device__ __forceinline__ double node_diff(int l, double a, double b, double c) {
+  return l == 0 ? fma(4.0, b, fma(-3.0, a, -c)) : (l == 1 ? c - a : fma(-4.0, b, fma(3.0, c, a)));
+}
+// its transpose: what the derivatives da, db, dc at the three nodes give to the value at position l
+__device__ __forceinline__ double node_gather(int l, double da, double db, double dc) {
+  return l == 0 ? fma(-3.0, da, dc - db) : (l == 1 ? 4.0 * (da - dc) : fma(3.0, dc, db - da));
+}
 
 struct Vec4 {
   const double *p[4];
@@ -168,13 +181,13 @@ __device__ __forceinline__ void line_coefs(const AfDev &d, const AfGrid &g, cons
 #pragma unroll
   for (int p = 1; p < 5; ++p) {
     const double s = pval(d, g, P[p], qsr);
-    if (s > al) { al = s; am = p; }
+    if ((long long)bits(s) > (long long)bits(al)) { al = s; am = p; }   // non-negative
   }
   double ga = 0.0;
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
-    const double up = fma(6.0, uval(d, g, P[2], k),
-                          fma(-4.0, uval(d, g, P[1], k) + uval(d, g, P[3], k), uval(d, g, P[0], k) + uval(d, g, P[4], k)));
+    const double up = up5(uval(d, g, P[0], k), uval(d, g, P[1], k), uval(d, g, P[2], k), uval(d, g, P[3], k),
+                          uval(d, g, P[4], k));
     ga = fma(vval(v, g, CLS, i, j, k), up, ga);
   }
   const size_t PS = (size_t)g.nxa * g.nya, o = (size_t)j * g.nxa + i;
@@ -231,12 +244,8 @@ __device__ __forceinline__ void cell_terms(const AfDev &d, const AfGrid &g, cons
   for (int m = 0; m < 3; ++m)
 #pragma unroll
     for (int l = 0; l < 3; ++l) {
-      double dx1 = 0.0, dy2 = 0.0;
-#pragma unroll
-      for (int t = 0; t < 3; ++t) {
-        dx1 = fma(kD1[l][t], uval(d, g, N[t + 3 * m], 4), dx1);
-        dy2 = fma(kD1[m][t], uval(d, g, N[l + 3 * t], 5), dy2);
-      }
+      const double dx1 = node_diff(l, uval(d, g, N[3 * m], 4), uval(d, g, N[1 + 3 * m], 4), uval(d, g, N[2 + 3 * m], 4));
+      const double dy2 = node_diff(m, uval(d, g, N[l], 5), uval(d, g, N[l + 3], 5), uval(d, g, N[l + 6], 5));
       const double W = w1[l] * w1[m];
       const double div = fma(dx1, rdx, dy2 * rdy);
       double dd = 0.0;
@@ -252,7 +261,7 @@ __device__ __forceinline__ void cell_terms(const AfDev &d, const AfGrid &g, cons
 __global__ void __launch_bounds__(128) k_adj1(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                               const __grid_constant__ Vec4 v, double *a, const double *co) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
-  const double rdx = 1.0 / g.dx, rdy = 1.0 / g.dy;
+  const double rdx = g.rdx, rdy = g.rdy;
   switch (blockIdx.z) {
     case 0:
       if (i < g.ex[CC] && j < g.ey[CC]) {
@@ -324,27 +333,30 @@ __device__ __forceinline__ void gather_lines(const AfDev &d, const AfGrid &g, co
     if (!candidate(g, OC, DIR, q, o, s)) continue;
     PI P[5];
     fvs_line(g, OC, DIR, s.i, s.j, P);
-    double cf = 0.0, cu = 0.0, csr = 0.0;
-    int hits = 0;
+    int cf = 0, cu = 0, csr = 0, hits = 0;
     const int am = (int)aval(a, g, s.i, s.j, sal + 2);
 #pragma unroll
     for (int p = 0; p < 5; ++p)
       if (same(P[p], q)) {
-        cf += kCoefF[p];
-        cu += kCoefU[p];
-        if (p == am) csr += 1.0;
+        cf += coef_f(p);
+        cu += coef_u(p);
+        csr += p == am;
         ++hits;
       }
     if (!hits) continue;
     const double al = aval(a, g, s.i, s.j, sal);
-    if (csr != 0.0) acc.sr[DIR] = fma(csr, aval(a, g, s.i, s.j, sal + 1), acc.sr[DIR]);
-    acc.B[DIR] = fma(cf * c, aval(a, g, s.i, s.j, sdbb), acc.B[DIR]);
-    const double cual = cu * al;
+    if (csr) acc.sr[DIR] = fma(small_int(csr), aval(a, g, s.i, s.j, sal + 1), acc.sr[DIR]);
+    if (cf) {
+      const double cc = small_int(cf) * c;
+      acc.B[DIR] = fma(cc, aval(a, g, s.i, s.j, sdbb), acc.B[DIR]);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const double gk = -c * vval(v, g, OC, s.i, s.j, k);
-      if (k != 4 + DIR) acc.F[DIR][k] = fma(cf, gk, acc.F[DIR][k]);
-      acc.U[k] = fma(cual, gk, acc.U[k]);
+      for (int k = 0; k < 8; ++k)
+        if (k != 4 + DIR) acc.F[DIR][k] = fma(-cc, vval(v, g, OC, s.i, s.j, k), acc.F[DIR][k]);
+    }
+    if (cu) {
+      const double ca = small_int(cu) * (al * c);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) acc.U[k] = fma(-ca, vval(v, g, OC, s.i, s.j, k), acc.U[k]);
     }
   }
 }
@@ -362,13 +374,14 @@ __device__ __forceinline__ void gather_central(const AfGrid &g, const Vec4 &v, c
     if (!candidate(g, oc, DIR, q, o, s)) continue;
     PI lo = {CC, s.i, s.j}, hi = lo;
     if (DIR == 0) hi.i = mface(s.i + 1, g.nx, g.bc); else hi.j = mface(s.j + 1, g.ny, g.bc);
-    const double sgn = (same(hi, q) ? 1.0 : 0.0) - (same(lo, q) ? 1.0 : 0.0);
-    if (sgn == 0.0) continue;
+    const int sgn = (int)same(hi, q) - (int)same(lo, q);
+    if (sgn == 0) continue;
     // L -= (F(hi) - F(lo))/h, divB += (B(hi) - B(lo))/h
-    acc.B[DIR] = fma(sgn * rh, aval(a, g, s.i, s.j, sdbb), acc.B[DIR]);
+    const double w = sgn > 0 ? rh : neg_i(rh);
+    acc.B[DIR] = fma(w, aval(a, g, s.i, s.j, sdbb), acc.B[DIR]);
 #pragma unroll
     for (int k = 0; k < 8; ++k)
-      if (k != 4 + DIR) acc.F[DIR][k] = fma(-sgn * rh, vval(v, g, oc, s.i, s.j, k), acc.F[DIR][k]);
+      if (k != 4 + DIR) acc.F[DIR][k] = fma(-w, vval(v, g, oc, s.i, s.j, k), acc.F[DIR][k]);
   }
 }
 
@@ -378,23 +391,24 @@ __device__ __forceinline__ void gather_central(const AfGrid &g, const Vec4 &v, c
 template <int DIR>
 __device__ __forceinline__ void face_cot(const AfGrid &g, const Vec4 &v, int fi, int fj, double wgt, double rh,
                                          Acc &acc, const double *co) {
-  wgt *= wface(co, g, DIR, fi, fj);
+  if (co) wgt *= wface(co, g, DIR, fi, fj);
+  wgt *= rh;
 #pragma unroll
   for (int o = -1; o <= 0; ++o) {
     int ci = fi, cj = fj;
     if (DIR == 0) ci += o; else cj += o;
     if (g.bc == 0) { ci = wrapi(ci, g.nx); cj = wrapi(cj, g.ny); }
     if (ci < 0 || cj < 0 || ci >= g.nx || cj >= g.ny) continue;
-    double sgn = 0.0;
+    int sgn = 0;
     if (DIR == 0) {
-      if (ci == fi && cj == fj) sgn += 1.0;                                   // left face of the cell
-      if (mface(ci + 1, g.nx, g.bc) == fi && cj == fj) sgn -= 1.0;            // right face
+      sgn += ci == fi && cj == fj;                                   // left face of the cell
+      sgn -= mface(ci + 1, g.nx, g.bc) == fi && cj == fj;            // right face
     } else {
-      if (ci == fi && cj == fj) sgn += 1.0;
-      if (mface(cj + 1, g.ny, g.bc) == fj && ci == fi) sgn -= 1.0;
+      sgn += ci == fi && cj == fj;
+      sgn -= mface(cj + 1, g.ny, g.bc) == fj && ci == fi;
     }
-    if (sgn == 0.0) continue;
-    const double w = sgn * wgt * rh;
+    if (sgn == 0) continue;
+    const double w = sgn > 0 ? wgt : neg_i(wgt);
 #pragma unroll
     for (int k = 0; k < 8; ++k)
       if (k != 4 + DIR) acc.F[DIR][k] = fma(w, vval(v, g, 0, ci, cj, k), acc.F[DIR][k]);
@@ -413,13 +427,13 @@ __device__ __forceinline__ void gather_simpson(const AfGrid &g, const Vec4 &v, c
       PI s;
       if (candidate(g, CX, 1, q, o, s)) {
         const int hj = mface(s.j + 1, g.ny, g.bc);
-        const double wgt = (s.j == q.j ? 1.0 : 0.0) + (hj == q.j ? 1.0 : 0.0);
-        if (wgt != 0.0) face_cot<0>(g, v, s.i, s.j, wgt / 6.0, rdx, acc, co);
+        const int n = (s.j == q.j) + (hj == q.j);
+        if (n) face_cot<0>(g, v, s.i, s.j, n == 1 ? 1.0 / 6.0 : 2.0 / 6.0, rdx, acc, co);
       }
       if (candidate(g, CY, 0, q, o, s)) {
         const int hi = mface(s.i + 1, g.nx, g.bc);
-        const double wgt = (s.i == q.i ? 1.0 : 0.0) + (hi == q.i ? 1.0 : 0.0);
-        if (wgt != 0.0) face_cot<1>(g, v, s.i, s.j, wgt / 6.0, rdy, acc, co);
+        const int n = (s.i == q.i) + (hi == q.i);
+        if (n) face_cot<1>(g, v, s.i, s.j, n == 1 ? 1.0 / 6.0 : 2.0 / 6.0, rdy, acc, co);
       }
     }
   }
@@ -449,15 +463,15 @@ __device__ __forceinline__ void gather_source(const AfGrid &g, const Vec4 &v, co
         const int n = nodes[t];
         if (!same(N[n], q)) continue;
         const int l = n % 3, m = n / 3;
-        const double wd = aval(a, g, ci, cj, A_WD + n) * wcell(co, g, ci, cj);
+        double wd = aval(a, g, ci, cj, A_WD + n);
+        if (co) wd *= wcell(co, g, ci, cj);
 #pragma unroll
         for (int k = 1; k < 8; ++k) acc.ps[k] = fma(-wd, vval(v, g, 0, ci, cj, k), acc.ps[k]);
-        double s1 = 0.0, s2 = 0.0;
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {
-          s1 = fma(aval(a, g, ci, cj, A_DIVB + r + 3 * m), kD1[r][l], s1);   // d/dx at node (r, m) uses node (l, m)
-          s2 = fma(aval(a, g, ci, cj, A_DIVB + l + 3 * r), kD1[r][m], s2);   // d/dy at node (l, r) uses node (l, m)
-        }
+        // d/dx at the nodes (r, m) and d/dy at the nodes (l, r) use node (l, m)
+        const double s1 = node_gather(l, aval(a, g, ci, cj, A_DIVB + 3 * m), aval(a, g, ci, cj, A_DIVB + 1 + 3 * m),
+                                      aval(a, g, ci, cj, A_DIVB + 2 + 3 * m));
+        const double s2 = node_gather(m, aval(a, g, ci, cj, A_DIVB + l), aval(a, g, ci, cj, A_DIVB + l + 3),
+                                      aval(a, g, ci, cj, A_DIVB + l + 6));
         acc.B[0] = fma(s1, rdx, acc.B[0]);
         acc.B[1] = fma(s2, rdy, acc.B[1]);
       }
@@ -608,7 +622,7 @@ __global__ void AF_LB_ADJ2 k_adj2(const __grid_constant__ AfDev d, const __grid_
                                               const __grid_constant__ Vec4 v, const double *a,
                                               const __grid_constant__ OVec4 tp, double *zc, const double *co) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
-  const double rdx = 1.0 / g.dx, rdy = 1.0 / g.dy;
+  const double rdx = g.rdx, rdy = g.rdy;
   switch (blockIdx.z) {
     case 0: adj_point<CX>(d, g, v, a, i, j, rdx, rdy, tp.p, zc, co); break;
     case 1: adj_point<CY>(d, g, v, a, i, j, rdx, rdy, tp.p, zc, co); break;
@@ -653,15 +667,16 @@ __device__ __forceinline__ void adj_final(const AfGrid &g, const double *zc, con
         if (ci < 0 || cj < 0 || ci >= g.nx || cj >= g.ny) continue;
         PI N[9];
         cell_nodes(g, ci, cj, N);
-        double wgt = 0.0;
+        int w16 = 0;   // weight in sixteenths
 #pragma unroll
         for (int n = 0; n < 9; ++n)
-          if (n != 4 && same(N[n], q)) wgt += (n == 1 || n == 3 || n == 5 || n == 7) ? -0.25 : -0.0625;
-        if (wgt == 0.0) continue;
+          if (n != 4 && same(N[n], q)) w16 += (n == 1 || n == 3 || n == 5 || n == 7) ? -4 : -1;
+        if (w16 == 0) continue;
+        const double wgt = ldexp_i<-4>(small_int(w16));
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-          const double m = co ? mweight(co, g, AFC_C1, ci, cj, k) : 1.0;
-          T[k] = fma(wgt * m, __ldg(zc + k * PS + (size_t)cj * g.nxa + ci), T[k]);
+          const double w = co ? wgt * mweight(co, g, AFC_C1, ci, cj, k) : wgt;
+          T[k] = fma(w, __ldg(zc + k * PS + (size_t)cj * g.nxa + ci), T[k]);
         }
       }
   }
@@ -705,14 +720,17 @@ __global__ void __launch_bounds__(128) k_adj0(const __grid_constant__ AfGrid g, 
   for (int k = 0; k < 8; ++k) vp.p[c][k * cs + oo] = mweight(co, g, s1, i, j, k) * __ldg(v.p[c] + k * cs + oo);
 }
 
-// What alpha^LLF along direction l and Psi need of one state
+// What alpha^LLF along direction l (2: both) and Psi need of one state
 struct LS {
-  double U[8], v[3], B[3], vB, cf, srho;
+  double U[8], v[3], B[3], vB, cf[2], srho;
 };
-__device__ __forceinline__ void lstate(const AfDev &d, const AfGrid &g, int c, int i, int j, int l, LS &s) {
+__device__ __forceinline__ void load_state(const AfDev &d, const AfGrid &g, int c, int i, int j, double *U) {
   const size_t cs = (size_t)g.ex[c] * g.ey[c], oo = (size_t)j * g.ex[c] + i;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) s.U[k] = __ldg(d.us[c] + k * cs + oo);
+  for (int k = 0; k < 8; ++k) U[k] = __ldg(d.us[c] + k * cs + oo);
+}
+__device__ __forceinline__ void lstate(const AfDev &d, const AfGrid &g, int c, int i, int j, int l, LS &s) {
+  load_state(d, g, c, i, j, s.U);
   const double rho = s.U[0], r = rcp(rho);
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
@@ -724,9 +742,13 @@ __device__ __forceinline__ void lstate(const AfDev &d, const AfGrid &g, int c, i
   const double mv = fma(s.U[1], s.v[0], fma(s.U[2], s.v[1], s.U[3] * s.v[2]));
   const double p = g.gm1 * fma(-0.5, mv + BB, s.U[7]);
   const double c2 = g.gamma * p * r, a = fma(BB, r, c2);
-  double dd = fma(-4.0 * (c2 * r), s.B[l] * s.B[l], a * a);
-  dd = dd > 0.0 ? dd : 0.0;
-  s.cf = dsqrt(fma(0.5, dsqrt(dd), 0.5 * a));
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    if (l != q && l != 2) continue;
+    double dd = fma(-4.0 * (c2 * r), s.B[q] * s.B[q], a * a);
+    dd = gt_zero(dd) ? dd : 0.0;
+    s.cf[q] = dsqrt(fma(0.5, dsqrt(dd), 0.5 * a));
+  }
   s.srho = dsqrt(rho);
 }
 
@@ -739,7 +761,8 @@ __device__ __forceinline__ void llf_vjp(int l, int which, const LS &a, const LS 
   const double va = absd(a.v[l]), vb = absd(b.v[l]);
   const double d0 = a.B[0] - b.B[0], d1 = a.B[1] - b.B[1], d2 = a.B[2] - b.B[2];
   const double n = dsqrt(fma(d0, d0, fma(d1, d1, d2 * d2))), den = a.srho + b.srho;
-  const double al = fmax(va, vb) + fmax(a.cf, b.cf) + n / den;
+  const double nd = ddiv(n, den);
+  const double al = maxnn(va, vb) + maxnn(a.cf[l], b.cf[l]) + nd;
   double T = 0.0;
 #pragma unroll
   for (int k = 0; k < 8; ++k) T = fma(c[k], b.U[k] - a.U[k], T);
@@ -750,13 +773,13 @@ __device__ __forceinline__ void llf_vjp(int l, int which, const LS &a, const LS 
     acc.U[k] = fma(sal, c[k], acc.U[k]);
   }
   if (which == 0 ? va >= vb : vb > va) acc.av[l] += h;
-  if (which == 0 ? a.cf >= b.cf : b.cf > a.cf) acc.cf[l] += h;
-  if (n > 0.0) {
-    const double sb = (which == 0 ? h : -h) / (n * den);
+  if (which == 0 ? a.cf[l] >= b.cf[l] : b.cf[l] > a.cf[l]) acc.cf[l] += h;
+  if (gt_zero(n)) {
+    const double sb = ddiv(which == 0 ? h : neg_i(h), n * den);
     acc.U[4] = fma(sb, d0, acc.U[4]);
     acc.U[5] = fma(sb, d1, acc.U[5]);
     acc.U[6] = fma(sb, d2, acc.U[6]);
-    acc.srho -= h * n / (den * den);
+    acc.srho -= ddiv(h * nd, den);
   }
 }
 
@@ -823,16 +846,18 @@ __device__ __forceinline__ void adj_llf(const AfDev &d, const AfGrid &g, const V
   if constexpr (C == 0) {
     if (i >= g.nx || j >= g.ny) return;
     // face fluxes F^LLF of the cell's four faces (weight 1 - w_f)
+    bool have = false;   // the cell's own state, formed at its first use
 #pragma unroll
     for (int dir = 0; dir < 2; ++dir) {
       const int n = dir ? g.ny : g.nx, io = dir ? j : i;
       const double rh = dir ? rdy : rdx;
-      lstate(d, g, 0, i, j, dir, me);
 #pragma unroll
       for (int side = 0; side < 2; ++side) {
         const int f = io + side, fs = mface(f, n, g.bc);
         const double w = wface(co, g, dir, dir ? i : fs, dir ? fs : j);
         if (w == 1.0) continue;
+        if (!have) lstate(d, g, 0, i, j, 2, me);
+        have = true;
         double cv[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) cv[k] = 0.0;
@@ -895,8 +920,9 @@ __device__ __forceinline__ void adj_llf(const AfDev &d, const AfGrid &g, const V
     const size_t cs = (size_t)g.nx * g.ny, oo = (size_t)j * g.nx + i;
     double o[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     if (touched) {
-      lstate(d, g, 0, i, j, 0, me);
-      pointwise_transpose(me.U, g, acc, o);
+      double U[8];
+      load_state(d, g, 0, i, j, U);
+      pointwise_transpose(U, g, acc, o);
     }
 #pragma unroll
     for (int k = 0; k < 8; ++k) tp[0][k * cs + oo] = o[k];
@@ -906,7 +932,10 @@ __device__ __forceinline__ void adj_llf(const AfDev &d, const AfGrid &g, const V
     double gq[8];
     PI nb[4];
     // its own LLF state: -(F1(q, xr) - F1(xl, q))/dx - (F2(q, yr) - F2(yl, q))/dy - div B Psi(q)
+    bool have = false;   // the point's own state, formed at its first use
     if (llf_cot(g, v, co, q, gq)) {
+      lstate(d, g, C, i, j, 2, me);
+      have = true;
       llf_nbrs(g, C, i, j, nb);
       double cp[8], cm[8];
 #pragma unroll
@@ -917,7 +946,6 @@ __device__ __forceinline__ void adj_llf(const AfDev &d, const AfGrid &g, const V
           cp[k] = rh * gq[k];
           cm[k] = -rh * gq[k];
         }
-        lstate(d, g, C, i, j, l, me);
         lstate(d, g, nb[2 * l].c, nb[2 * l].i, nb[2 * l].j, l, ot);
         llf_vjp(l, 1, ot, me, cp, acc);
         lstate(d, g, nb[2 * l + 1].c, nb[2 * l + 1].i, nb[2 * l + 1].j, l, ot);
@@ -944,7 +972,8 @@ __device__ __forceinline__ void adj_llf(const AfDev &d, const AfGrid &g, const V
         const int l = r >> 1;
         const double rh = l ? rdy : rdx;
         double cv[8];
-        lstate(d, g, C, i, j, l, me);
+        if (!have) lstate(d, g, C, i, j, 2, me);
+        have = true;
         lstate(d, g, p.c, p.i, p.j, l, ot);
         if (r & 1) {   // q is the right/high neighbour: flux F(p, q), cotangent -g_p/h
 #pragma unroll
