@@ -132,6 +132,12 @@ void build_tables(af_batch *b) {
         d.lim1 = w; w += 8 * PS;
         d.thx = w; w += PS;
         d.thy = w; w += PS;
+        d.pq_cap = (int)(3 * PS);
+        d.cq_cap = (int)PS;
+        d.pqu = w; w += 24 * PS;
+        d.cqe = w; w += 2 * PS;
+        d.pq = reinterpret_cast<int *>(w); w += (3 * PS + 1) / 2;
+        d.cq = reinterpret_cast<int *>(w); w += (PS + 1) / 2;
         d.sc = b->sc + r;
         d.st = b->st + r;
       }
@@ -199,6 +205,7 @@ void batch_stage(af_batch *b, int s, int with_dt, int bps_cap) {
   launch_pass(b, AF_K_POINTS, tab, RK_A[s], RK_B[s], any_upwind(b), bps_cap);
   launch_pass(b, AF_K_FACES, tab, RK_A[s], RK_B[s], 0, bps_cap);
   launch_pass(b, AF_K_CELLS, tab, RK_A[s], RK_B[s], 0, bps_cap);
+  af_launch_batch(AF_K_CELLS_SLOW, tab, b->nruns, b->items, b->nitems, b->block, 1, RK_A[s], RK_B[s], 0, b->stream);
   launch_pass(b, AF_K_FINAL, tab, RK_A[s], RK_B[s], 0, bps_cap);
   af_launch_batch(AF_K_REPAIR, tab, b->nruns, b->items, b->nitems, b->block, 1, RK_A[s], RK_B[s], 0, b->stream);
 }
@@ -246,7 +253,9 @@ int af_batch_create(int nruns, const int *nx, const int *ny, const double *gamma
   b->state_off.resize(nruns);
   b->work_off.resize(nruns);
   size_t st = 0, wk = 0;
-  const size_t per_point = AF_NQA + 4 * AF_NQP + 8 + 4 + 2 * AF_NQF + 4 + 8 + 2;
+  // stage work arrays, then the limiter work lists (points: 8 doubles and an int each, three classes;
+  // cells: 2 doubles and an int)
+  const size_t per_point = AF_NQA + 4 * AF_NQP + 8 + 4 + 2 * AF_NQF + 4 + 8 + 2 + 24 + 2 + 2;
   for (int r = 0; r < nruns; ++r) {
     fill_grid(b, r);
     const AfGrid &g = b->grid[r];
@@ -258,7 +267,7 @@ int af_batch_create(int nruns, const int *nx, const int *ny, const double *gamma
     }
     st += (off + 31) / 32 * 32;   // keep every run 256-byte aligned
     b->work_off[r] = wk;
-    wk += ((size_t)g.nxa * g.nya * per_point + 31) / 32 * 32;
+    wk += ((size_t)g.nxa * g.nya * per_point + 1 + 31) / 32 * 32;
   }
   b->state_total = st;
   int rc = AF_OK;

@@ -39,6 +39,10 @@ namespace {
 #ifndef AF_KBCL
 #define AF_KBCL 2
 #endif
+// Batches hand limited points and cells to work lists of their own runs, as single runs do: with
+// the slow paths inline the point pass spilled 2.2 kB a thread (kBatchListBlocks blocks walk the
+// lists of each run).
+constexpr int kBatchListBlocks = 8;
 // the nz parts of the work of a tile (DoF classes, face directions) are items of their own, one part
 // after the other over all tiles
 #define AF_BATCH_LOOP(nz, call)                                   \
@@ -61,7 +65,7 @@ __global__ void kb_dt(const AfRun *__restrict__ runs, int nruns) {
 template <bool UP>
 __global__ void __launch_bounds__(256, AF_KBPT) kb_points(const AfRun *__restrict__ runs, const int4 *__restrict__ items,
                                                  int nitems, double a, double b) {
-  AF_BATCH_LOOP(4, (b_points<false, UP, kStage>(r->d, r->g, i, j, a, b, 0, z)));
+  AF_BATCH_LOOP(4, (b_points<false, UP, kPlain>(r->d, r->g, i, j, a, b, 0, z)));
 }
 __global__ void __launch_bounds__(256) kb_faces(const AfRun *__restrict__ runs, const int4 *__restrict__ items,
                                                 int nitems) {
@@ -69,7 +73,7 @@ __global__ void __launch_bounds__(256) kb_faces(const AfRun *__restrict__ runs, 
 }
 __global__ void __launch_bounds__(256, AF_KBCL) kb_cells(const AfRun *__restrict__ runs, const int4 *__restrict__ items,
                                                 int nitems, double a, double b) {
-  AF_BATCH_LOOP(1, (b_cells<false, false>(r->d, r->g, i, j, a, b, 0)));
+  AF_BATCH_LOOP(1, (b_cells<false, true, true>(r->d, r->g, i, j, a, b, 0)));
 }
 __global__ void __launch_bounds__(256) kb_final(const AfRun *__restrict__ runs, const int4 *__restrict__ items,
                                                 int nitems, double a, double b) {
@@ -77,7 +81,16 @@ __global__ void __launch_bounds__(256) kb_final(const AfRun *__restrict__ runs, 
 }
 __global__ void kb_repair(const AfRun *__restrict__ runs, int nruns, double a, double b) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < nruns && runs[t].g.pp_on) b_repair(runs[t].d, runs[t].g, a, b);
+  if (t >= nruns) return;
+  if (runs[t].g.pp_on) b_repair(runs[t].d, runs[t].g, a, b);
+  runs[t].d.st->npq = runs[t].d.st->ncq = 0;   // the next stage's work lists start empty
+}
+// the work lists of the runs, blockIdx.y the run: its cells, then its points
+__global__ void __launch_bounds__(kListThreads) kb_lists(const AfRun *__restrict__ runs, double a, double b) {
+  const AfRun *r = runs + blockIdx.y;
+  if (!r->g.pp_on) return;
+  b_cells_lists(r->d, r->g, blockIdx.x, gridDim.x);
+  b_points_slow<false>(r->d, r->g, a, b, blockIdx.x, gridDim.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -381,6 +394,10 @@ void af_launch_batch(int pass, const AfRun *runs, int nruns, const int4 *items, 
     case AF_K_FACES: kb_faces<<<nblocks, block, 0, s>>>(runs, items, nitems); break;
     case AF_K_CELLS: kb_cells<<<nblocks, block, 0, s>>>(runs, items, nitems, a, b); break;
     case AF_K_FINAL: kb_final<<<nblocks, block, 0, s>>>(runs, items, nitems, a, b); break;
+    case AF_K_CELLS_SLOW:
+      for (int r0 = 0; r0 < nruns; r0 += 65535)   // blockIdx.y
+        kb_lists<<<dim3(kBatchListBlocks, nruns - r0 < 65535 ? nruns - r0 : 65535), kListThreads, 0, s>>>(runs + r0, a, b);
+      break;
     case AF_K_REPAIR: kb_repair<<<(nruns + 127) / 128, 128, 0, s>>>(runs, nruns, a, b); break;
     default: break;
   }

@@ -13,18 +13,20 @@ namespace {
 // ---------------------------------------------------------------------------
 // indexing helpers: af_device.cuh
 
+// lane of the thread in its warp (tiles may be narrower than a warp)
+__device__ __forceinline__ int lane_id() { return (int)(threadIdx.y * blockDim.x + threadIdx.x) & 31; }
 // warp-aggregated event counters
 __device__ __forceinline__ void count(AfStatus *st, int slot, bool pred) {
   unsigned act = __activemask();
   unsigned m = __ballot_sync(act, pred);
-  if (m && (threadIdx.x & 31) == (__ffs(act) - 1)) atomicAdd(&st->cnt[slot], (unsigned long long)__popc(m));
+  if (m && lane_id() == __ffs(act) - 1) atomicAdd(&st->cnt[slot], (unsigned long long)__popc(m));
 }
 
 // Slot of this thread in a work list (warp-aggregated; every active thread enqueues
 // one entry), or -1 with the overflow bit set when the list is full.
 __device__ __forceinline__ int enqueue(AfStatus *st, int *counter, int cap) {
   const unsigned act = __activemask();
-  const int lane = threadIdx.x & 31, leader = __ffs(act) - 1;
+  const int lane = lane_id(), leader = __ffs(act) - 1;
   int base = 0;
   if (lane == leader) base = atomicAdd(counter, __popc(act));
   base = __shfl_sync(act, base, leader);
@@ -1096,7 +1098,7 @@ __device__ __forceinline__ void b_faces(const AfDev &d, const AfGrid &g, const i
   if (sens && !is_zero(g.kappa)) {
     const unsigned act = __activemask();
     const int tot = __reduce_add_sync(act, nsens);
-    if (tot && (threadIdx.x & 31) == (__ffs(act) - 1)) atomicAdd(&d.st->cnt[ST_SENSOR_LT099], (unsigned long long)tot);
+    if (tot && lane_id() == __ffs(act) - 1) atomicAdd(&d.st->cnt[ST_SENSOR_LT099], (unsigned long long)tot);
   }
 }
 
@@ -1316,8 +1318,8 @@ __device__ __forceinline__ void cell_H(const AfDev &d, const AfGrid &g, int i, i
   }
 }
 
-// PL: as in the point pass, with the positivity limiters on
-template <bool GB, bool PL>
+// PL: as in the point pass, with the positivity limiters on (ANY: on or off, by run)
+template <bool GB, bool PL, bool ANY = false>
 __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const int i, const int j, double a, double b,
                                         int mode) {
   const size_t PS = (size_t)g.nxa * g.nya;
@@ -1446,7 +1448,7 @@ __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const i
       // theta^s_ij = min over the four faces
       const double tsL = FX(i, j, QF_TS), tsR = FX(ip, j, QF_TS), tsD = FY(i, j, QF_TS), tsU = FY(i, jp, QF_TS);
       const double tsc = minnn(minnn(tsL, tsR), minnn(tsD, tsU));
-      if (!PL && !g.pp_on) {
+      if ((!PL || ANY) && !g.pp_on) {
         // sensor-blended high-order update: F^ss = F^LLF + G, S^ss = S^LLF + theta^s (S - S^LLF)
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
