@@ -90,60 +90,61 @@ EXEC_FP64_DIVB = {}
 # count them per cell-stage, as the DMUL and DADD counts of the same captures on the
 # build that ran every product on the FP64 pipe (kernel digest e1110cc7...) minus those
 # of the build that first moved them (before the FP32 certificates, which remove FP64
-# work outright): a lower bound, since later changes moved a few more operations.  The literal count of the paper's formulas (ALGO_FLOPS) is larger where a
+# work outright): a lower bound, since later changes moved a few more operations; int_add of
+# k_points: the FP64 flops of its line sums before they became fixed-point sums.  The literal count of the paper's formulas (ALGO_FLOPS) is larger where a
 # kernel uses a cheaper algebraic form (the LLF-FVS line as one expression, products
 # by 1/h), so it is reported beside the roofline, never divided by the peak.  Each
 # table names the capture it comes from and a digest of the kernel sources it was
 # taken on: once the kernels change, the line says so ("counts_stale") until the
 # capture is retaken.  The work-list kernels of the limiter slow paths are summed as
-# k_points_slow and k_cells_slow (the box and the Newton pass), the names af_timing
+# k_points_slow and k_cells_slow, the names af_timing
 # reports them under.
 EXEC_FP64 = {
-    "blast_low_beta": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "7013560c17a537ed1abec9766d30c1192bfdcd19", "kernels": {
-        "k_pointdata": {"dadd": 93.04, "dmul": 0.01, "dfma": 183.15, "pipe": 276.19, "dram_bytes": 1119.0, "int_mul": 124.09, "int_add": 0.00},
-        "k_points": {"dadd": 155.22, "dmul": 8.01, "dfma": 222.38, "pipe": 385.60, "dram_bytes": 1946.1, "int_mul": 40.06, "int_add": 0.00},
-        "k_points_slow": {"dadd": 0.14, "dmul": 0.19, "dfma": 0.39, "pipe": 0.74, "dram_bytes": 1.9, "int_mul": 0.02, "int_add": 0.00},
-        "k_faces": {"dadd": 74.11, "dmul": 5.95, "dfma": 52.36, "pipe": 134.39, "dram_bytes": 744.0, "int_mul": 44.08, "int_add": 0.00},
-        "k_cells": {"dadd": 58.01, "dmul": 3.00, "dfma": 122.02, "pipe": 183.03, "dram_bytes": 1224.2, "int_mul": 51.00, "int_add": 0.00},
-        "k_cells_slow": {"dadd": 0.06, "dmul": 0.18, "dfma": 0.20, "pipe": 0.54, "dram_bytes": 0.8, "int_mul": 0.00, "int_add": 0.00},
+    "blast_low_beta": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "1a570010dcdba859bc3ba306e21a4c24882b893e", "kernels": {
+        "k_pointdata": {"dadd": 98.04, "dmul": 0.01, "dfma": 188.15, "pipe": 286.20, "dram_bytes": 1383.8, "int_mul": 124.09, "int_add": 0.00},
+        "k_points": {"dadd": 95.13, "dmul": 6.01, "dfma": 160.29, "pipe": 261.42, "dram_bytes": 1618.9, "int_mul": 40.06, "int_add": 184.28},
+        "k_points_slow": {"dadd": 0.18, "dmul": 0.29, "dfma": 0.49, "pipe": 1.00, "dram_bytes": 1.9, "int_mul": 0.02, "int_add": 0.00},
+        "k_faces": {"dadd": 74.11, "dmul": 5.95, "dfma": 52.36, "pipe": 134.39, "dram_bytes": 823.4, "int_mul": 44.08, "int_add": 0.00},
+        "k_cells": {"dadd": 59.01, "dmul": 4.00, "dfma": 121.02, "pipe": 184.03, "dram_bytes": 793.4, "int_mul": 51.00, "int_add": 0.00},
+        "k_cells_slow": {"dadd": 0.07, "dmul": 0.19, "dfma": 0.19, "pipe": 0.55, "dram_bytes": 0.7, "int_mul": 0.00, "int_add": 0.00},
         "k_final": {"dadd": 0.00, "dmul": 0.00, "dfma": 21.33, "pipe": 21.33, "dram_bytes": 329.5, "int_mul": 8.33, "int_add": 16.00},
     }},
-    "orszag_tang": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "7013560c17a537ed1abec9766d30c1192bfdcd19", "kernels": {
-        "k_pointdata": {"dadd": 93.00, "dmul": 0.00, "dfma": 183.00, "pipe": 276.00, "dram_bytes": 948.2, "int_mul": 124.00, "int_add": 0.00},
-        "k_points": {"dadd": 156.00, "dmul": 8.00, "dfma": 228.00, "pipe": 392.00, "dram_bytes": 1803.4, "int_mul": 42.00, "int_add": 0.00},
-        "k_points_slow": {"dadd": 0.00, "dmul": 0.00, "dfma": 0.00, "pipe": 0.00, "dram_bytes": 0.2, "int_mul": 0.00, "int_add": 0.00},
-        "k_faces": {"dadd": 74.00, "dmul": 0.00, "dfma": 74.00, "pipe": 148.00, "dram_bytes": 637.8, "int_mul": 46.00, "int_add": 0.00},
-        "k_cells": {"dadd": 58.00, "dmul": 3.00, "dfma": 122.00, "pipe": 183.00, "dram_bytes": 1073.7, "int_mul": 51.00, "int_add": 0.00},
+    "orszag_tang": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "1a570010dcdba859bc3ba306e21a4c24882b893e", "kernels": {
+        "k_pointdata": {"dadd": 98.00, "dmul": 0.00, "dfma": 188.00, "pipe": 286.00, "dram_bytes": 1206.4, "int_mul": 124.00, "int_add": 0.00},
+        "k_points": {"dadd": 96.00, "dmul": 6.00, "dfma": 166.00, "pipe": 268.00, "dram_bytes": 1564.1, "int_mul": 42.00, "int_add": 184.00},
+        "k_points_slow": {"dadd": 0.00, "dmul": 0.00, "dfma": 0.00, "pipe": 0.00, "dram_bytes": 0.3, "int_mul": 0.00, "int_add": 0.00},
+        "k_faces": {"dadd": 74.00, "dmul": 0.00, "dfma": 74.00, "pipe": 148.00, "dram_bytes": 703.5, "int_mul": 46.00, "int_add": 0.00},
+        "k_cells": {"dadd": 59.00, "dmul": 4.00, "dfma": 121.00, "pipe": 184.00, "dram_bytes": 727.4, "int_mul": 51.00, "int_add": 0.00},
         "k_cells_slow": {"dadd": 0.00, "dmul": 0.00, "dfma": 0.00, "pipe": 0.00, "dram_bytes": 0.3, "int_mul": 0.00, "int_add": 0.00},
-        "k_final": {"dadd": 0.00, "dmul": 0.00, "dfma": 21.33, "pipe": 21.33, "dram_bytes": 277.4, "int_mul": 8.33, "int_add": 16.00},
+        "k_final": {"dadd": 0.00, "dmul": 0.00, "dfma": 21.33, "pipe": 21.33, "dram_bytes": 277.7, "int_mul": 8.33, "int_add": 16.00},
     }},
-    "jets": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "7013560c17a537ed1abec9766d30c1192bfdcd19", "kernels": {
-        "k_pointdata": {"dadd": 93.05, "dmul": 0.00, "dfma": 183.17, "pipe": 276.21, "dram_bytes": 1098.4, "int_mul": 124.13, "int_add": 0.00},
-        "k_points": {"dadd": 189.44, "dmul": 8.27, "dfma": 222.40, "pipe": 420.13, "dram_bytes": 2399.5, "int_mul": 39.14, "int_add": 0.00},
-        "k_points_slow": {"dadd": 0.02, "dmul": 0.02, "dfma": 0.05, "pipe": 0.10, "dram_bytes": 0.2, "int_mul": 0.00, "int_add": 0.00},
-        "k_faces": {"dadd": 83.13, "dmul": 6.02, "dfma": 52.13, "pipe": 143.30, "dram_bytes": 723.8, "int_mul": 44.08, "int_add": 0.00},
-        "k_cells": {"dadd": 58.52, "dmul": 3.00, "dfma": 122.01, "pipe": 183.54, "dram_bytes": 1212.2, "int_mul": 51.00, "int_add": 0.00},
-        "k_cells_slow": {"dadd": 0.03, "dmul": 0.09, "dfma": 0.10, "pipe": 0.27, "dram_bytes": 0.2, "int_mul": 0.00, "int_add": 0.00},
-        "k_final": {"dadd": 0.00, "dmul": 0.00, "dfma": 21.33, "pipe": 21.33, "dram_bytes": 322.2, "int_mul": 8.33, "int_add": 16.00},
+    "jets": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "1a570010dcdba859bc3ba306e21a4c24882b893e", "kernels": {
+        "k_pointdata": {"dadd": 98.05, "dmul": 0.00, "dfma": 188.18, "pipe": 286.22, "dram_bytes": 1366.0, "int_mul": 124.13, "int_add": 0.00},
+        "k_points": {"dadd": 101.04, "dmul": 6.10, "dfma": 160.23, "pipe": 267.38, "dram_bytes": 1729.8, "int_mul": 39.14, "int_add": 212.74},
+        "k_points_slow": {"dadd": 0.03, "dmul": 0.04, "dfma": 0.06, "pipe": 0.13, "dram_bytes": 0.2, "int_mul": 0.00, "int_add": 0.00},
+        "k_faces": {"dadd": 75.74, "dmul": 6.03, "dfma": 52.12, "pipe": 135.91, "dram_bytes": 837.1, "int_mul": 44.08, "int_add": 0.00},
+        "k_cells": {"dadd": 59.09, "dmul": 4.00, "dfma": 121.01, "pipe": 184.09, "dram_bytes": 850.2, "int_mul": 51.00, "int_add": 0.00},
+        "k_cells_slow": {"dadd": 0.03, "dmul": 0.09, "dfma": 0.10, "pipe": 0.27, "dram_bytes": 0.1, "int_mul": 0.00, "int_add": 0.00},
+        "k_final": {"dadd": 0.00, "dmul": 0.00, "dfma": 21.33, "pipe": 21.33, "dram_bytes": 322.1, "int_mul": 8.33, "int_add": 16.00},
     }},
-    "rarefaction_lattice": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "7013560c17a537ed1abec9766d30c1192bfdcd19", "kernels": {
-        "k_pointdata": {"dadd": 93.50, "dmul": 1.87, "dfma": 187.23, "pipe": 283.05, "dram_bytes": 942.7, "int_mul": 124.00, "int_add": 0.00},
-        "k_points": {"dadd": 156.00, "dmul": 8.00, "dfma": 228.80, "pipe": 392.77, "dram_bytes": 1865.1, "int_mul": 39.81, "int_add": 0.00},
-        "k_points_slow": {"dadd": 49.23, "dmul": 68.69, "dfma": 141.61, "pipe": 271.05, "dram_bytes": 529.2, "int_mul": 6.84, "int_add": 0.00},
-        "k_faces": {"dadd": 74.00, "dmul": 0.57, "dfma": 75.13, "pipe": 149.66, "dram_bytes": 637.8, "int_mul": 46.00, "int_add": 0.00},
-        "k_cells": {"dadd": 64.34, "dmul": 4.36, "dfma": 136.73, "pipe": 206.08, "dram_bytes": 1092.5, "int_mul": 51.00, "int_add": 0.00},
-        "k_cells_slow": {"dadd": 44.31, "dmul": 54.71, "dfma": 233.66, "pipe": 347.47, "dram_bytes": 321.6, "int_mul": 0.00, "int_add": 0.00},
-        "k_final": {"dadd": 0.00, "dmul": 2.86, "dfma": 24.20, "pipe": 27.05, "dram_bytes": 277.8, "int_mul": 8.33, "int_add": 13.14},
+    "rarefaction_lattice": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "1a570010dcdba859bc3ba306e21a4c24882b893e", "kernels": {
+        "k_pointdata": {"dadd": 98.99, "dmul": 2.36, "dfma": 191.73, "pipe": 293.55, "dram_bytes": 1204.2, "int_mul": 124.00, "int_add": 0.00},
+        "k_points": {"dadd": 96.00, "dmul": 6.00, "dfma": 166.80, "pipe": 268.77, "dram_bytes": 1617.8, "int_mul": 39.81, "int_add": 183.99},
+        "k_points_slow": {"dadd": 58.64, "dmul": 78.11, "dfma": 132.19, "pipe": 280.47, "dram_bytes": 546.7, "int_mul": 6.84, "int_add": 0.00},
+        "k_faces": {"dadd": 74.00, "dmul": 0.57, "dfma": 75.13, "pipe": 149.67, "dram_bytes": 703.7, "int_mul": 46.00, "int_add": 0.00},
+        "k_cells": {"dadd": 66.25, "dmul": 6.27, "dfma": 134.82, "pipe": 207.98, "dram_bytes": 734.2, "int_mul": 51.00, "int_add": 0.00},
+        "k_cells_slow": {"dadd": 51.57, "dmul": 61.52, "dfma": 226.48, "pipe": 354.38, "dram_bytes": 206.3, "int_mul": 0.00, "int_add": 0.00},
+        "k_final": {"dadd": 0.00, "dmul": 2.86, "dfma": 24.20, "pipe": 27.05, "dram_bytes": 277.7, "int_mul": 8.33, "int_add": 13.14},
     }},
-    "blast1d": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "8915d37b6cf721a281ba9d891fc8e24ab5bd1867", "kernels": {
-        "k1_pointdata": {"dadd": 31.00, "dmul": 8.00, "dfma": 106.00, "pipe": 145.00, "dram_bytes": 667.8, "int_mul": 76.00, "int_add": 0.00},
-        "k1_points": {"dadd": 41.00, "dmul": 9.33, "dfma": 55.33, "pipe": 107.67, "dram_bytes": 430.6, "int_mul": 9.00, "int_add": 0.00},
-        "k1_faces": {"dadd": 30.00, "dmul": 20.00, "dfma": 19.00, "pipe": 72.00, "dram_bytes": 358.9, "int_mul": 4.00, "int_add": 0.00},
-        "k1_cells": {"dadd": 9.00, "dmul": 19.00, "dfma": 8.00, "pipe": 37.00, "dram_bytes": 289.9, "int_mul": 10.00, "int_add": 0.00},
-        "k1_final": {"dadd": 0.00, "dmul": 14.33, "dfma": 28.33, "pipe": 45.67, "dram_bytes": 252.5, "int_mul": 3.00, "int_add": 0.00},
+    "blast1d": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "472deb0f4847642bfe445c15c516cdc6c4f11431", "kernels": {
+        "k1_pointdata": {"dadd": 0.69, "dmul": 0.01, "dfma": 2.75, "pipe": 3.45, "dram_bytes": 21.6, "int_mul": 0.00, "int_add": 0.00},
+        "k1_points": {"dadd": 0.01, "dmul": 0.00, "dfma": 5.35, "pipe": 5.36, "dram_bytes": 162.9, "int_mul": 0.00, "int_add": 0.00},
+        "k1_faces": {"dadd": 0.02, "dmul": 0.01, "dfma": 0.01, "pipe": 0.04, "dram_bytes": 0.2, "int_mul": 0.00, "int_add": 0.00},
+        "k1_cells": {"dadd": 0.00, "dmul": 0.04, "dfma": 0.00, "pipe": 0.32, "dram_bytes": 32.9, "int_mul": 0.00, "int_add": 0.00},
+        "k1_final": {"dadd": 0.00, "dmul": 0.00, "dfma": 5.34, "pipe": 5.35, "dram_bytes": 162.4, "int_mul": 0.00, "int_add": 0.00},
     }},
 }
-EXEC_FP64_DIVB["blast_low_beta"] = {"source": "profiles/divb_blast512.md", "digest": "7013560c17a537ed1abec9766d30c1192bfdcd19",
+EXEC_FP64_DIVB["blast_low_beta"] = {"source": "profiles/divb_blast512.md", "digest": "1a570010dcdba859bc3ba306e21a4c24882b893e",
                                      "dadd": 67.99, "dmul": 19.01, "dfma": 57.03, "pipe": 143.98}
 # FP64 roofline from unit counts and clock: the GB300 SM retires 2 DFMA thread
 # instructions per cycle (ncu: sm__sass_thread_inst_executed_op_dfma_pred_on
@@ -166,8 +167,8 @@ ALGO_BYTES_PER_CS = (512.0 + 768.0 + 768.0) / 3.0
 # Kernels launched on the library's second stream, concurrently with the main stream's.
 SIDE_STREAM_KERNELS = ("k_points_slow",)
 
-KERNEL_FILES_2D = ("af_kernels.cu", "af_math.cuh", "af_device.cuh", "af_internal.h")
-KERNEL_FILES_1D = ("af_kernels1d.cuh", "af_math.cuh", "af_device.cuh", "af_internal.h")
+KERNEL_FILES_2D = ("af_stage.cuh", "af_kernels.cu", "af_math.cuh", "af_device.cuh", "af_internal.h")
+KERNEL_FILES_1D = ("af_kernels1d.cuh", "af_stage.cuh", "af_math.cuh", "af_device.cuh", "af_internal.h")
 
 
 def kernel_digest(files=KERNEL_FILES_2D) -> str:
