@@ -90,17 +90,17 @@ EXEC_FP64_DIVB = {}
 # count them per cell-stage, as the DMUL and DADD counts of the same captures on the
 # build that ran every product on the FP64 pipe (kernel digest e1110cc7...) minus those
 # of the build that first moved them (before the FP32 certificates, which remove FP64
-# work outright): a lower bound, since later changes moved a few more operations; int_add of
-# k_points: the FP64 flops of its line sums before they became fixed-point sums.  The literal count of the paper's formulas (ALGO_FLOPS) is larger where a
-# kernel uses a cheaper algebraic form (the LLF-FVS line as one expression, products
-# by 1/h), so it is reported beside the roofline, never divided by the peak.  Each
-# table names the capture it comes from and a digest of the kernel sources it was
-# taken on: once the kernels change, the line says so ("counts_stale") until the
-# capture is retaken.  The work-list kernels of the limiter slow paths are summed as
-# k_points_slow and k_cells_slow, the names af_timing
-# reports them under.
+# work outright): a lower bound, since later changes moved a few more operations; int_add
+# of k_points holds the FP64 flops of its line sums before they became fixed-point sums.
+# The literal count of the paper's formulas (ALGO_FLOPS) is larger where a kernel uses a
+# cheaper algebraic form (the LLF-FVS line as one expression, products by 1/h), so it is
+# reported beside the roofline, never divided by the peak.  Each table names the capture
+# it comes from and a digest of the kernel sources it was taken on: once the kernels
+# change, the line says so ("counts_stale") until the capture is retaken.  The work-list
+# kernels of the limiter slow paths are k_points_slow and k_cells_slow, the names
+# af_timing reports them under.
 EXEC_FP64 = {
-    "blast_low_beta": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "1a570010dcdba859bc3ba306e21a4c24882b893e", "kernels": {
+    "blast_low_beta": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "c3cebdfe574378ad3452407dd94e4f33c64511e4", "kernels": {
         "k_pointdata": {"dadd": 98.04, "dmul": 0.01, "dfma": 188.15, "pipe": 286.20, "dram_bytes": 1383.8, "int_mul": 124.09, "int_add": 0.00},
         "k_points": {"dadd": 95.13, "dmul": 6.01, "dfma": 160.29, "pipe": 261.42, "dram_bytes": 1618.9, "int_mul": 40.06, "int_add": 184.28},
         "k_points_slow": {"dadd": 0.18, "dmul": 0.29, "dfma": 0.49, "pipe": 1.00, "dram_bytes": 1.9, "int_mul": 0.02, "int_add": 0.00},
@@ -109,7 +109,7 @@ EXEC_FP64 = {
         "k_cells_slow": {"dadd": 0.07, "dmul": 0.19, "dfma": 0.19, "pipe": 0.55, "dram_bytes": 0.7, "int_mul": 0.00, "int_add": 0.00},
         "k_final": {"dadd": 0.00, "dmul": 0.00, "dfma": 21.33, "pipe": 21.33, "dram_bytes": 329.5, "int_mul": 8.33, "int_add": 16.00},
     }},
-    "orszag_tang": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "1a570010dcdba859bc3ba306e21a4c24882b893e", "kernels": {
+    "orszag_tang": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "c3cebdfe574378ad3452407dd94e4f33c64511e4", "kernels": {
         "k_pointdata": {"dadd": 98.00, "dmul": 0.00, "dfma": 188.00, "pipe": 286.00, "dram_bytes": 1206.4, "int_mul": 124.00, "int_add": 0.00},
         "k_points": {"dadd": 96.00, "dmul": 6.00, "dfma": 166.00, "pipe": 268.00, "dram_bytes": 1564.1, "int_mul": 42.00, "int_add": 184.00},
         "k_points_slow": {"dadd": 0.00, "dmul": 0.00, "dfma": 0.00, "pipe": 0.00, "dram_bytes": 0.3, "int_mul": 0.00, "int_add": 0.00},
@@ -118,7 +118,7 @@ EXEC_FP64 = {
         "k_cells_slow": {"dadd": 0.00, "dmul": 0.00, "dfma": 0.00, "pipe": 0.00, "dram_bytes": 0.3, "int_mul": 0.00, "int_add": 0.00},
         "k_final": {"dadd": 0.00, "dmul": 0.00, "dfma": 21.33, "pipe": 21.33, "dram_bytes": 277.7, "int_mul": 8.33, "int_add": 16.00},
     }},
-    "jets": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "1a570010dcdba859bc3ba306e21a4c24882b893e", "kernels": {
+    "jets": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "c3cebdfe574378ad3452407dd94e4f33c64511e4", "kernels": {
         "k_pointdata": {"dadd": 98.05, "dmul": 0.00, "dfma": 188.18, "pipe": 286.22, "dram_bytes": 1366.0, "int_mul": 124.13, "int_add": 0.00},
         "k_points": {"dadd": 101.04, "dmul": 6.10, "dfma": 160.23, "pipe": 267.38, "dram_bytes": 1729.8, "int_mul": 39.14, "int_add": 212.74},
         "k_points_slow": {"dadd": 0.03, "dmul": 0.04, "dfma": 0.06, "pipe": 0.13, "dram_bytes": 0.2, "int_mul": 0.00, "int_add": 0.00},
@@ -127,7 +127,7 @@ EXEC_FP64 = {
         "k_cells_slow": {"dadd": 0.03, "dmul": 0.09, "dfma": 0.10, "pipe": 0.27, "dram_bytes": 0.1, "int_mul": 0.00, "int_add": 0.00},
         "k_final": {"dadd": 0.00, "dmul": 0.00, "dfma": 21.33, "pipe": 21.33, "dram_bytes": 322.1, "int_mul": 8.33, "int_add": 16.00},
     }},
-    "rarefaction_lattice": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "1a570010dcdba859bc3ba306e21a4c24882b893e", "kernels": {
+    "rarefaction_lattice": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "c3cebdfe574378ad3452407dd94e4f33c64511e4", "kernels": {
         "k_pointdata": {"dadd": 98.99, "dmul": 2.36, "dfma": 191.73, "pipe": 293.55, "dram_bytes": 1204.2, "int_mul": 124.00, "int_add": 0.00},
         "k_points": {"dadd": 96.00, "dmul": 6.00, "dfma": 166.80, "pipe": 268.77, "dram_bytes": 1617.8, "int_mul": 39.81, "int_add": 183.99},
         "k_points_slow": {"dadd": 58.64, "dmul": 78.11, "dfma": 132.19, "pipe": 280.47, "dram_bytes": 546.7, "int_mul": 6.84, "int_add": 0.00},
@@ -136,7 +136,7 @@ EXEC_FP64 = {
         "k_cells_slow": {"dadd": 51.57, "dmul": 61.52, "dfma": 226.48, "pipe": 354.38, "dram_bytes": 206.3, "int_mul": 0.00, "int_add": 0.00},
         "k_final": {"dadd": 0.00, "dmul": 2.86, "dfma": 24.20, "pipe": 27.05, "dram_bytes": 277.7, "int_mul": 8.33, "int_add": 13.14},
     }},
-    "blast1d": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "472deb0f4847642bfe445c15c516cdc6c4f11431", "kernels": {
+    "blast1d": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "d2eb860adae4bba34b365caa7c99558845379714", "kernels": {
         "k1_pointdata": {"dadd": 0.69, "dmul": 0.01, "dfma": 2.75, "pipe": 3.45, "dram_bytes": 21.6, "int_mul": 0.00, "int_add": 0.00},
         "k1_points": {"dadd": 0.01, "dmul": 0.00, "dfma": 5.35, "pipe": 5.36, "dram_bytes": 162.9, "int_mul": 0.00, "int_add": 0.00},
         "k1_faces": {"dadd": 0.02, "dmul": 0.01, "dfma": 0.01, "pipe": 0.04, "dram_bytes": 0.2, "int_mul": 0.00, "int_add": 0.00},
@@ -144,7 +144,7 @@ EXEC_FP64 = {
         "k1_final": {"dadd": 0.00, "dmul": 0.00, "dfma": 5.34, "pipe": 5.35, "dram_bytes": 162.4, "int_mul": 0.00, "int_add": 0.00},
     }},
 }
-EXEC_FP64_DIVB["blast_low_beta"] = {"source": "profiles/divb_blast512.md", "digest": "1a570010dcdba859bc3ba306e21a4c24882b893e",
+EXEC_FP64_DIVB["blast_low_beta"] = {"source": "profiles/divb_blast512.md", "digest": "c3cebdfe574378ad3452407dd94e4f33c64511e4",
                                      "dadd": 67.99, "dmul": 19.01, "dfma": 57.03, "pipe": 143.98}
 # FP64 roofline from unit counts and clock: the GB300 SM retires 2 DFMA thread
 # instructions per cycle (ncu: sm__sass_thread_inst_executed_op_dfma_pred_on

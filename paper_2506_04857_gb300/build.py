@@ -1,7 +1,7 @@
 """Build libaf (the CUDA kernels and C ABI) in-tree for sm_103a with nvcc.
 
-The library is written to paper_2506_04857_gb300/_build/libaf.so.  The two
-translation units compile in parallel; the whole build takes a few seconds.
+The library is written to paper_2506_04857_gb300/_build/libaf.so.  The
+translation units compile in parallel.
 """
 from __future__ import annotations
 

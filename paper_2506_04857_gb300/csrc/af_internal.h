@@ -93,7 +93,7 @@ struct AfDev {
   const double *inflow;   // inflow state [8], its point data as a point [AF_NQP] and as an average [AF_NQA]
   double *rec;            // when set: the stage writes its limiter coefficients here (AFC_* slots)
   const double *frz;      // when set: the stage takes its limiter coefficients from here (frozen branch)
-  // work lists of the limiter slow paths (single runs; NULL: slow paths inline, as in batches):
+  // work lists of the limiter slow paths:
   // points whose update leaves the 1e-13 floors (packed class << 28 | index, and their
   // high-order update, component-major), cells whose Sec. 3.2 box is not certified
   // (index, eps_rho, eps_p)

@@ -30,6 +30,9 @@
 
 namespace {
 
+// Blocks of 256 threads per SM the batch kernels are compiled for: the fastest of a sweep (at
+// most 64 registers for the point pass, 80 for the point data, 128 for the cells: a 32-run ensemble
+// 21.6 -> 20.8 ms with them).
 #ifndef AF_KBPT
 #define AF_KBPT 4
 #endif
@@ -296,7 +299,10 @@ inline dim3 grid2(int nx, int ny) { return dim3((nx + 31) / 32, (ny + 3) / 4); }
 #ifndef AF_SMALL
 #define AF_SMALL 1216
 #endif
-// small grids
+// Small grids: up to two warps of a part per scheduler (152 SMs x 4 x 2 row tiles of 32).  There a
+// pass is one chain of dependent operations long and the short chains of AF_LAT pay; above it the
+// FP64 pipe fills and AF_LAT's additional operations cost (10 steps, AF_LAT against the other build:
+// 64 x 64 2036 against 2655 us, 128 x 128 2376 against 2843, 256 x 256 3009 against 2789).
 bool af_small_grid(const AfGrid &g) { return (long long)((g.nxa + 31) / 32) * g.nya <= AF_SMALL; }
 
 #ifndef AF_QUIET_MIN
@@ -340,12 +346,11 @@ void af_launch_divb(const AfDev &d, const AfGrid &g, double *partials, double *o
 }
 // a fixed grid of 4 blocks per SM walks the list
 void af_launch_points_slow(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s) {
-  if (!d.pq) return;
   if (g.special) pass(k_points_slow<true>, 152 * 4, kListThreads, s, d, g, a, b);
   else pass(k_points_slow<false>, 152 * 4, kListThreads, s, d, g, a, b);
 }
 void af_launch_cells_slow(const AfDev &d, const AfGrid &g, cudaStream_t s) {
-  if (d.cq) pass(k_cells_slow, 152 * 4, kListThreads, s, d, g);
+  pass(k_cells_slow, 152 * 4, kListThreads, s, d, g);
 }
 float af_run_fp64_probe(cudaStream_t s, double *flops) {
   int dev = 0, sms = 0;

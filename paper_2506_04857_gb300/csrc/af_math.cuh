@@ -161,7 +161,8 @@ __device__ __forceinline__ double rcp44(float xh, float xl) {
 
 __device__ __forceinline__ double mul_i(double a, double b);
 
-// AF_LAT (the small-grid build): see the end of this file
+// AF_LAT (the build for small grids): a pass runs each function from cold, one warp per scheduler, so
+// the larger ones are compiled once and called (instruction cache), and chains are kept short
 #ifdef AF_LAT
 #define AF_ONCE static __device__ __noinline__
 #else

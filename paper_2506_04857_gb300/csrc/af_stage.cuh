@@ -1,5 +1,8 @@
-// af_stage.cuh -- device functions and kernels of one stage (included by af_kernels.cu and, for
-// small grids, af_kernels_lat.cu).
+// af_stage.cuh -- device functions, kernels and launches of one stage, compiled twice: in
+// af_kernels.cu for large grids and batches, which the FP64 pipe bounds, and with AF_LAT in
+// af_kernels_lat.cu for small grids, which the latency of the passes bounds.  The two builds give
+// bitwise the same results (no contraction beyond the fma written here; the integer variants of
+// AF_LAT are exact restatements).
 #pragma once
 #include "../../include/af.h"
 #include "af_internal.h"
@@ -795,9 +798,6 @@ __device__ __forceinline__ void rk_store(double *out, const double *un, double a
   *out = is_zero(a) ? v : fma(a, AF_LD(un), mul_i(b, v));
 }
 
-struct PointCount {
-  int lim, shr, bad;
-};
 
 // The point value of class cls (1 x-face, 2 y-face, 3 corner) at (i, j), inside its extents.
 // K: what is formed.
@@ -809,7 +809,7 @@ struct PointCount {
 enum { kStage = 0, kPlain = 1, kRhs = 2, kQuiet = 3 };
 template <int cls, bool GB, bool UP, int K>
 __device__ __forceinline__ void b_point(const AfDev &d, const AfGrid &g, const int i, const int j, double a, double b,
-                                        PointCount &n, bool quiet) {
+                                        int &nlim, bool quiet) {
   constexpr bool PL = K == kPlain || K == kQuiet, RHS = K == kRhs;
   if (K == kQuiet && quiet) {   // L(U) = 0: the RK combination of the state itself
     const SV v = sview(d.us[cls], g, cls);
@@ -904,28 +904,18 @@ __device__ __forceinline__ void b_point(const AfDev &d, const AfGrid &g, const i
         double UL[8], out[8];
         point_llf_state<GB>(d, g, cls, i, j, dt, UL);
         scaling_blend(acc, UL, t1, t2, out);
-        n.lim += 1;
+        nlim += 1;
         for (int k = 0; k < 8; ++k) acc[k] = out[k];
       }
     } else if (!clear_of_floor(acc, g)) {
-      if (PL || d.pq) {   // slow path in k_points_slow, over a dense list (the warp does not wait here)
-        const int slot = enqueue(d.st, &d.st->npq, d.pq_cap);
-        if (slot >= 0) {
-          d.pq[slot] = (cls << 28) | (int)op;
+      // slow path in k_points_slow, over a dense list (the warp does not wait here)
+      const int slot = enqueue(d.st, &d.st->npq, d.pq_cap);
+      if (slot >= 0) {
+        d.pq[slot] = (cls << 28) | (int)op;
 #pragma unroll
-          for (int k = 0; k < 8; ++k) d.pqu[(size_t)k * d.pq_cap + slot] = acc[k];
-        }
-        return;
+        for (int k = 0; k < 8; ++k) d.pqu[(size_t)k * d.pq_cap + slot] = acc[k];
       }
-      if constexpr (!PL) {
-        double out[8];
-        int lim, shr, bad;
-        point_pp<GB>(d, g, cls, i, j, acc, dt, out, lim, shr, bad, t1, t2);
-        n.lim += lim;
-        n.shr += shr;
-        n.bad += bad;
-        for (int k = 0; k < 8; ++k) acc[k] = out[k];
-      }
+      return;
     }
     if (!PL && d.rec) {
       d.rec[s1] = t1;
@@ -959,21 +949,15 @@ __device__ __forceinline__ void b_sensor(const AfDev &d, const AfGrid &g, const 
 template <bool GB, bool UP, int K>
 __device__ __forceinline__ void b_points(const AfDev &d, const AfGrid &g, const int i, const int j, double a, double b,
                                          int mode, int z, int lev = 0) {
-  PointCount n = {0, 0, 0};
+  int nlim = 0;
   if (z == 3) {
     if (K != kRhs && lev <= 3) b_sensor<GB>(d, g, i, j);
   } else if (mode != 2 && i < g.ex[z + 1] && j < g.ey[z + 1]) {
-    if (z == 0) b_point<1, GB, UP, K>(d, g, i, j, a, b, n, lev > 0);
-    else if (z == 1) b_point<2, GB, UP, K>(d, g, i, j, a, b, n, lev > 0);
-    else b_point<3, GB, UP, K>(d, g, i, j, a, b, n, lev > 0);
+    if (z == 0) b_point<1, GB, UP, K>(d, g, i, j, a, b, nlim, lev > 0);
+    else if (z == 1) b_point<2, GB, UP, K>(d, g, i, j, a, b, nlim, lev > 0);
+    else b_point<3, GB, UP, K>(d, g, i, j, a, b, nlim, lev > 0);
   }
-  if (K != kStage) return;
-  if (n.lim) atomicAdd(&d.st->cnt[ST_POINT_LIMITED], (unsigned long long)n.lim);
-  if (n.shr) atomicAdd(&d.st->cnt[ST_SHRINK], (unsigned long long)n.shr);
-  if (n.bad) {
-    atomicAdd(&d.st->cnt[ST_NONADMISSIBLE], (unsigned long long)n.bad);
-    atomicOr(&d.st->err, AFE_NONADMISSIBLE);
-  }
+  if (K == kStage && nlim) atomicAdd(&d.st->cnt[ST_POINT_LIMITED], (unsigned long long)nlim);
 }
 
 // ---------------------------------------------------------------------------
@@ -1294,15 +1278,6 @@ __device__ __forceinline__ void cell_source_limit(const double *Ullf, const doub
   th_out = th;
 }
 
-// Full Sec. 3.2 steps (1)-(2) for one cell (slow path).
-__device__ __noinline__ void cell_limiter_full(const double *Ullf, const double *dS, double dtts, const double (*H)[8],
-                                               const AfGrid &g, double *L1, double *Lam, int &srclim, NewtonLog &nl,
-                                               double &th_out) {
-  double eps_rho, eps_p;
-  cell_source_limit(Ullf, dS, dtts, g, L1, srclim, th_out, eps_rho, eps_p);
-  flux_limiter_box(L1, H, eps_rho, eps_p, g.gm1, Lam, nl);
-}
-
 // The anti-diffusive fluxes H_L, H_R, H_D, H_U of cell (i, j) (Sec. 3.2 step 2)
 // from the stored G = theta^s (F - F^LLF) of its faces.
 __device__ __forceinline__ void cell_H(const AfDev &d, const AfGrid &g, int i, int j, double cxf, double cyf,
@@ -1324,8 +1299,7 @@ __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const i
                                         int mode) {
   const size_t PS = (size_t)g.nxa * g.nya;
   const size_t o = (size_t)j * g.nxa + i;
-  int nsrc = 0, nlam = 0, ncfl = 0;
-  NewtonLog nl = {0, 0};
+  int nsrc = 0, ncfl = 0;
   if (i < g.nx && j < g.ny) {
     const double dt = !PL && mode == 1 ? 1.0 : d.sc->dt;
     const int ip = mface(i + 1, g.nx, g.bc), jp = mface(j + 1, g.ny, g.bc);
@@ -1501,7 +1475,7 @@ __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const i
         if (!PL && d.frz) {
         } else if (fast) {
           Lam[0] = Lam[1] = Lam[2] = Lam[3] = 1.0;
-        } else if (PL || d.cq) {   // step (1) here, the box of step (2) in k_cells_slow over a dense list
+        } else {   // step (1) here, the box of step (2) in k_cells_slow over a dense list
           int sl = 0;
           double eps_rho, eps_p;
           cell_source_limit(Ullf, dS, dtts, g, L1, sl, th_src, eps_rho, eps_p);
@@ -1513,19 +1487,6 @@ __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const i
             d.cqe[2 * slot + 1] = eps_p;
           }
           listed = true;
-        } else if constexpr (!PL) {
-          double H[4][8];
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            H[0][k] = cxf * Gf[0][k];
-            H[1][k] = -(cxf * Gf[1][k]);
-            H[2][k] = cyf * Gf[2][k];
-            H[3][k] = -(cyf * Gf[3][k]);
-          }
-          int sl = 0;
-          cell_limiter_full(Ullf, dS, dtts, H, g, L1, Lam, sl, nl, th_src);
-          nsrc += sl;
-          nlam += (Lam[0] < 1.0 || Lam[1] < 1.0 || Lam[2] < 1.0 || Lam[3] < 1.0);
         }
 #pragma unroll
         for (int k = 0; k < 8; ++k) d.lim1[k * PS + o] = L1[k];
@@ -1537,12 +1498,7 @@ __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const i
     }
   }
   if (nsrc) atomicAdd(&d.st->cnt[ST_SRC_LIMITED], (unsigned long long)nsrc);
-  if (nlam) atomicAdd(&d.st->cnt[ST_LAMBDA_LT1], (unsigned long long)nlam);
   if (ncfl) atomicAdd(&d.st->cnt[ST_CFL_VIOLATIONS], (unsigned long long)ncfl);
-  if (nl.solves) {
-    atomicAdd(&d.st->cnt[ST_NEWTON_SOLVES], (unsigned long long)nl.solves);
-    atomicMax(&d.st->cnt[ST_NEWTON_MAXIT], (unsigned long long)nl.maxit);
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1595,7 +1551,7 @@ __device__ __forceinline__ void b_final(const AfDev &d, const AfGrid &g, const i
     const size_t o = (size_t)j * g.nxa + i;
     // with the work lists the box of Sec. 3.2 ran in its own passes: count its cells
     // with some Lambda_I < 1 here (Lambda >= 0: bit-pattern compares on the integer pipe)
-    if (d.cq && !d.frz)
+    if (!d.frz)
       nlam = lt_one(L(i, j, 0)) || lt_one(L(i, j, 1)) || lt_one(L(i, j, 2)) || lt_one(L(i, j, 3));
     double th[4];
     if (d.frz) {   // frozen branch: the recorded face coefficients (after Remark 4.1)
@@ -1747,15 +1703,15 @@ __device__ __forceinline__ void b_repair(const AfDev &d, const AfGrid &g, double
 
 // Programmatic dependent launch: a pass is launched while its predecessor's last blocks run and
 // waits here, before it touches memory, until the predecessor has completed and its writes are
-// visible.  It lets its own successor be launched at once (every block of this pass is resident
-// or done by the time all of them have said so).
+// visible (10 steps of a 64 x 64 vortex: 2008 -> 1550 us).  On large
+// grids it lets its own successor be launched at once (every block of this pass is resident or done
+// by the time all of them have said so); on small grids the successor's blocks then crowd the free
+// SMs (128 x 128: 2531 -> 2929 us), and it is launched when the pass ends.
 __device__ __forceinline__ void pass_begin() {
-#ifndef AF_NOPDL
-#if !defined(AF_LAT) || defined(AF_EARLY)
+#ifndef AF_LAT
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 #endif
   asm volatile("griddepcontrol.wait;" ::: "memory");
-#endif
 }
 
 // True in the one block of a launch that arrives last: every write of the others is visible to it.
@@ -2223,9 +2179,10 @@ __device__ __forceinline__ void quiet_final(const AfDev &d, const AfGrid &g, con
 // Launch bounds of the stage kernels (128 threads): a kernel given AF_MINB_x
 // resident blocks per SM is capped at 65536 / (128 x blocks) registers; without
 // it ptxas picks the count.  The kernels keep the FP64 pipe and the integer
-// pipes busy at once; the defaults are the fastest of a sweep on the 2048x2048
-// blast (point data at 5 blocks = 96 registers, point pass at 8 = 64, cell pass
-// at 5 = 96; faces and final pass at the compiler's count).
+// pipes busy at once; the defaults are the fastest of a sweep (point data and
+// point pass at 8 blocks = 64 registers, cell pass at 5 = 96; faces and final
+// pass at the compiler's count).  On small grids a pass has fewer warps than the
+// chip has schedulers: one warp a block, and all the registers it asks for.
 #ifdef AF_LAT
 #define AF_LB_PD __launch_bounds__(32)
 #define AF_LB_PT __launch_bounds__(32)
@@ -2261,7 +2218,7 @@ __global__ void AF_LB_PD k_pointdata(const __grid_constant__ AfDev d, const __gr
                                                    int reduce_dt) {
   pass_begin();
   // a stage's first pass: the work lists of its point and cell passes start empty
-  if (d.pq && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && threadIdx.y == 0) {
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && threadIdx.y == 0) {
     d.st->npq = 0;
     d.st->ncq = 0;
   }
@@ -2277,8 +2234,6 @@ __global__ void k_dt(const __grid_constant__ AfDev d, const __grid_constant__ Af
   pass_begin();
   if (threadIdx.x == 0 && blockIdx.x == 0) b_dt(d, g);
 }
-// At most 128 registers (4 blocks per SM): the limiter slow path spills a
-// little, the common path runs at twice the occupancy (measured 8 % faster).
 // UP: the velocity-upwind point source (Example 4.2 variant) is compiled in
 // only where it is asked for; the central scheme pays nothing for it.
 template <bool GB, bool UP, int K>
@@ -2389,10 +2344,8 @@ void pass(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t s, A... args) {
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
-#ifndef AF_NOPDL
   c.attrs = &at;
   c.numAttrs = 1;
-#endif
   cudaLaunchKernelEx(&c, k, P(args)...);
 }
 inline Shape shape(int nx, int ny, int nz) {
@@ -2422,7 +2375,7 @@ void launch_pointdata(const AfDev &d, const AfGrid &g, int reduce_dt, cudaStream
 }
 void launch_points(const AfDev &d, const AfGrid &g, double a, double b, int mode, cudaStream_t s) {
   const Shape h = shape(g, g.nxa, g.nya, mode != 1 && g.kappa != 0.0 ? 4 : 3);
-  const int kind = mode == 1 ? kRhs : (mode == 0 && d.pq && !d.rec && !d.frz && !g.upwind ? kPlain : kStage);
+  const int kind = mode == 1 ? kRhs : (mode == 0 && !d.rec && !d.frz && !g.upwind ? kPlain : kStage);
   auto go = [&](auto k) { pass(k, h.g, h.b, s, d, g, a, b, mode); };
   if (g.special) {
     if (kind == kPlain) go(k_points<true, false, kPlain>);
@@ -2442,7 +2395,7 @@ void launch_faces(const AfDev &d, const AfGrid &g, int mode, cudaStream_t s) {
 }
 void launch_cells(const AfDev &d, const AfGrid &g, double a, double b, int mode, cudaStream_t s) {
   const Shape h = shape(g, g.nx, g.ny, 1);
-  const bool plain = mode == 0 && g.pp_on && d.cq && !d.rec && !d.frz;
+  const bool plain = mode == 0 && g.pp_on && !d.rec && !d.frz;
   if (g.special) {
     if (plain) pass(k_cells<true, true>, h.g, h.b, s, d, g, a, b, mode);
     else pass(k_cells<true, false>, h.g, h.b, s, d, g, a, b, mode);
