@@ -5,13 +5,11 @@
 
 #include "af_internal.h"
 
-// Loads of the stage's arrays.  The small-grid build runs several passes in one kernel
-// (k1_step), where the read-only path must not be used for what the kernel itself wrote.
-#ifdef AF_LAT
-#define AF_LD(p) (*(p))
-#else
-#define AF_LD(p) __ldg(p)
-#endif
+// The stage's arrays are read by ordinary loads.  The read-only path (__ldg) wants data that
+// nothing writes while the reading kernel lives: here a pass is launched while the pass before it
+// still writes (pass_begin), and k1_step runs all the passes in one kernel.  An ordinary load
+// stays behind the wait of pass_begin, and behind every store in front of it: the passes load
+// what they need before their first store.
 
 namespace {
 
@@ -32,7 +30,7 @@ struct SV {   // one DoF class of a state: component k at (i,j) is p[k*cs + j*ex
   size_t cs;
   int ex;
   __device__ __forceinline__ double operator()(int i, int j, int k) const {
-    return AF_LD(p + (size_t)k * cs + (size_t)j * ex + i);
+    return p[(size_t)k * cs + (size_t)j * ex + i];
   }
 };
 __device__ __forceinline__ SV sview(const double *p, const AfGrid &g, int c) {
@@ -47,7 +45,7 @@ struct WV {   // a work array [q][nya][nxa]
   size_t PS;
   int nxa;
   __device__ __forceinline__ double operator()(int i, int j, int q) const {
-    return AF_LD(p + (size_t)q * PS + (size_t)j * nxa + i);
+    return p[(size_t)q * PS + (size_t)j * nxa + i];
   }
 };
 __device__ __forceinline__ WV wview(const double *p, const AfGrid &g) {

@@ -137,13 +137,7 @@ __device__ __forceinline__ void b1_points(const AfDev &d, const AfGrid &g, int f
       for (int k = 0; k < 8; ++k) acc[k] = out[k];
     }
     const size_t cs = (size_t)g.ex[1];
-    if (a == 0.0) {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) d.uo[1][k * cs + f] = acc[k];
-    } else {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) d.uo[1][k * cs + f] = fma(a, AF_LD(d.un[1] + k * cs + f), b * acc[k]);
-    }
+    rk_store(d.uo[1] + f, d.un[1] + f, cs, a, b, acc);
   }
   if ((parts & 2) && f < g.nx && g.kappa != 0.0) {
     double phi[4];
@@ -175,18 +169,23 @@ __device__ __forceinline__ void b1_faces(const AfDev &d, const AfGrid &g, int f)
     // unmapped cell indices: an outflow ghost cell's phi comes from its own (mirrored) neighbours
     const double ts = theta_s<false>(d, g, 0, f - 1, 0, f, 0);
     double *out = d.fx + f;
+    double Fl[8], G[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      double Fh = 0.0, Fl;
+      double Fh = 0.0;
       if (k != 4) {
         const int s = QP_F1 + fslot(0, k);
         Fh = PW(f, 0, s);
-        Fl = 0.5 * fma(-al, Ub(cb, 0, k) - Ub(ca, 0, k), A(ca, 0, s) + A(cb, 0, s));
+        Fl[k] = 0.5 * fma(-al, Ub(cb, 0, k) - Ub(ca, 0, k), A(ca, 0, s) + A(cb, 0, s));
       } else {
-        Fl = -0.5 * al * (Ub(cb, 0, k) - Ub(ca, 0, k));
+        Fl[k] = -0.5 * al * (Ub(cb, 0, k) - Ub(ca, 0, k));
       }
-      out[(QF_FLLF + k) * PS] = Fl;
-      out[(QF_G + k) * PS] = is_one(ts) ? Fh - Fl : ts * (Fh - Fl);
+      G[k] = is_one(ts) ? Fh - Fl[k] : ts * (Fh - Fl[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      out[(QF_FLLF + k) * PS] = Fl[k];
+      out[(QF_G + k) * PS] = G[k];
     }
     out[QF_TS * PS] = ts;
     out[QF_AL * PS] = al;
@@ -236,11 +235,10 @@ __device__ __forceinline__ void b1_cells(const AfDev &d, const AfGrid &g, int i,
     const size_t cs0 = (size_t)g.nx;
     if (!g.pp_on) {
       // no PP: the blended high-order update, then the RK combination
+      double fe[8];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const double fe = Ullf[k] + H[0][k] + H[1][k];
-        d.uo[0][k * cs0 + i] = a == 0.0 ? fe : fma(a, AF_LD(d.un[0] + k * cs0 + i), b * fe);
-      }
+      for (int k = 0; k < 8; ++k) fe[k] = Ullf[k] + H[0][k] + H[1][k];
+      rk_store(d.uo[0] + i, d.un[0] + i, cs0, a, b, fe);
     } else {
       if (dt * ((FX(i, 0, QF_AL) + FX(ip, 0, QF_AL)) * g.rdx) > 1.0 + 1e-12) ncfl = 1;   // Lemma 3.1 (count only)
       double Lam[4];
@@ -301,14 +299,15 @@ __device__ __forceinline__ void b1_final(const AfDev &d, const AfGrid &g, int i,
     const double dt = d.sc->dt;
     const WV L = wview(d.lam, g);
     const double tl = theta1(g, L, i), tr = theta1(g, L, i + 1);
+    double fe[8];
+    value1(d, g, i, tl, tr, dt, fe);
+    rk_store(d.uo[0] + i, d.un[0] + i, (size_t)g.nx, a, b, fe);
     d.thx[i] = tl;
     nface += lt_one(tl);
     if (g.bc == 1 && i == g.nx - 1) {
       d.thx[i + 1] = tr;
       nface += lt_one(tr);
     }
-    double fe[8];
-    value1(d, g, i, tl, tr, dt, fe);
     bool ok = fe[0] > 0.0 && qform(fe, 0.0) > 0.0;
 #pragma unroll
     for (int k = 0; k < 8; ++k) ok = ok && finite_bits(fe[k]);
@@ -317,9 +316,6 @@ __device__ __forceinline__ void b1_final(const AfDev &d, const AfGrid &g, int i,
       if (slot < AF_MAX_REPAIR) d.st->repair[slot] = i;
       else atomicOr(&d.st->err, AFE_REPAIR_OVERFLOW);
     }
-    const size_t cs0 = (size_t)g.nx;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) d.uo[0][k * cs0 + i] = a == 0.0 ? fe[k] : fma(a, AF_LD(d.un[0] + k * cs0 + i), b * fe[k]);
   }
   if (nface) atomicAdd(&d.st->cnt[ST_FACE_THETA_LT1], (unsigned long long)nface);
 }
@@ -437,7 +433,7 @@ __global__ void __launch_bounds__(3 * kStepThreads) k1_step(const __grid_constan
 #else
 // Quiet tiles of 128 indices, as in 2D (levels d.lev, one per block)
 constexpr int kTile1 = 128;
-__device__ __forceinline__ int level1(const AfDev &d) { return d.lev ? AF_LD(d.lev + blockIdx.x) : 0; }
+__device__ __forceinline__ int level1(const AfDev &d) { return d.lev ? d.lev[blockIdx.x] : 0; }
 __global__ void __launch_bounds__(kTile1) k1_quiet1(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g) {
   pass_begin();
   const int i0 = blockIdx.x * kTile1, i = i0 + threadIdx.x;
@@ -492,11 +488,11 @@ __global__ void __launch_bounds__(128) k1_points(const __grid_constant__ AfDev d
   pass_begin();
   const int lev = level1(d), i = blockIdx.x * blockDim.x + threadIdx.x;
   if (blockIdx.y == 0 && lev > 0) {
-    const SV P = sview(d.us[1], g, 1);
-    const size_t cs = (size_t)g.ex[1];
-    if (i < g.ex[1])
-#pragma unroll
-      for (int k = 0; k < 8; ++k) rk_store(d.uo[1] + k * cs + i, d.un[1] + k * cs + i, a, b, P(i, 0, k));
+    if (i < g.ex[1]) {
+      double V[8];
+      load8(sview(d.us[1], g, 1), i, 0, V);
+      rk_store(d.uo[1] + i, d.un[1] + i, (size_t)g.ex[1], a, b, V);
+    }
     return;
   }
   if (blockIdx.y == 0 || lev <= 3) b1_points(d, g, i, a, b, 1 << blockIdx.y);
@@ -513,9 +509,10 @@ __global__ void __launch_bounds__(128) k1_cells(const __grid_constant__ AfDev d,
     if (i < g.nx && threadIdx.x % 32 == 0 && quiet_cfl1(d, g, i))
       atomicAdd(&d.st->cnt[ST_CFL_VIOLATIONS], (unsigned long long)min(32, g.nx - i));
     if (i < g.nx && lev == 1) {
-      const SV A = sview(d.us[0], g, 0);
+      double V[8];
+      load8(sview(d.us[0], g, 0), i, 0, V);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) d.lim1[(size_t)k * g.nxa + i] = A(i, 0, k);
+      for (int k = 0; k < 8; ++k) d.lim1[(size_t)k * g.nxa + i] = V[k];
       d.lam[i] = d.lam[(size_t)g.nxa + i] = 1.0;
     }
     return;
@@ -528,10 +525,9 @@ __global__ void __launch_bounds__(128) k1_final(const __grid_constant__ AfDev d,
   const int lev = level1(d), i = blockIdx.x * blockDim.x + threadIdx.x;
   if (lev > 0) {
     if (i >= g.nx) return;
-    const SV A = sview(d.us[0], g, 0);
-    const size_t cs0 = (size_t)g.nx;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) rk_store(d.uo[0] + k * cs0 + i, d.un[0] + k * cs0 + i, a, b, A(i, 0, k));
+    double V[8];
+    load8(sview(d.us[0], g, 0), i, 0, V);
+    rk_store(d.uo[0] + i, d.un[0] + i, (size_t)g.nx, a, b, V);
     if (lev == 1) {
       d.thx[i] = 1.0;
       if (g.bc == 1 && i == g.nx - 1) d.thx[i + 1] = 1.0;

@@ -423,9 +423,9 @@ __device__ __forceinline__ PP pref(const AfDev &d, const AfGrid &g, int c, int i
   p.j = j;
   return p;
 }
-__device__ __forceinline__ double pu(const PP &p, int k) { return AF_LD(p.u + (size_t)k * p.ucs + (size_t)p.j * p.uex + p.i); }
+__device__ __forceinline__ double pu(const PP &p, int k) { return p.u[(size_t)k * p.ucs + (size_t)p.j * p.uex + p.i]; }
 __device__ __forceinline__ double pw(const PP &p, size_t PS, int nxa, int q) {
-  return AF_LD(p.w + (size_t)q * PS + (size_t)p.j * nxa + p.i);
+  return p.w[(size_t)q * PS + (size_t)p.j * nxa + p.i];
 }
 
 // ---- reflective and inflow sides -------------------------------------------
@@ -506,7 +506,7 @@ __device__ __forceinline__ PPG prefg(const AfDev &d, const AfGrid &g, int c, int
 }
 __device__ __forceinline__ double pug(const PPG &q, int k) { return flipv(pu(q.p, k), q.um, k); }
 __device__ __forceinline__ double pwg(const PPG &q, int s) {
-  return flipv(AF_LD(q.p.w + (size_t)s * q.wps + (size_t)q.p.j * q.wnx + q.p.i), q.wm, s);
+  return flipv(q.p.w[(size_t)s * q.wps + (size_t)q.p.j * q.wnx + q.p.i], q.wm, s);
 }
 // the 8 state values of DoF (cls, i, j) (unmapped; cls 0..3)
 template <bool GB>
@@ -763,14 +763,14 @@ __device__ void sensor_phi(const AfDev &d, const AfGrid &g, int ci, int cj, doub
     if constexpr (GB) {
       return pwg(prefg(d, g, 0, a, b), q);
     } else {
-      return AF_LD(d.pd[0] + (size_t)q * g.nxa * g.nya + (size_t)mcell(b, g.ny, g.bc) * g.nxa + mcell(a, g.nx, g.bc));
+      return d.pd[0][(size_t)q * g.nxa * g.nya + (size_t)mcell(b, g.ny, g.bc) * g.nxa + mcell(a, g.nx, g.bc)];
     }
   };
   auto Ub = [&](int a, int b, int k) -> double {
     if constexpr (GB) {
       return pug(prefg(d, g, 0, a, b), k);
     } else {
-      return AF_LD(d.us[0] + (size_t)k * g.nx * g.ny + (size_t)mcell(b, g.ny, g.bc) * g.nx + mcell(a, g.nx, g.bc));
+      return d.us[0][(size_t)k * g.nx * g.ny + (size_t)mcell(b, g.ny, g.bc) * g.nx + mcell(a, g.nx, g.bc)];
     }
   };
   const int e = ci + 1, w = ci - 1, n = cj + 1, s = cj - 1;
@@ -793,9 +793,18 @@ __device__ void sensor_phi(const AfDev &d, const AfGrid &g, int ci, int cj, doub
   phi[3] = ddiv(absd(num), absd(Ub(ci, cj, 4) + Ub(ci, cj, 5)) + 1e-40);
 }
 
-// out = a U^n + b v of the Runge-Kutta stage (a = 0: v itself)
-__device__ __forceinline__ void rk_store(double *out, const double *un, double a, double b, double v) {
-  *out = is_zero(a) ? v : fma(a, AF_LD(un), mul_i(b, v));
+// out_k = a U^n_k + b v_k of the Runge-Kutta stage (a = 0: v itself), components cs apart
+__device__ __forceinline__ void rk_store(double *out, const double *un, size_t cs, double a, double b, const double *v) {
+  if (is_zero(a)) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) out[k * cs] = v[k];
+  } else {
+    double n[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) n[k] = un[k * cs];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) out[k * cs] = fma(a, n[k], mul_i(b, v[k]));
+  }
 }
 
 
@@ -812,10 +821,10 @@ __device__ __forceinline__ void b_point(const AfDev &d, const AfGrid &g, const i
                                         int &nlim, bool quiet) {
   constexpr bool PL = K == kPlain || K == kQuiet, RHS = K == kRhs;
   if (K == kQuiet && quiet) {   // L(U) = 0: the RK combination of the state itself
-    const SV v = sview(d.us[cls], g, cls);
     const size_t cs = (size_t)g.ex[cls] * g.ey[cls], oo = (size_t)j * g.ex[cls] + i;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) rk_store(d.uo[cls] + k * cs + oo, d.un[cls] + k * cs + oo, a, b, v(i, j, k));
+    double v[8];
+    load8(sview(d.us[cls], g, cls), i, j, v);
+    rk_store(d.uo[cls] + oo, d.un[cls] + oo, cs, a, b, v);
     return;
   }
   const size_t PS = (size_t)g.nxa * g.nya;
@@ -922,14 +931,7 @@ __device__ __forceinline__ void b_point(const AfDev &d, const AfGrid &g, const i
       d.rec[s1 + PS] = t2;
     }
   }
-  if (is_zero(a)) {
-#pragma unroll
-    for (int k = 0; k < 8; ++k) uo[k * cs + oo] = acc[k];
-  } else {
-    const double *un = d.un[cls];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) uo[k * cs + oo] = fma(a, AF_LD(un + k * cs + oo), mul_i(b, acc[k]));
-  }
+  rk_store(uo + oo, d.un[cls] + oo, cs, a, b, acc);
 }
 
 template <bool GB>
@@ -1022,18 +1024,24 @@ __device__ __forceinline__ void face(const AfDev &d, const AfGrid &g, double *ou
                    A(cbi, cbj, QA_SRHO), Ba, Bb);
   }
   const int f0 = L == 0 ? QP_F1 : QP_F2;
+  double Fl[8], G[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
-    double Fh = 0.0, Fl = 0.0;
+    double Fh = 0.0;
+    Fl[k] = 0.0;
     if (k != 4 + L) {
       const int s = f0 + fslot(L, k);
       Fh = mul_i(fma(4.0, pw(mid, PS, g.nxa, s), pw(lo, PS, g.nxa, s) + pw(hi, PS, g.nxa, s)), 1.0 / 6.0);
-      if (llf) Fl = ldexp_i<-1>(fma(-al, Ub(cbi, cbj, k) - Ub(cai, caj, k), A(cai, caj, s) + A(cbi, cbj, s)));
+      if (llf) Fl[k] = ldexp_i<-1>(fma(-al, Ub(cbi, cbj, k) - Ub(cai, caj, k), A(cai, caj, s) + A(cbi, cbj, s)));
     } else if (llf) {
-      Fl = mul_i(ldexp_i<-1>(neg_i(al)), Ub(cbi, cbj, k) - Ub(cai, caj, k));
+      Fl[k] = mul_i(ldexp_i<-1>(neg_i(al)), Ub(cbi, cbj, k) - Ub(cai, caj, k));
     }
-    out[(QF_FLLF + k) * PS] = Fl;
-    out[(QF_G + k) * PS] = is_one(ts) ? Fh - Fl : mul_i(ts, Fh - Fl);
+    G[k] = is_one(ts) ? Fh - Fl[k] : mul_i(ts, Fh - Fl[k]);
+  }
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    out[(QF_FLLF + k) * PS] = Fl[k];
+    out[(QF_G + k) * PS] = G[k];
   }
   out[QF_TS * PS] = ts;
   out[QF_AL * PS] = al;
@@ -1382,12 +1390,15 @@ __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const i
     const size_t cs0 = (size_t)g.nx * g.ny, o0 = (size_t)j * g.nx + i;
     if (!PL && mode == 1) {
       // semi-discrete rhs: -(F_R - F_L)/dx - (F_U - F_D)/dy - S (G holds the Simpson flux here)
+      double L[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         const double fl = FX(i, j, QF_G + k), fr = FX(ip, j, QF_G + k);
         const double fd = FY(i, j, QF_G + k), fu = FY(i, jp, QF_G + k);
-        uo[k * cs0 + o0] = fma(fl - fr, g.rdx, (fd - fu) * g.rdy) - S[k];
+        L[k] = fma(fl - fr, g.rdx, (fd - fu) * g.rdy) - S[k];
       }
+#pragma unroll
+      for (int k = 0; k < 8; ++k) uo[k * cs0 + o0] = L[k];
     } else {
       // S^LLF = (central div Bbar) Psi(Ubar)
       double be, bw, bn, bs;
@@ -1424,14 +1435,15 @@ __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const i
       const double tsc = minnn(minnn(tsL, tsR), minnn(tsD, tsU));
       if ((!PL || ANY) && !g.pp_on) {
         // sensor-blended high-order update: F^ss = F^LLF + G, S^ss = S^LLF + theta^s (S - S^LLF)
+        double fe[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           const double fl = FX(i, j, QF_FLLF + k) + FX(i, j, QF_G + k), fr = FX(ip, j, QF_FLLF + k) + FX(ip, j, QF_G + k);
           const double fd = FY(i, j, QF_FLLF + k) + FY(i, j, QF_G + k), fu = FY(i, jp, QF_FLLF + k) + FY(i, jp, QF_G + k);
           const double sss = fma(tsc, S[k] - SL[k], SL[k]);
-          const double fe = fma(-dt, sss, fma(-cyf, fu - fd, fma(-cxf, fr - fl, Ubar[k])));
-          uo[k * cs0 + o0] = a == 0.0 ? fe : fma(a, AF_LD(d.un[0] + k * cs0 + o0), b * fe);
+          fe[k] = fma(-dt, sss, fma(-cyf, fu - fd, fma(-cxf, fr - fl, Ubar[k])));
         }
+        rk_store(uo + o0, d.un[0] + o0, cs0, a, b, fe);
       } else {
         // eq. (2d_llf): U^LLF; U^src - U^LLF = -dt theta^s_ij (S - S^LLF)
         double Ullf[8], dS[8], Gf[4][8];
@@ -1567,6 +1579,10 @@ __device__ __forceinline__ void b_final(const AfDev &d, const AfGrid &g, const i
       th[2] = theta_y(g, L, i, j);
       th[3] = theta_y(g, L, i, j + 1);
     }
+    double fe[8];
+    limited_value(d, g, i, j, th, dt, fe);
+    const size_t cs0 = (size_t)g.nx * g.ny, o0 = (size_t)j * g.nx + i;
+    rk_store(d.uo[0] + o0, d.un[0] + o0, cs0, a, b, fe);
     d.thx[o] = th[0];
     d.thy[o] = th[2];
     nface += lt_one(th[0]) + lt_one(th[2]);
@@ -1578,8 +1594,6 @@ __device__ __forceinline__ void b_final(const AfDev &d, const AfGrid &g, const i
       d.thy[o + g.nxa] = th[3];
       nface += lt_one(th[3]);
     }
-    double fe[8];
-    limited_value(d, g, i, j, th, dt, fe);
     // rho > 0 and p > 0 and all finite, on the integer pipe: for finite doubles
     // x > 0 exactly when the bit pattern, read as a signed integer, is > 0
     bool ok = (long long)bits(fe[0]) > 0;
@@ -1590,14 +1604,6 @@ __device__ __forceinline__ void b_final(const AfDev &d, const AfGrid &g, const i
       const int slot = atomicAdd(&d.st->nrepair, 1);
       if (slot < AF_MAX_REPAIR) d.st->repair[slot] = j * g.nx + i;
       else atomicOr(&d.st->err, AFE_REPAIR_OVERFLOW);
-    }
-    const size_t cs0 = (size_t)g.nx * g.ny, o0 = (size_t)j * g.nx + i;
-    if (is_zero(a)) {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) d.uo[0][k * cs0 + o0] = fe[k];
-    } else {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) d.uo[0][k * cs0 + o0] = fma(a, AF_LD(d.un[0] + k * cs0 + o0), mul_i(b, fe[k]));
     }
   }
   if (nface) atomicAdd(&d.st->cnt[ST_FACE_THETA_LT1], (unsigned long long)nface);
@@ -1856,8 +1862,7 @@ __device__ __forceinline__ void points_short(const AfDev &d, const AfGrid &g, do
     d.rec[s1 + PS] = t2;
   }
   const size_t cs = (size_t)g.ex[cls] * g.ey[cls], oo = (size_t)j * g.ex[cls] + i;
-#pragma unroll
-  for (int k = 0; k < 8; ++k) rk_store(d.uo[cls] + k * cs + oo, d.un[cls] + k * cs + oo, a, b, out[k]);
+  rk_store(d.uo[cls] + oo, d.un[cls] + oo, cs, a, b, out);
   if (lim) atomicAdd(&d.st->cnt[ST_POINT_LIMITED], 1ull);
   if (shr) atomicAdd(&d.st->cnt[ST_SHRINK], 1ull);
   if (bad) {
@@ -1893,16 +1898,8 @@ __device__ __forceinline__ void b_points_slow(const AfDev &d, const AfGrid &g, d
       d.rec[s1] = t1;
       d.rec[s1 + PS] = t2;
     }
-    double *uo = d.uo[cls];
     const size_t cs = (size_t)g.ex[cls] * g.ey[cls], oo = (size_t)j * g.ex[cls] + i;
-    if (a == 0.0) {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) uo[k * cs + oo] = out[k];
-    } else {
-      const double *un = d.un[cls];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) uo[k * cs + oo] = fma(a, AF_LD(un + k * cs + oo), b * out[k]);
-    }
+    rk_store(d.uo[cls] + oo, d.un[cls] + oo, cs, a, b, out);
   }
   if (nlim) atomicAdd(&d.st->cnt[ST_POINT_LIMITED], (unsigned long long)nlim);
   if (nshr) atomicAdd(&d.st->cnt[ST_SHRINK], (unsigned long long)nshr);
@@ -2133,7 +2130,7 @@ __global__ void __launch_bounds__(128) k_quiet23(const __grid_constant__ AfDev d
 }
 // level of the block's tile (0 where no levels are kept)
 __device__ __forceinline__ int tile_level(const AfDev &d) {
-  return d.lev ? AF_LD(d.lev + (size_t)blockIdx.y * d.ntx + blockIdx.x) : 0;
+  return d.lev ? d.lev[(size_t)blockIdx.y * d.ntx + blockIdx.x] : 0;
 }
 // The Lemma 3.1 CFL count of the cells of a quiet tile, all alike: the cell pass's expression with
 // both states V.  An FP32 upper bound of it decides first (cf^2 <= (gamma (gamma - 1) E + |B|^2) / rho).
@@ -2157,19 +2154,20 @@ __device__ __forceinline__ void quiet_cells(const AfDev &d, const AfGrid &g, con
     atomicAdd(&d.st->cnt[ST_CFL_VIOLATIONS], (unsigned long long)min(32, g.nx - t.i));
   if (!in || lev > 1) return;
   const size_t PS = (size_t)g.nxa * g.nya, o = (size_t)t.j * g.nxa + t.i;
-  const SV U = sview(d.us[0], g, 0);
+  double V[8];
+  load8(sview(d.us[0], g, 0), t.i, t.j, V);
 #pragma unroll
-  for (int k = 0; k < 8; ++k) d.lim1[k * PS + o] = U(t.i, t.j, k);
+  for (int k = 0; k < 8; ++k) d.lim1[k * PS + o] = V[k];
 #pragma unroll
   for (int I = 0; I < 4; ++I) d.lam[I * PS + o] = 1.0;
 }
 __device__ __forceinline__ void quiet_final(const AfDev &d, const AfGrid &g, const int i, const int j, double a, double b,
                                             int lev) {
   if (!(i < g.nx && j < g.ny)) return;
-  const SV U = sview(d.us[0], g, 0);
   const size_t cs0 = (size_t)g.nx * g.ny, o0 = (size_t)j * g.nx + i, o = (size_t)j * g.nxa + i;
-#pragma unroll
-  for (int k = 0; k < 8; ++k) rk_store(d.uo[0] + k * cs0 + o0, d.un[0] + k * cs0 + o0, a, b, U(i, j, k));
+  double V[8];
+  load8(sview(d.us[0], g, 0), i, j, V);
+  rk_store(d.uo[0] + o0, d.un[0] + o0, cs0, a, b, V);
   if (lev > 1) return;
   d.thx[o] = d.thy[o] = 1.0;
   if (g.bc == 1 && i == g.nx - 1) d.thx[o + 1] = 1.0;
@@ -2180,8 +2178,8 @@ __device__ __forceinline__ void quiet_final(const AfDev &d, const AfGrid &g, con
 // resident blocks per SM is capped at 65536 / (128 x blocks) registers; without
 // it ptxas picks the count.  The kernels keep the FP64 pipe and the integer
 // pipes busy at once; the defaults are the fastest of a sweep (point data and
-// point pass at 8 blocks = 64 registers, cell pass at 5 = 96; faces and final
-// pass at the compiler's count).  On small grids a pass has fewer warps than the
+// point pass at 8 blocks = 64 registers, cell pass at 5 = 96, faces at 9 = 56; the
+// final pass at the compiler's count).  On small grids a pass has fewer warps than the
 // chip has schedulers: one warp a block, and all the registers it asks for.
 #ifdef AF_LAT
 #define AF_LB_PD __launch_bounds__(32)
@@ -2199,11 +2197,11 @@ __device__ __forceinline__ void quiet_final(const AfDev &d, const AfGrid &g, con
 #define AF_MINB_PT 8
 #endif
 #define AF_LB_PT AF_LB(AF_MINB_PT)
-#ifdef AF_MINB_FC
-#define AF_LB_FC AF_LB(AF_MINB_FC)
-#else
-#define AF_LB_FC __launch_bounds__(128)
+// faces: 56 registers (9 blocks) 706 us at 1536 x 1536, 72 (the compiler's count) 738, 64 716
+#ifndef AF_MINB_FC
+#define AF_MINB_FC 9
 #endif
+#define AF_LB_FC AF_LB(AF_MINB_FC)
 #ifndef AF_MINB_CL
 #define AF_MINB_CL 5
 #endif
