@@ -1707,18 +1707,15 @@ __device__ __forceinline__ void b_repair(const AfDev &d, const AfGrid &g, double
 // ---------------------------------------------------------------------------
 #define AF_IJ blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y
 
-// Programmatic dependent launch: a pass is launched while its predecessor's last blocks run and
+// Programmatic dependent launch: the next pass is launched as the blocks of its predecessor end, and
 // waits here, before it touches memory, until the predecessor has completed and its writes are
-// visible (10 steps of a 64 x 64 vortex: 2008 -> 1550 us).  On large
-// grids it lets its own successor be launched at once (every block of this pass is resident or done
-// by the time all of them have said so); on small grids the successor's blocks then crowd the free
-// SMs (128 x 128: 2531 -> 2929 us), and it is launched when the pass ends.
-__device__ __forceinline__ void pass_begin() {
-#ifndef AF_LAT
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-#endif
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-}
+// visible (10 steps of a 64 x 64 vortex: 2008 -> 1550 us).  No pass lets its successor start earlier
+// (griddepcontrol.launch_dependents): the blocks of the successor then wait on the SMs, and hold
+// them against whatever runs beside the pass -- the point list on the second stream (a step of a
+// limited lattice, with the early start and without: 256 x 256 1.47 and 1.19 ms, 512 x 512 3.75 and
+// 3.46) and, on small grids, the pass itself (128 x 128 vortex, 10 steps: 2929 and 2531 us).
+// Nothing gains from it (2048 x 2048 blast: 17.6 and 17.2 ms; 4M cells in 1D 11.3 and 11.1).
+__device__ __forceinline__ void pass_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // True in the one block of a launch that arrives last: every write of the others is visible to it.
 // On small grids, what follows a whole pass in one thread (dt, the repair list) runs there instead
@@ -2197,11 +2194,12 @@ __device__ __forceinline__ void quiet_final(const AfDev &d, const AfGrid &g, con
 #define AF_MINB_PT 8
 #endif
 #define AF_LB_PT AF_LB(AF_MINB_PT)
-// faces: 56 registers (9 blocks) 706 us at 1536 x 1536, 72 (the compiler's count) 738, 64 716
+// faces: 56 registers (9 blocks) 706 us at 1536 x 1536, 72 (the compiler's count) 738, 64 716; the
+// ghost code of special sides would spill at that
 #ifndef AF_MINB_FC
 #define AF_MINB_FC 9
 #endif
-#define AF_LB_FC AF_LB(AF_MINB_FC)
+#define AF_LB_FC AF_LB(GB ? 1 : AF_MINB_FC)
 #ifndef AF_MINB_CL
 #define AF_MINB_CL 5
 #endif

@@ -1,6 +1,8 @@
 """Kernels launched programmatically dependent on their predecessor (`pass` in af_stage.cuh) run
 beside it: each must wait (pass_begin) before it touches memory, and none may read the stage's arrays
-through the read-only path, whose data must not change while the kernel lives.  Checked on the source."""
+through the read-only path, whose data must not change while the kernel lives.  None starts its
+successor early either: blocks that wait hold the SMs against the point list on the second stream.
+Checked on the source."""
 import os
 import re
 
@@ -27,3 +29,7 @@ def test_dependent_kernels_wait_first():
         assert bodies, k
         for b in bodies:
             assert b.strip() == "pass_begin();", (k, b)
+
+
+def test_no_early_start():
+    assert "launch_dependents" not in "".join(code(f) for f in FILES)
