@@ -47,7 +47,7 @@ __device__ __forceinline__ int enqueue(AfStatus *st, int *counter, int cap) {
 __device__ __forceinline__ double pressure(const double *U, double gm1) {
   double m2 = fma(U[1], U[1], fma(U[2], U[2], U[3] * U[3]));
   double b2 = fma(U[4], U[4], fma(U[5], U[5], U[6] * U[6]));
-  return gm1 * (U[7] - 0.5 * ddiv(m2, U[0]) - 0.5 * b2);
+  return gm1 * fma(-0.5, b2, fma(-0.5, ddiv(m2, U[0]), U[7]));
 }
 // q = rho E - |m|^2/2 - rho |B|^2/2 - rho c; q >= 0 <=> p >= (gamma-1) c for rho > 0
 __device__ __forceinline__ double qform(const double *U, double c) {
@@ -1460,7 +1460,7 @@ __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const i
         }
         // Lemma 3.1 CFL condition (diagnostic count only)
         {
-          const double lhs = mul_i(dt, (FX(i, j, QF_AL) + FX(ip, j, QF_AL)) * g.rdx + (FY(i, j, QF_AL) + FY(i, jp, QF_AL)) * g.rdy +
+          const double lhs = mul_i(dt, fma(FX(i, j, QF_AL) + FX(ip, j, QF_AL), g.rdx, (FY(i, j, QF_AL) + FY(i, jp, QF_AL)) * g.rdy) +
                                    ddiv(absd(divBb), A(i, j, QA_SRHO)));
           ncfl += gt_pos(lhs, 1.0 + 1e-12);
         }
@@ -2143,7 +2143,7 @@ __device__ __noinline__ bool quiet_cfl(const AfDev &d, const AfGrid &g, int i, i
   full_data(V, g, f);
   const double a1 = alpha_llf(f.v[0], f.v[0], f.cf[0], f.cf[0], f.srho, f.srho, f.B, f.B);
   const double a2 = alpha_llf(f.v[1], f.v[1], f.cf[1], f.cf[1], f.srho, f.srho, f.B, f.B);
-  return gt_pos(mul_i(dt, (a1 + a1) * g.rdx + (a2 + a2) * g.rdy), 1.0 + 1e-12);
+  return gt_pos(mul_i(dt, fma(a1 + a1, g.rdx, (a2 + a2) * g.rdy)), 1.0 + 1e-12);
 }
 __device__ __forceinline__ void quiet_cells(const AfDev &d, const AfGrid &g, const Tile &t, int lev) {
   const bool in = t.i < g.nx && t.j < g.ny;
