@@ -43,9 +43,7 @@ namespace {
 #define AF_KBCL 2
 #endif
 // Batches hand limited points and cells to work lists of their own runs, as single runs do: with
-// the slow paths inline the point pass spilled 2.2 kB a thread (kBatchListBlocks blocks walk the
-// lists of each run).
-constexpr int kBatchListBlocks = 8;
+// the slow paths inline the point pass spilled 2.2 kB a thread.
 // the nz parts of the work of a tile (DoF classes, face directions) are items of their own, one part
 // after the other over all tiles
 #define AF_BATCH_LOOP(nz, call)                                   \
@@ -88,12 +86,42 @@ __global__ void kb_repair(const AfRun *__restrict__ runs, int nruns, double a, d
   if (runs[t].g.pp_on) b_repair(runs[t].d, runs[t].g, a, b);
   runs[t].d.st->npq = runs[t].d.st->ncq = 0;   // the next stage's work lists start empty
 }
-// the work lists of the runs, blockIdx.y the run: its cells, then its points
-__global__ void __launch_bounds__(kListThreads) kb_lists(const AfRun *__restrict__ runs, double a, double b) {
-  const AfRun *r = runs + blockIdx.y;
-  if (!r->g.pp_on) return;
-  b_cells_lists(r->d, r->g, blockIdx.x, gridDim.x);
-  b_points_slow<false>(r->d, r->g, a, b, blockIdx.x, gridDim.x);
+// The work lists of all runs in one grid: the cell lists of the runs one after the other, then their
+// point lists, cut into pieces that the blocks take in turn.  So one limited run among many, or a
+// batch of one, has the whole chip for its lists.  A list is cut finely (a half-warp per cell, four
+// lanes per point) while the lists of all runs, were they as long, would still fit the grid.
+// With 8 blocks for each run's lists a step of one limited 512 x 512 lattice took 33.2 ms (the same run
+// alone 3.5), with two of 768 x 768 79.6; now 3.6 and 14.6.
+template <class Count, class Piece>
+__device__ __forceinline__ void batch_pieces(int nruns, int fine, int &it, int &done, Count count, Piece piece) {
+  const int lane = threadIdx.x & 31;
+  for (int r0 = 0; r0 < nruns; r0 += 32) {
+    const int mine = r0 + lane < nruns ? count(r0 + lane) : 0;
+    for (unsigned m = __ballot_sync(0xffffffffu, mine > 0); m; m &= m - 1) {
+      const int q = __ffs(m) - 1, n = __shfl_sync(0xffffffffu, mine, q);
+      const bool shrt = (long long)n * nruns <= (long long)gridDim.x * fine;
+      const int np = shrt ? (n + fine - 1) / fine : (n + kListThreads - 1) / kListThreads;
+      for (; it < done + np; it += gridDim.x) piece(r0 + q, n, it - done, shrt);
+      done += np;
+    }
+  }
+}
+__global__ void __launch_bounds__(kListThreads) kb_lists(const AfRun *__restrict__ runs, int nruns, double a, double b) {
+  int it = blockIdx.x, done = 0;   // the block's next piece, the pieces of the lists passed
+  batch_pieces(
+      nruns, kListThreads / 16, it, done,
+      [&](int r) { return runs[r].g.pp_on ? list_length(&runs[r].d.st->ncq, runs[r].d.cq_cap) : 0; },
+      [&](int r, int n, int p, bool shrt) {
+        if (shrt) cells_box_short(runs[r].d, runs[r].g, n, p);
+        else cells_box_long(runs[r].d, runs[r].g, n, p * kListThreads, n);
+      });
+  batch_pieces(
+      nruns, kListThreads / 4, it, done,
+      [&](int r) { return runs[r].g.pp_on ? list_length(&runs[r].d.st->npq, runs[r].d.pq_cap) : 0; },
+      [&](int r, int n, int p, bool shrt) {
+        if (shrt) points_short<false>(runs[r].d, runs[r].g, a, b, n, p);
+        else points_long<false>(runs[r].d, runs[r].g, a, b, n, p * kListThreads + (int)threadIdx.x, n);
+      });
 }
 
 // ---------------------------------------------------------------------------
@@ -400,8 +428,7 @@ void af_launch_batch(int pass, const AfRun *runs, int nruns, const int4 *items, 
     case AF_K_CELLS: kb_cells<<<nblocks, block, 0, s>>>(runs, items, nitems, a, b); break;
     case AF_K_FINAL: kb_final<<<nblocks, block, 0, s>>>(runs, items, nitems, a, b); break;
     case AF_K_CELLS_SLOW:
-      for (int r0 = 0; r0 < nruns; r0 += 65535)   // blockIdx.y
-        kb_lists<<<dim3(kBatchListBlocks, nruns - r0 < 65535 ? nruns - r0 : 65535), kListThreads, 0, s>>>(runs + r0, a, b);
+      kb_lists<<<152 * 2, kListThreads, 0, s>>>(runs, nruns, a, b);
       break;
     case AF_K_REPAIR: kb_repair<<<(nruns + 127) / 128, 128, 0, s>>>(runs, nruns, a, b); break;
     default: break;

@@ -1868,18 +1868,13 @@ __device__ __forceinline__ void points_short(const AfDev &d, const AfGrid &g, do
   }
 }
 
+// Entries t, t + step, ... of a long list: one thread per point.
 template <bool GB>
-__device__ __forceinline__ void b_points_slow(const AfDev &d, const AfGrid &g, double a, double b, const int bid,
-                                              const int nb) {
-  const int n = min(*(volatile int *)&d.st->npq, d.pq_cap);
-  if (n <= (int)(nb * blockDim.x) >> 2) {
-    points_short<GB>(d, g, a, b, n, bid);
-    return;
-  }
+__device__ __forceinline__ void points_long(const AfDev &d, const AfGrid &g, double a, double b, int n, int t, int step) {
   const double dt = d.sc->dt;
   const size_t PS = (size_t)g.nxa * g.nya;
   int nlim = 0, nshr = 0, nbad = 0;
-  for (int t = bid * blockDim.x + threadIdx.x; t < n; t += nb * blockDim.x) {
+  for (; t < n; t += step) {
     const int packed = d.pq[t], cls = packed >> 28, op = packed & ((1 << 28) - 1);
     const int i = op % g.nxa, j = op / g.nxa;
     double UH[8], out[8], t1, t2;
@@ -1904,6 +1899,15 @@ __device__ __forceinline__ void b_points_slow(const AfDev &d, const AfGrid &g, d
     atomicAdd(&d.st->cnt[ST_NONADMISSIBLE], (unsigned long long)nbad);
     atomicOr(&d.st->err, AFE_NONADMISSIBLE);
   }
+}
+__device__ __forceinline__ int list_length(const int *count, int cap) { return min(*(const volatile int *)count, cap); }
+// The point list of a run, by block bid of nb
+template <bool GB>
+__device__ __forceinline__ void b_points_slow(const AfDev &d, const AfGrid &g, double a, double b, const int bid,
+                                              const int nb) {
+  const int n = list_length(&d.st->npq, d.pq_cap);
+  if (n <= (int)(nb * blockDim.x) >> 2) points_short<GB>(d, g, a, b, n, bid);
+  else points_long<GB>(d, g, a, b, n, (int)(bid * blockDim.x + threadIdx.x), (int)(nb * blockDim.x));
 }
 
 // Cells whose box was not certified: Sec. 3.2 step (2) over the list.  A block takes a
@@ -1972,19 +1976,15 @@ __device__ __forceinline__ void cells_box_short(const AfDev &d, const AfGrid &g,
 }
 
 constexpr int kListThreads = 128;   // threads of a block of the list passes
-__device__ __forceinline__ void b_cells_lists(const AfDev &d, const AfGrid &g, const int bid, const int nb) {
-  const int n = min(*(volatile int *)&d.st->ncq, d.cq_cap);
-  if (n <= (nb * kListThreads) >> 4) {
-    cells_box_short(d, g, n, bid);
-    return;
-  }
+// Batches base, base + step, ... of kListThreads cells of a long list, by one block.
+__device__ __forceinline__ void cells_box_long(const AfDev &d, const AfGrid &g, int n, int base, int step) {
   __shared__ double rect[kListThreads][4];
   __shared__ unsigned short vq[16 * kListThreads];   // cell of the batch << 4 | vertex
   __shared__ int nv;
   const double dt = d.sc->dt, cxf = dt * g.rdx, cyf = dt * g.rdy;
   const size_t PS = (size_t)g.nxa * g.nya;
   NewtonLog nl = {0, 0};
-  for (int base = bid * kListThreads; base < n; base += nb * kListThreads) {
+  for (; base < n; base += step) {
     if (threadIdx.x == 0) nv = 0;
     __syncthreads();
     const int t = base + threadIdx.x;
@@ -2029,6 +2029,13 @@ __device__ __forceinline__ void b_cells_lists(const AfDev &d, const AfGrid &g, c
     atomicAdd(&d.st->cnt[ST_NEWTON_SOLVES], (unsigned long long)nl.solves);
     atomicMax(&d.st->cnt[ST_NEWTON_MAXIT], (unsigned long long)nl.maxit);
   }
+}
+
+// The cell list of a run, by block bid of nb
+__device__ __forceinline__ void b_cells_lists(const AfDev &d, const AfGrid &g, const int bid, const int nb) {
+  const int n = list_length(&d.st->ncq, d.cq_cap);
+  if (n <= (nb * kListThreads) >> 4) cells_box_short(d, g, n, bid);
+  else cells_box_long(d, g, n, bid * kListThreads, nb * kListThreads);
 }
 
 // ---------------------------------------------------------------------------

@@ -48,3 +48,40 @@ def test_limited_runs(tuned):
     assert total["point_limited"] > 0 and total["lambda_lt1"] > 0
     assert af.af_batch_status(b)[1] == total
     af.af_batch_destroy(b)
+
+
+# One limited run has the whole chip for its lists in a batch too: alone, with a second one, and among
+# small runs that nothing limits.  The batch runs the same passes without the overlap of the two lists
+# with the others: less than twice the time is expected, three times is allowed.
+@pytest.mark.parametrize("others", ["none", "same", "small"])
+def test_one_limited_run_has_the_whole_chip(others):
+    big = ai.rarefaction_lattice(512, periods=16, kappa=0.0)
+    pbs = [big] + {"none": [], "same": [big], "small": [ai.orszag_tang(32)] * 15}[others]
+    U = {id(p): [torch.from_numpy(u).cuda() for u in ai.dofs(p)] for p in pbs}
+    b = af.af_batch_create([p.nx for p in pbs], [p.ny for p in pbs], [p.gamma for p in pbs], [p.bc for p in pbs])
+    runs = []
+    for r, p in enumerate(pbs):
+        af.af_batch_set_domain(b, r, p.x0, p.x1, p.y0, p.y1)
+        af.af_batch_set_params(b, r, cfl=p.cfl, kappa=p.kappa)
+        af.af_batch_set_state(b, r, U[id(p)])
+        runs.append(af.Solver(p.nx, p.ny, p.gamma, p.bc, domain=(p.x0, p.x1, p.y0, p.y1), cfl=p.cfl, kappa=p.kappa))
+        runs[-1].set_state(U[id(p)])
+
+    def best(step):
+        times = []
+        for _ in range(4):
+            t = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            t[0].record()
+            step()
+            t[1].record()
+            torch.cuda.synchronize()
+            times.append(t[0].elapsed_time(t[1]))
+        return min(times[1:])
+
+    t_batch = best(lambda: af.af_batch_step(b, 1))
+    t_runs = best(lambda: [s.step(False) for s in runs])
+    assert runs[0].status()[1]["point_limited"] > 100000
+    for s in runs:
+        s.close()
+    af.af_batch_destroy(b)
+    assert t_batch < 3.0 * t_runs
