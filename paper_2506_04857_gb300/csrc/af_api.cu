@@ -262,9 +262,8 @@ int af_create(int nx, int ny, double gamma, int bc, af_ctx **out) {
   }
   c->state_len = off;
   const size_t PS = (size_t)c->g.nxa * c->g.nya;
-  // stage work arrays, then the limiter work lists: points (3 PS entries: an int and 8
-  // doubles each), cells (PS entries: an int and 2 doubles each)
-  const size_t nwork = PS * (AF_NQA + 4 * AF_NQP + 8 + 4 + 2 * AF_NQF + 4 + 8 + 2) + PS * (24 + 2) + 2 * PS + 1 +
+  // stage work arrays, then the limiter work lists: an int for each of 3 PS points and PS cells
+  const size_t nwork = PS * (AF_NQA + 4 * AF_NQP + 8 + 4 + 2 * AF_NQF + 4 + 8 + 2) + 2 * PS + 1 +
                        (3 * af_quiet_tiles(c->g) + 7) / 8;
   int rc = AF_OK;
   for (int b = 0; b < 3; ++b) {
@@ -299,8 +298,6 @@ int af_create(int nx, int ny, double gamma, int bc, af_ctx **out) {
   c->dev.thy = w; w += PS;
   c->dev.pq_cap = (int)(3 * PS);
   c->dev.cq_cap = (int)PS;
-  c->dev.pqu = w; w += 24 * PS;
-  c->dev.cqe = w; w += 2 * PS;
   c->dev.pq = reinterpret_cast<int *>(w); w += (3 * PS + 1) / 2;
   c->dev.cq = reinterpret_cast<int *>(w); w += (PS + 1) / 2;
   c->dev.quiet = reinterpret_cast<unsigned char *>(w);

@@ -134,10 +134,10 @@ void build_tables(af_batch *b) {
         d.thy = w; w += PS;
         d.pq_cap = (int)(3 * PS);
         d.cq_cap = (int)PS;
-        d.pqu = w; w += 24 * PS;
-        d.cqe = w; w += 2 * PS;
-        d.pq = reinterpret_cast<int *>(w); w += (3 * PS + 1) / 2;
-        d.cq = reinterpret_cast<int *>(w); w += (PS + 1) / 2;
+        // the limiter work lists (an int for each of 3 PS points and PS cells) lie over theta, which
+        // the final pass writes when the lists are done
+        d.pq = reinterpret_cast<int *>(d.thx);
+        d.cq = d.pq + 3 * PS;
         d.sc = b->sc + r;
         d.st = b->st + r;
       }
@@ -253,9 +253,7 @@ int af_batch_create(int nruns, const int *nx, const int *ny, const double *gamma
   b->state_off.resize(nruns);
   b->work_off.resize(nruns);
   size_t st = 0, wk = 0;
-  // stage work arrays, then the limiter work lists (points: 8 doubles and an int each, three classes;
-  // cells: 2 doubles and an int)
-  const size_t per_point = AF_NQA + 4 * AF_NQP + 8 + 4 + 2 * AF_NQF + 4 + 8 + 2 + 24 + 2 + 2;
+  const size_t per_point = AF_NQA + 4 * AF_NQP + 8 + 4 + 2 * AF_NQF + 4 + 8 + 2;   // stage work arrays
   for (int r = 0; r < nruns; ++r) {
     fill_grid(b, r);
     const AfGrid &g = b->grid[r];
@@ -267,7 +265,7 @@ int af_batch_create(int nruns, const int *nx, const int *ny, const double *gamma
     }
     st += (off + 31) / 32 * 32;   // keep every run 256-byte aligned
     b->work_off[r] = wk;
-    wk += ((size_t)g.nxa * g.nya * per_point + 1 + 31) / 32 * 32;
+    wk += ((size_t)g.nxa * g.nya * per_point + 31) / 32 * 32;
   }
   b->state_total = st;
   int rc = AF_OK;

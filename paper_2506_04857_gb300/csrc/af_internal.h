@@ -94,11 +94,10 @@ struct AfDev {
   double *rec;            // when set: the stage writes its limiter coefficients here (AFC_* slots)
   const double *frz;      // when set: the stage takes its limiter coefficients from here (frozen branch)
   // work lists of the limiter slow paths:
-  // points whose update leaves the 1e-13 floors (packed class << 28 | index, and their
-  // high-order update, component-major), cells whose Sec. 3.2 box is not certified
-  // (index, eps_rho, eps_p)
+  // points whose update leaves the 1e-13 floors (packed class << 28 | index; their
+  // high-order update is in the output), cells whose Sec. 3.2 box is not certified (index;
+  // their eps_rho and eps_p are in the first two slots of lam)
   int *pq, *cq;
-  double *pqu, *cqe;
   int pq_cap, cq_cap;
   // quiet tiles (large grids): flags, deep flags and levels, a byte per tile of 32 x 4 index
   // points each; lev is set for the stages that use the levels

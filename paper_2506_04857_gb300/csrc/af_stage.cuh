@@ -917,13 +917,12 @@ __device__ __forceinline__ void b_point(const AfDev &d, const AfGrid &g, const i
         for (int k = 0; k < 8; ++k) acc[k] = out[k];
       }
     } else if (!clear_of_floor(acc, g)) {
-      // slow path in k_points_slow, over a dense list (the warp does not wait here)
+      // slow path in k_points_slow, over a dense list (the warp does not wait here); the high-order
+      // update waits there in the point's own place of the output
       const int slot = enqueue(d.st, &d.st->npq, d.pq_cap);
-      if (slot >= 0) {
-        d.pq[slot] = (cls << 28) | (int)op;
+      if (slot >= 0) d.pq[slot] = (cls << 28) | (int)op;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) d.pqu[(size_t)k * d.pq_cap + slot] = acc[k];
-      }
+      for (int k = 0; k < 8; ++k) uo[k * cs + oo] = acc[k];
       return;
     }
     if (!PL && d.rec) {
@@ -1493,11 +1492,9 @@ __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const i
           cell_source_limit(Ullf, dS, dtts, g, L1, sl, th_src, eps_rho, eps_p);
           nsrc += sl;
           const int slot = enqueue(d.st, &d.st->ncq, d.cq_cap);
-          if (slot >= 0) {
-            d.cq[slot] = (int)o;
-            d.cqe[2 * slot] = eps_rho;
-            d.cqe[2 * slot + 1] = eps_p;
-          }
+          if (slot >= 0) d.cq[slot] = (int)o;
+          d.lam[o] = eps_rho;   // until the list pass writes the cell's Lambda there
+          d.lam[PS + o] = eps_p;
           listed = true;
         }
 #pragma unroll
@@ -1848,9 +1845,10 @@ __device__ __forceinline__ void points_short(const AfDev &d, const AfGrid &g, do
     UL[k] = u;
   }
   if (!live || q) return;
+  const size_t cs = (size_t)g.ex[cls] * g.ey[cls], oo = (size_t)j * g.ex[cls] + i;
   double UH[8], out[8], t1, t2;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) UH[k] = d.pqu[(size_t)k * d.pq_cap + t];
+  for (int k = 0; k < 8; ++k) UH[k] = d.uo[cls][k * cs + oo];
   int lim, shr, bad;
   point_limit(g, UH, UL, out, lim, shr, bad, t1, t2);
   if (d.rec) {
@@ -1858,7 +1856,6 @@ __device__ __forceinline__ void points_short(const AfDev &d, const AfGrid &g, do
     d.rec[s1] = t1;
     d.rec[s1 + PS] = t2;
   }
-  const size_t cs = (size_t)g.ex[cls] * g.ey[cls], oo = (size_t)j * g.ex[cls] + i;
   rk_store(d.uo[cls] + oo, d.un[cls] + oo, cs, a, b, out);
   if (lim) atomicAdd(&d.st->cnt[ST_POINT_LIMITED], 1ull);
   if (shr) atomicAdd(&d.st->cnt[ST_SHRINK], 1ull);
@@ -1877,9 +1874,10 @@ __device__ __forceinline__ void points_long(const AfDev &d, const AfGrid &g, dou
   for (; t < n; t += step) {
     const int packed = d.pq[t], cls = packed >> 28, op = packed & ((1 << 28) - 1);
     const int i = op % g.nxa, j = op / g.nxa;
+    const size_t cs = (size_t)g.ex[cls] * g.ey[cls], oo = (size_t)j * g.ex[cls] + i;
     double UH[8], out[8], t1, t2;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) UH[k] = d.pqu[(size_t)k * d.pq_cap + t];
+    for (int k = 0; k < 8; ++k) UH[k] = d.uo[cls][k * cs + oo];
     int lim, shr, bad;
     point_pp<GB>(d, g, cls, i, j, UH, dt, out, lim, shr, bad, t1, t2);
     nlim += lim;
@@ -1890,7 +1888,6 @@ __device__ __forceinline__ void points_long(const AfDev &d, const AfGrid &g, dou
       d.rec[s1] = t1;
       d.rec[s1 + PS] = t2;
     }
-    const size_t cs = (size_t)g.ex[cls] * g.ey[cls], oo = (size_t)j * g.ex[cls] + i;
     rk_store(d.uo[cls] + oo, d.un[cls] + oo, cs, a, b, out);
   }
   if (nlim) atomicAdd(&d.st->cnt[ST_POINT_LIMITED], (unsigned long long)nlim);
@@ -1956,12 +1953,13 @@ __device__ __forceinline__ void cells_box_short(const AfDev &d, const AfGrid &g,
 #pragma unroll
   for (int k = 0; k < 8; ++k) L1[k] = d.lim1[k * PS + o];
   cell_H(d, g, i, j, cxf, cyf, H);
-  rect_rho(L1, H, d.cqe[2 * tt], LamRho);
+  const double eps_rho = d.lam[o], eps_p = d.lam[PS + o];
+  rect_rho(L1, H, eps_rho, LamRho);
   box_vertex(v, LamRho, H, A, D);
   for (int k = 0; k < 8; ++k) V[k] = L1[k] + D[k];
   NewtonLog nl = {0, 0};
   double r = 1.0;
-  if (live && pressure(V, g.gm1) < d.cqe[2 * tt + 1]) r = newton_root(L1, D, d.cqe[2 * tt + 1], g.gm1, nl);
+  if (live && pressure(V, g.gm1) < eps_p) r = newton_root(L1, D, eps_p, g.gm1, nl);
 #pragma unroll
   for (int I = 0; I < 4; ++I) {
     double m = ((v >> I) & 1) ? r * A[I] : INFINITY;
@@ -1978,7 +1976,7 @@ __device__ __forceinline__ void cells_box_short(const AfDev &d, const AfGrid &g,
 constexpr int kListThreads = 128;   // threads of a block of the list passes
 // Batches base, base + step, ... of kListThreads cells of a long list, by one block.
 __device__ __forceinline__ void cells_box_long(const AfDev &d, const AfGrid &g, int n, int base, int step) {
-  __shared__ double rect[kListThreads][4];
+  __shared__ double rect[kListThreads][5];           // Lambda^rho and eps_p of a cell of the batch
   __shared__ unsigned short vq[16 * kListThreads];   // cell of the batch << 4 | vertex
   __shared__ int nv;
   const double dt = d.sc->dt, cxf = dt * g.rdx, cyf = dt * g.rdy;
@@ -1994,8 +1992,9 @@ __device__ __forceinline__ void cells_box_long(const AfDev &d, const AfGrid &g, 
 #pragma unroll
       for (int k = 0; k < 8; ++k) L1[k] = d.lim1[k * PS + o];
       cell_H(d, g, i, j, cxf, cyf, H);
-      rect_rho(L1, H, d.cqe[2 * t], LamRho);
-      const double eps_p = d.cqe[2 * t + 1];
+      const double eps_rho = d.lam[o], eps_p = d.lam[PS + o];
+      rect_rho(L1, H, eps_rho, LamRho);
+      rect[threadIdx.x][4] = eps_p;
       for (int I = 0; I < 4; ++I) {
         rect[threadIdx.x][I] = LamRho[I];
         d.lam[I * PS + o] = LamRho[I];
@@ -2017,7 +2016,7 @@ __device__ __forceinline__ void cells_box_long(const AfDev &d, const AfGrid &g, 
       cell_H(d, g, i, j, cxf, cyf, H);
       for (int I = 0; I < 4; ++I) LamRho[I] = rect[tl][I];
       box_vertex(kk, LamRho, H, A, D);
-      const double r = newton_root(L1, D, d.cqe[2 * (base + tl) + 1], g.gm1, nl);
+      const double r = newton_root(L1, D, rect[tl][4], g.gm1, nl);
       for (int I = 0; I < 4; ++I)
         if ((kk >> I) & 1)
           atomicMin(reinterpret_cast<unsigned long long *>(d.lam + I * PS + o),

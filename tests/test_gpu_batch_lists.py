@@ -85,3 +85,17 @@ def test_one_limited_run_has_the_whole_chip(others):
         s.close()
     af.af_batch_destroy(b)
     assert t_batch < 3.0 * t_runs
+
+
+def test_memory_of_a_batch():
+    """What a batch holds per index point: three states (8 components of 4 classes) and 163 doubles of
+    stage work arrays; the limiter lists take none of their own."""
+    n = 1024
+    args = lambda m: ([m], [m], [1.4], [af.AF_BC_PERIODIC])   # noqa: E731
+    af.af_batch_destroy(af.af_batch_create(*args(8)))
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    b = af.af_batch_create(*args(n))
+    used = free - torch.cuda.mem_get_info()[0]
+    af.af_batch_destroy(b)
+    assert 0 < used <= n * n * (3 * 32 + 163) * 8 + (32 << 20)
