@@ -285,20 +285,31 @@ __device__ __forceinline__ void load8(const SV &v, int i, int j, double *U) {
   for (int k = 0; k < 8; ++k) U[k] = v(i, j, k);
 }
 
-// Whether component k of the eight points of cell (i, j) equals a bit for bit
-__device__ __forceinline__ bool same_nine(const SV &X, const SV &Y, const SV &C, int i, int ip, int j, int jp, int k,
-                                          double a) {
-  const unsigned long long b = bits(a);
-  return ((bits(X(i, j, k)) ^ b) | (bits(X(ip, j, k)) ^ b) | (bits(Y(i, j, k)) ^ b) | (bits(Y(i, jp, k)) ^ b) |
-          (bits(C(i, j, k)) ^ b) | (bits(C(ip, j, k)) ^ b) | (bits(C(i, jp, k)) ^ b) | (bits(C(ip, jp, k)) ^ b)) == 0;
+// Whether x and y are equal bit for bit, or zeros of either sign: the equality of uniform gas, here
+// and in the quiet tiles
+__device__ __forceinline__ bool same_value(double x, double y) {
+  return bits(x) == bits(y) || ((bits(x) | bits(y)) << 1) == 0;
 }
-// Whether all nine states of cell (i, j) are equal: its centre value is then that state exactly, not
+// Whether the energies of the eight points of cell (i, j) equal a, that of its average, bit for bit
+// (a zero energy, of either sign, is not that of a gas)
+__device__ __forceinline__ bool same_energy(const SV &X, const SV &Y, const SV &C, int i, int ip, int j, int jp,
+                                            double a) {
+  const unsigned long long b = bits(a);
+  return ((bits(X(i, j, 7)) ^ b) | (bits(X(ip, j, 7)) ^ b) | (bits(Y(i, j, 7)) ^ b) | (bits(Y(i, jp, 7)) ^ b) |
+          (bits(C(i, j, 7)) ^ b) | (bits(C(ip, j, 7)) ^ b) | (bits(C(i, jp, 7)) ^ b) | (bits(C(ip, jp, 7)) ^ b)) == 0;
+}
+// Whether all nine states of cell (i, j), whose energies are, are equal: its centre value is then that state exactly, not
 // within rounding, and uniform gas stays uniform bit for bit (quiet tiles).  Not inlined: the rare
 // case, and its loads would cost the point-data pass spills.
 __device__ __noinline__ bool uniform_cell(const AfDev &d, const AfGrid &g, int i, int ip, int j, int jp) {
   const SV A = sview(d.us[0], g, 0), X = sview(d.us[1], g, 1), Y = sview(d.us[2], g, 2), C = sview(d.us[3], g, 3);
-  for (int k = 0; k < 8; ++k)
-    if (!same_nine(X, Y, C, i, ip, j, jp, k, A(i, j, k))) return false;
+  for (int k = 0; k < 7; ++k) {
+    const double a = A(i, j, k);
+    if (!(same_value(X(i, j, k), a) && same_value(X(ip, j, k), a) && same_value(Y(i, j, k), a) &&
+          same_value(Y(i, jp, k), a) && same_value(C(i, j, k), a) && same_value(C(ip, j, k), a) &&
+          same_value(C(i, jp, k), a) && same_value(C(ip, jp, k), a)))
+      return false;
+  }
   return true;
 }
 
@@ -316,7 +327,7 @@ __device__ __forceinline__ bool centre_value(const AfDev &d, const AfGrid &g, in
   }
   // a cell whose nine states are equal has that state at its centre (the energies end the test
   // almost everywhere else)
-  if (same_nine(X, Y, C, i, ip, j, jp, 7, A[7]) && uniform_cell(d, g, i, ip, j, jp))
+  if (same_energy(X, Y, C, i, ip, j, jp, A[7]) && uniform_cell(d, g, i, ip, j, jp))
 #pragma unroll
     for (int k = 0; k < 8; ++k) uc[k] = A[k];
   const size_t PS = (size_t)g.nxa * g.nya, o = (size_t)j * g.nxa + i;
@@ -2056,10 +2067,6 @@ __device__ __forceinline__ void b_cells_lists(const AfDev &d, const AfGrid &g, c
 // 14.12 -> 14.3 ms for a step with its copies); the 2048 x 2048 blast, 1/6 of it disturbed, takes
 // 19.7 ms for two steps instead of 45.4.
 // ---------------------------------------------------------------------------
-// equal bit for bit, or zeros of either sign
-__device__ __forceinline__ bool same_value(double x, double y) {
-  return bits(x) == bits(y) || ((bits(x) | bits(y)) << 1) == 0;
-}
 __device__ __forceinline__ bool same_state(const AfDev &d, const AfGrid &g, int cls, int ia, int ja, int ib, int jb) {
   const SV C = sview(d.us[cls], g, cls);
   for (int k = 0; k < 8; ++k)

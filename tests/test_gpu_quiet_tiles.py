@@ -1,5 +1,7 @@
 """Quiet tiles: large grids whose gas is uniform outside a disturbance, against the same run
 without the levels (a batch; a short 1D grid), bitwise and with equal counters."""
+from fractions import Fraction as F
+
 import numpy as np
 import pytest
 
@@ -91,3 +93,46 @@ def test_1d_quiet_equals_short_grid(n, at, kappa):
     (L, cl), (S, cs) = states
     assert torch.equal(L[0][:, off:off + m], S[0]) and torch.equal(L[1][:, off:off + m + 1], S[1])
     assert cl == cs
+
+
+def centre_misses(v):
+    """Whether 36/16 v - 4 4/16 v - 4/16 v, rounded as the centre value is, is not v."""
+    r = float(F(-5, 4) * F(v))
+    return float(F(9, 4) * F(v) + F(r)) != v
+
+
+# Uniform gas whose zeros are of either sign, and whose centre value would not be the state itself
+# were it formed from the nine states: uniform bit for bit, so it takes the state, and the quiet
+# tiles and the others (here: a batch) agree.
+@pytest.mark.parametrize("nx,ny,bc", [(1025, 517, ai.PERIODIC), (1024, 516, ai.OUTFLOW)])
+def test_zeros_of_either_sign(nx, ny, bc):
+    rng = np.random.default_rng(1)
+    V = np.array([1.0, 0.3, -0.2, 0.0, 0.5, 0.4, 0.0, 3.0])
+    for k in (0, 1, 4, 7):
+        while not centre_misses(V[k]):
+            V[k] += 1e-3 * rng.random()
+    U = []
+    for ex, ey in ai.class_extents(nx, ny, bc):
+        u = np.empty((8, ey, ex))
+        for k in range(8):
+            u[k] = V[k]
+        for k in (3, 6):
+            u[k] = np.copysign(0.0, rng.random((ey, ex)) - 0.5)
+        u[7, ey // 2: ey // 2 + 9, ex // 2: ex // 2 + 9] += 0.01 * rng.random((9, 9))
+        U.append(torch.from_numpy(u).cuda())
+    s = af.Solver(nx, ny, 1.4, bc, kappa=1.0, cfl=0.9)
+    s.set_state(U)
+    s.stage(0, 2e-4)   # the forward-Euler stage leaves the state, and the tiles near the disturbance do too
+    for p in s.get_stage():
+        assert torch.equal(p[:, :248], torch.from_numpy(V).cuda()[:, None, None].expand_as(p[:, :248]))
+    s.set_state(U)
+    b = af.af_batch_create([nx], [ny], [1.4], [bc])
+    af.af_batch_set_params(b, 0, kappa=1.0, cfl=0.9)
+    af.af_batch_set_state(b, 0, U)
+    s.step(False)
+    af.af_batch_step(b, 1)
+    got = af.af_batch_get_state(b, 0, [torch.empty_like(u) for u in U])
+    for p, q in zip(s.get_state(), got):
+        assert torch.equal(p, q)
+    s.close()
+    af.af_batch_destroy(b)
