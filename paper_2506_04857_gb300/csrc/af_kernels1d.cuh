@@ -114,9 +114,10 @@ __device__ __noinline__ void point_pp1(const AfDev &d, const AfGrid &g, int f, c
 
 // P2 (1D): point update, its limiter and the RK combination; the sensor phi
 // parts: 1 the point, 2 the sensor values of cell f
-__device__ __forceinline__ void b1_points(const AfDev &d, const AfGrid &g, int f, double a, double b, int parts = 3) {
+__device__ __forceinline__ void b1_points(const AfDev &d, const AfGrid &g, int f, double a, double b, int parts = 3,
+                                          bool pois = false) {
   const size_t PS = (size_t)g.nxa;
-  const double dt = d.sc->dt;
+  const double dt = pois ? nan_value() : d.sc->dt;
   int nlim = 0, nshr = 0, nbad = 0;
   if ((parts & 1) && f < g.ex[1]) {
     const int fm = mface(f - 1, g.nx, g.bc), fp = mface(f + 1, g.nx, g.bc);
@@ -209,12 +210,12 @@ __device__ __noinline__ bool box_cert64_1d(const AfDev &d, const AfGrid &g, int 
   return box_certified(L1, D, g);
 }
 
-__device__ __forceinline__ void b1_cells(const AfDev &d, const AfGrid &g, int i, double a, double b) {
+__device__ __forceinline__ void b1_cells(const AfDev &d, const AfGrid &g, int i, double a, double b, bool pois = false) {
   const size_t PS = (size_t)g.nxa;
   int nlam = 0, ncfl = 0;
   NewtonLog nl = {0, 0};
   if (i < g.nx) {
-    const double dt = d.sc->dt, cxf = dt * g.rdx;
+    const double dt = pois ? nan_value() : d.sc->dt, cxf = dt * g.rdx;
     const int ip = mface(i + 1, g.nx, g.bc);
     const WV FX = wview(d.fx, g);
     const SV Ub = sview(d.us[0], g, 0);
@@ -487,7 +488,8 @@ __global__ void __launch_bounds__(128) k1_points(const __grid_constant__ AfDev d
                                                  double a, double b) {
   pass_begin();
   const int lev = level1(d), i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (blockIdx.y == 0 && lev > 0) {
+  const bool pois = lev > 0 && poisoned(d);
+  if (blockIdx.y == 0 && lev > 0 && !pois) {
     if (i < g.ex[1]) {
       double V[8];
       load8(sview(d.us[1], g, 1), i, 0, V);
@@ -495,7 +497,7 @@ __global__ void __launch_bounds__(128) k1_points(const __grid_constant__ AfDev d
     }
     return;
   }
-  if (blockIdx.y == 0 || lev <= 3) b1_points(d, g, i, a, b, 1 << blockIdx.y);
+  if (blockIdx.y == 0 || lev <= 3) b1_points(d, g, i, a, b, 1 << blockIdx.y, pois);
 }
 __global__ void __launch_bounds__(128) k1_faces(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g) {
   pass_begin();
@@ -505,25 +507,26 @@ __global__ void __launch_bounds__(128) k1_cells(const __grid_constant__ AfDev d,
                                                 double a, double b) {
   pass_begin();
   const int lev = level1(d), i = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool pois = lev > 0 && poisoned(d);
   if (lev > 0) {
     if (i < g.nx && threadIdx.x % 32 == 0 && quiet_cfl1(d, g, i))
       atomicAdd(&d.st->cnt[ST_CFL_VIOLATIONS], (unsigned long long)min(32, g.nx - i));
-    if (i < g.nx && lev == 1) {
+    if (i < g.nx && lev == 1 && !pois) {
       double V[8];
       load8(sview(d.us[0], g, 0), i, 0, V);
 #pragma unroll
       for (int k = 0; k < 8; ++k) d.lim1[(size_t)k * g.nxa + i] = V[k];
       d.lam[i] = d.lam[(size_t)g.nxa + i] = 1.0;
     }
-    return;
+    if (!pois) return;
   }
-  b1_cells(d, g, i, a, b);
+  b1_cells(d, g, i, a, b, pois);
 }
 __global__ void __launch_bounds__(128) k1_final(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                                 double a, double b) {
   pass_begin();
   const int lev = level1(d), i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (lev > 0) {
+  if (lev > 0 && !poisoned(d)) {
     if (i >= g.nx) return;
     double V[8];
     load8(sview(d.us[0], g, 0), i, 0, V);

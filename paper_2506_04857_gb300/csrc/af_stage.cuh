@@ -827,11 +827,17 @@ __device__ __forceinline__ void rk_store(double *out, const double *un, size_t c
 //   kQuiet: a plain stage with the levels of the quiet tiles.
 //   kStage: any stage.  kRhs: the semi-discrete right-hand side.
 enum { kStage = 0, kPlain = 1, kRhs = 2, kQuiet = 3 };
+// With a time step that is not finite (a NaN in the state, say), V + dt 0 is NaN and no tile is passed
+// over: its points, cells and averages run the ordinary code, with NaN for the step, since the
+// point data and faces of the tile have not been formed.
+__device__ __forceinline__ double nan_value() { return from_bits(0x7ff8000000000000ULL); }
+__device__ __forceinline__ bool poisoned(const AfDev &d) { return !finite_bits(d.sc->dt); }
 template <int cls, bool GB, bool UP, int K>
 __device__ __forceinline__ void b_point(const AfDev &d, const AfGrid &g, const int i, const int j, double a, double b,
                                         int &nlim, bool quiet) {
   constexpr bool PL = K == kPlain || K == kQuiet, RHS = K == kRhs;
-  if (K == kQuiet && quiet) {   // L(U) = 0: the RK combination of the state itself
+  const bool pois = K == kQuiet && quiet && poisoned(d);
+  if (K == kQuiet && quiet && !pois) {   // L(U) = 0: the RK combination of the state itself
     const size_t cs = (size_t)g.ex[cls] * g.ey[cls], oo = (size_t)j * g.ex[cls] + i;
     double v[8];
     load8(sview(d.us[cls], g, cls), i, j, v);
@@ -839,7 +845,7 @@ __device__ __forceinline__ void b_point(const AfDev &d, const AfGrid &g, const i
     return;
   }
   const size_t PS = (size_t)g.nxa * g.nya;
-  const double dt = RHS ? 1.0 : d.sc->dt;
+  const double dt = RHS ? 1.0 : (pois ? nan_value() : d.sc->dt);
   const double cxc = mul_i(dt, g.rdx), cyc = mul_i(dt, g.rdy);   // central differences
   const double cx = ldexp_i<-1>(cxc), cy = ldexp_i<-1>(cyc);      // the FVS lines carry a factor 1/2
   const int im = mface(i - 1, g.nx, g.bc), ip = mface(i + 1, g.nx, g.bc);
@@ -1314,12 +1320,12 @@ __device__ __forceinline__ void cell_H(const AfDev &d, const AfGrid &g, int i, i
 // PL: as in the point pass, with the positivity limiters on (ANY: on or off, by run)
 template <bool GB, bool PL, bool ANY = false>
 __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const int i, const int j, double a, double b,
-                                        int mode) {
+                                        int mode, bool pois = false) {
   const size_t PS = (size_t)g.nxa * g.nya;
   const size_t o = (size_t)j * g.nxa + i;
   int nsrc = 0, ncfl = 0;
   if (i < g.nx && j < g.ny) {
-    const double dt = !PL && mode == 1 ? 1.0 : d.sc->dt;
+    const double dt = !PL && mode == 1 ? 1.0 : (pois ? nan_value() : d.sc->dt);
     const int ip = mface(i + 1, g.nx, g.bc), jp = mface(j + 1, g.ny, g.bc);
     const SV X = sview(d.us[1], g, 1), Y = sview(d.us[2], g, 2), C = sview(d.us[3], g, 3);
     const WV PX = wview(d.pd[1], g), PY = wview(d.pd[2], g), PC = wview(d.pd[3], g), PZ = wview(d.pd[4], g);
@@ -2290,15 +2296,16 @@ __global__ void AF_LB_CL k_cells(const __grid_constant__ AfDev d, const __grid_c
   } else {
     const Tile t = tile();
     const int lev = PL ? tile_level(d) : 0;
-    if (lev > 0) quiet_cells(d, g, t, lev);
-    else b_cells<false, PL>(d, g, t.i, t.j, a, b, mode);
+    const bool pois = lev > 0 && poisoned(d);
+    if (lev > 0) quiet_cells(d, g, t, pois ? 5 : lev);
+    if (lev == 0 || pois) b_cells<false, PL>(d, g, t.i, t.j, a, b, mode, pois);
   }
 }
 __global__ void AF_LB_FN k_final(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                                double a, double b) {
   pass_begin();
   const int lev = tile_level(d);
-  if (lev > 0) quiet_final(d, g, AF_IJ, a, b, lev);
+  if (lev > 0 && !poisoned(d)) quiet_final(d, g, AF_IJ, a, b, lev);
   else b_final(d, g, AF_IJ, a, b);
 #ifdef AF_LAT
   if (last_block(&d.sc->ticket[1]) && threadIdx.x == 0) b_repair(d, g, a, b);

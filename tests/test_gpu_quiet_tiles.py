@@ -136,3 +136,40 @@ def test_zeros_of_either_sign(nx, ny, bc):
         assert torch.equal(p, q)
     s.close()
     af.af_batch_destroy(b)
+
+
+# A NaN anywhere makes the time step NaN and with it every degree of freedom, in the quiet tiles too;
+# the counters and the error are those of the run without tiles.
+@pytest.mark.parametrize("nx,ny,bc", [(1024, 516, ai.OUTFLOW)])
+def test_poisoned_state(nx, ny, bc):
+    U = [torch.from_numpy(u).cuda() for u in disturbed(nx, ny, bc, nx // 2, ny // 2, strong=False)]
+    U[3][7, ny // 2, nx // 2] = float("nan")
+    s = af.Solver(nx, ny, 1.4, bc, kappa=1.0)
+    s.set_state(U)
+    b = af.af_batch_create([nx], [ny], [1.4], [bc])
+    af.af_batch_set_params(b, 0, kappa=1.0)
+    af.af_batch_set_state(b, 0, U)
+    s.step(False)
+    af.af_batch_step(b, 1)
+    got = af.af_batch_get_state(b, 0, [torch.empty_like(u) for u in U])
+    for p, q in zip(s.get_state(), got):
+        assert bool(torch.isnan(p).all()) and bool(torch.isnan(q).all())
+    rc, cnt = s.status()
+    assert (rc, cnt) == tuple(af.af_batch_status(b)) and rc == af.AF_EBOUNDS   # the repair list overflowed
+    s.close()
+    af.af_batch_destroy(b)
+
+
+def test_poisoned_state_1d():
+    n = 1 << 20
+    P = ai.prim_to_cons([np.full(n + 1, v) for v in (1.0, 0.3, -0.2, 0.1, 0.5, 0.4, 0.2, 1.0)], 1.4)
+    A = np.ascontiguousarray(P[:, :-1])
+    P[7, n // 2] = np.nan
+    s = af.Solver1D(n, 1.4, af.AF_BC_OUTFLOW, domain=(0.0, n / 1024.0))
+    s.set_state([torch.from_numpy(u).cuda() for u in (A, P)])
+    s.step(False)
+    for p in s.get_state():
+        assert bool(torch.isnan(p).all())
+    rc, cnt = s.status()
+    assert rc == af.AF_EBOUNDS and cnt["nonadmissible"] >= 3 * (n + 1)
+    s.close()
