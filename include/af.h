@@ -325,7 +325,13 @@ enum { AF_K_POINTDATA = 0, AF_K_DT, AF_K_POINTS, AF_K_FACES, AF_K_CELLS, AF_K_FI
  * pair of CUDA events on its stream; enable = 0 stops, synchronises the
  * stream and writes, per kernel (AF_K_* order), the summed device time in
  * milliseconds to ms[AF_NKERNEL] and the number of launches to
- * launches[AF_NKERNEL] (either may be NULL). */
+ * launches[AF_NKERNEL] (either may be NULL).
+ * Grids of up to 1216 rows of 32 index points run some of these in one launch,
+ * which is what is reported: the time step within AF_K_POINTDATA, the repair
+ * within AF_K_FINAL, the point list within AF_K_CELLS_SLOW.  From 2^19 index
+ * points on AF_K_POINTDATA includes the passes that look for uniform gas
+ * before it.  The point list of a larger grid runs on a second stream beside
+ * AF_K_FACES and AF_K_CELLS: their times overlap. */
 int af_timing(af_ctx *ctx, int enable, double *ms, long long *launches);
 
 /* Message of the last error on this context ("" when none). */
@@ -456,7 +462,9 @@ int af1d_step(af1d_ctx *ctx, double *dt_used, int on_device);
 int af1d_status(af1d_ctx *ctx, long long *counters, int reset);
 const char *af1d_last_error(const af1d_ctx *ctx);
 /* Per-kernel device timing of the 1D stages, as af_timing (the AF_K_* ids name
- * the 1D kernels of the same passes). */
+ * the 1D kernels of the same passes).  A grid of up to 4096 indices runs a
+ * step in one launch; while it is timed it runs pass by pass, with the same
+ * results, in more time than untimed. */
 int af1d_timing(af1d_ctx *ctx, int enable, double *ms, long long *launches);
 void af1d_destroy(af1d_ctx *ctx);
 

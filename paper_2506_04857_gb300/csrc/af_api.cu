@@ -163,6 +163,7 @@ void bind_ptrs(af_ctx *c, const double *n, const double *st, double *o) {
 // One stage: P1..P5 on the bound buffers.  keep_pd: the point data of every DoF is used after
 // the stage (the adjoint), so no tile is passed over.
 void run_stage(af_ctx *c, double a, double b, int reduce_dt, bool keep_pd = false) {
+  const bool small = af_small_grid(c->g);
   c->dev.lev = nullptr;
   if (!keep_pd && af_quiet_grid(c->g) && !c->dev.rec && !c->dev.frz) {
     c->dev.lev = c->dev.quiet + 2 * af_quiet_tiles(c->g);
@@ -172,8 +173,9 @@ void run_stage(af_ctx *c, double a, double b, int reduce_dt, bool keep_pd = fals
     if (c->dev.lev) af_launch_quiet(c->dev, c->g, c->stream);
     af_launch_pointdata(c->dev, c->g, reduce_dt, c->stream);
   });
+  if (reduce_dt && !small) TIMED(AF_K_DT, af_launch_dt(c->dev, c->g, c->stream));
   TIMED(AF_K_POINTS, af_launch_points(c->dev, c->g, a, b, 0, c->stream));
-  const bool lists = c->g.pp_on && !c->dev.frz, small = af_small_grid(c->g);
+  const bool lists = c->g.pp_on && !c->dev.frz;
   if (lists && !small) {
     // the point list: only the next stage reads what it writes, so it runs on the
     // second stream beside the face and cell passes and joins at the end of the stage
@@ -188,6 +190,7 @@ void run_stage(af_ctx *c, double a, double b, int reduce_dt, bool keep_pd = fals
   if (lists && small) TIMED(AF_K_CELLS_SLOW, af_lat_lists(c->dev, c->g, a, b, c->stream));
   else if (lists) TIMED(AF_K_CELLS_SLOW, af_launch_cells_slow(c->dev, c->g, c->stream));
   if (c->g.pp_on) TIMED(AF_K_FINAL, af_launch_final(c->dev, c->g, a, b, c->stream));
+  if (c->g.pp_on && !small) TIMED(AF_K_REPAIR, af_launch_repair(c->dev, c->g, a, b, c->stream));
   if (lists && !small) cudaStreamWaitEvent(c->stream, c->ev_join, 0);
   c->dev.lev = nullptr;   // the levels are those of this stage's input
 }
@@ -429,6 +432,7 @@ int af_dt(af_ctx *c, double *dt_out, int on_device) {
   CK(cudaSetDevice(c->device), "set device");
   bind_states(c, c->cur, c->cur, (c->cur + 1) % 3);
   af_launch_pointdata(c->dev, c->g, 1, c->stream);
+  if (!af_small_grid(c->g)) af_launch_dt(c->dev, c->g, c->stream);
   CK(cudaGetLastError(), "dt launch");
   if (dt_out) {
     CK(cudaMemcpyAsync(dt_out, &c->sc->dt, sizeof(double), on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,

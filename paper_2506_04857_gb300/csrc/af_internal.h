@@ -112,13 +112,16 @@ struct AfRun {
   AfGrid g;
 };
 
-// kernel launchers (af_kernels.cu).  The point-data pass forms dt too when reduce_dt is set;
-// the final pass also runs the repair list.
+// kernel launchers (af_kernels.cu).  On small grids (af_small_grid) the point-data pass forms dt
+// too when reduce_dt is set, and the final pass runs the repair list; on larger ones these are
+// launches of their own.
 void af_launch_pointdata(const AfDev &d, const AfGrid &g, int reduce_dt, cudaStream_t s);
 void af_launch_points(const AfDev &d, const AfGrid &g, double a, double b, int mode, cudaStream_t s);
 void af_launch_faces(const AfDev &d, const AfGrid &g, int mode, cudaStream_t s);
 void af_launch_cells(const AfDev &d, const AfGrid &g, double a, double b, int mode, cudaStream_t s);
 void af_launch_final(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s);
+void af_launch_dt(const AfDev &d, const AfGrid &g, cudaStream_t s);
+void af_launch_repair(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s);
 // the same passes compiled for small grids (af_kernels_lat.cu)
 void af_lat_pointdata(const AfDev &d, const AfGrid &g, int reduce_dt, cudaStream_t s);
 void af_lat_points(const AfDev &d, const AfGrid &g, double a, double b, int mode, cudaStream_t s);

@@ -360,6 +360,10 @@ void af_launch_final(const AfDev &d, const AfGrid &g, double a, double b, cudaSt
   if (af_small_grid(g)) af_lat_final(d, g, a, b, s);
   else launch_final(d, g, a, b, s);
 }
+void af_launch_dt(const AfDev &d, const AfGrid &g, cudaStream_t s) { pass(k_dt, 1, 32, s, d, g); }
+void af_launch_repair(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s) {
+  pass(k_repair, 1, 32, s, d, g, a, b);
+}
 int af_divb_nblocks(const AfGrid &g) { const dim3 b = grid2(g.nx, g.ny); return (int)(b.x * b.y); }
 int af_diag_nblocks(const AfGrid &g) { const dim3 b = grid2(g.nxa, g.nya); return (int)(b.x * b.y); }
 void af_launch_diag(const AfDev &d, const AfGrid &g, double *partials, double *out, cudaStream_t s) {

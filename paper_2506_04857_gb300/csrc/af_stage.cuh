@@ -2385,9 +2385,6 @@ void launch_quiet(const AfDev &d, const AfGrid &g, cudaStream_t s) {
 void launch_pointdata(const AfDev &d, const AfGrid &g, int reduce_dt, cudaStream_t s) {
   const Shape h = shape(g.nxa, g.nya, 5);
   pass(k_pointdata, h.g, h.b, s, d, g, reduce_dt);
-#ifndef AF_LAT
-  if (reduce_dt) pass(k_dt, 1, 32, s, d, g);
-#endif
 }
 void launch_points(const AfDev &d, const AfGrid &g, double a, double b, int mode, cudaStream_t s) {
   const Shape h = shape(g, g.nxa, g.nya, mode != 1 && g.kappa != 0.0 ? 4 : 3);
@@ -2423,9 +2420,6 @@ void launch_cells(const AfDev &d, const AfGrid &g, double a, double b, int mode,
 void launch_final(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s) {
   const Shape h = shape(g.nx, g.ny, 1);
   pass(k_final, h.g, h.b, s, d, g, a, b);
-#ifndef AF_LAT
-  pass(k_repair, 1, 32, s, d, g, a, b);
-#endif
 }
 // both lists in one launch (a stage of a small grid)
 void launch_lists(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s) {

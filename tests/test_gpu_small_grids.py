@@ -62,3 +62,22 @@ def test_limiter_lists(n, periods):
         assert cnt[name] == ref[name], (name, cnt[name], ref[name])
     assert cnt["lambda_lt1"] > 0
     s.close()
+
+
+# af_timing reports what is launched, kernel by kernel: two steps (six stages) of a large grid have
+# launches of their own for everything, of a small one three kernels hold more than one part
+@pytest.mark.parametrize("n", [64, 256])
+def test_timing_counts_every_launch(n):
+    pb = ai.random_smooth(n, n, seed=1, amp=0.3)
+    s = af.Solver(n, n, pb.gamma, pb.bc, domain=(pb.x0, pb.x1, pb.y0, pb.y1), kappa=1.0)
+    s.set_state([torch.from_numpy(u).cuda() for u in ai.dofs(pb)])
+    s.timing(True)
+    for _ in range(2):
+        s.step(False)
+    t = s.timing(False)
+    s.close()
+    own = 0 if n == 64 else 6
+    want = {"k_pointdata": 6, "k_dt": own // 3, "k_points": 6, "k_faces": 6, "k_cells": 6, "k_final": 6, "k_repair": own,
+            "k_points_slow": own, "k_cells_slow": 6}
+    assert {k: v[1] for k, v in t.items()} == want
+    assert all((v[0] > 0.0) == (v[1] > 0) for v in t.values())
