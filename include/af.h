@@ -462,7 +462,7 @@ int af1d_step(af1d_ctx *ctx, double *dt_used, int on_device);
 int af1d_status(af1d_ctx *ctx, long long *counters, int reset);
 const char *af1d_last_error(const af1d_ctx *ctx);
 /* Per-kernel device timing of the 1D stages, as af_timing (the AF_K_* ids name
- * the 1D kernels of the same passes).  A grid of up to 4096 indices runs a
+ * the 1D kernels of the same passes).  A grid of up to 2048 indices runs a
  * step in one launch; while it is timed it runs pass by pass, with the same
  * results, in more time than untimed. */
 int af1d_timing(af1d_ctx *ctx, int enable, double *ms, long long *launches);

@@ -126,12 +126,6 @@ void bind_stage1(af1d_ctx *c, int s) {
 #ifndef AF_QUIET1_MIN
 #define AF_QUIET1_MIN (1 << 20)
 #endif
-// Up to 4096 indices a step is one launch of a 16-CTA cluster: the passes then cost a cluster barrier
-// each instead of a launch, on 16 SMs instead of 152 (20 steps: 800 cells 4240 us in passes, 1903 in
-// the cluster; 8000 cells 4237 in passes, 6340 in the cluster).
-#ifndef AF_STEP1D_MAX
-#define AF_STEP1D_MAX 4096
-#endif
 // Stages s0..s1 of a step
 int stages1(af1d_ctx *c, int s0, int s1, int reduce_dt) {
   AfDev d[3];
@@ -225,7 +219,7 @@ int af1d_create(int n, double gamma, int bc, af1d_ctx **out) {
   c->dev.quiet = reinterpret_cast<unsigned char *>(w);
   c->dev.sc = c->sc;
   c->dev.st = c->st;
-  c->cluster = c->nf <= AF_STEP1D_MAX ? af_lat_step1d_cluster(c->nf) : 0;
+  c->cluster = af_lat_step1d_cluster(c->nf);
   c->cur = 0;
   c->next_stage = 0;
   *out = c;

@@ -571,10 +571,14 @@ cudaLaunchConfig_t step_config(int n, int cs, cudaLaunchAttribute *at, cudaStrea
 }
 }  // namespace
 
-// The cluster size of k1_step on the current device for n indices: 16, else 8, else 0 (no cluster fits)
+// The cluster size of k1_step on the current device for n indices: 16, else 8, else 0 (no such cluster
+// fits, or it has fewer threads of a role than there are indices).  In the cluster a pass costs a
+// barrier instead of a launch, on 16 SMs instead of 152: us a step of smooth data, cluster and pass by
+// pass, 800 cells 86 and 118, 2047 99 and 116; with a second round of indices 2300 155 and 120, 4095
+// 156 and 128 (blast 273 and 295 at 2047, 333 and 315 at 4095).
 int af_lat_step1d_cluster(int n) {
   cudaFuncSetAttribute(k1_step, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  for (int cs = 16; cs >= 8; cs /= 2) {
+  for (int cs = 16; cs >= 8 && n <= cs * kStepThreads; cs /= 2) {
     cudaLaunchAttribute at;
     cudaLaunchConfig_t c = step_config(n, cs, &at, nullptr);
     int k = 0;

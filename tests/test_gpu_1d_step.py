@@ -45,3 +45,28 @@ def test_step_equals_passes(n, bc, kappa, pp_on):
     assert a.status()[1] == b.status()[1]
     a.close()
     b.close()
+
+
+# Beyond one index per thread (16 CTAs of 128) a second round of indices costs more than the launches it
+# saves: the step of 3000 cells runs pass by pass, in little more time than that of 2047.  (In two
+# rounds: 1.57 times; pass by pass both: 1.05; a launch for each pass against one: at most 1.25.)
+def test_longer_grids_do_not_take_a_second_round():
+    t = []
+    for n in (2047, 3000):
+        x = np.linspace(0.0, 1.0, n + 1)
+        w = [1.0 + 0.1 * np.sin(2.0 * np.pi * x)] + [np.full(n + 1, v) for v in (0.3, -0.2, 0.1, 0.5, 0.4, 0.2, 1.0)]
+        P = ai.prim_to_cons(w, 1.4)
+        s = af.Solver1D(n, 1.4, af.AF_BC_OUTFLOW, kappa=1.0)
+        s.set_state([torch.from_numpy(np.ascontiguousarray(u)).cuda() for u in (0.5 * (P[:, :-1] + P[:, 1:]), P)])
+        best = 1e9
+        for _ in range(5):
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            e[0].record()
+            for _ in range(20):
+                s.step(False)
+            e[1].record()
+            torch.cuda.synchronize()
+            best = min(best, e[0].elapsed_time(e[1]))
+        t.append(best)
+        s.close()
+    assert t[1] < 1.4 * t[0]
