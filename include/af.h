@@ -330,8 +330,9 @@ enum { AF_K_POINTDATA = 0, AF_K_DT, AF_K_POINTS, AF_K_FACES, AF_K_CELLS, AF_K_FI
  * which is what is reported: the time step within AF_K_POINTDATA, the repair
  * within AF_K_FINAL, the point list within AF_K_CELLS_SLOW.  From 2^19 index
  * points on AF_K_POINTDATA includes the passes that look for uniform gas
- * before it.  The point list of a larger grid runs on a second stream beside
- * AF_K_FACES and AF_K_CELLS: their times overlap. */
+ * before it.  A short point list of a larger grid runs on a second stream
+ * beside AF_K_FACES and AF_K_CELLS (AF_K_POINTS_SLOW: their times overlap), a
+ * long one within AF_K_CELLS_SLOW. */
 int af_timing(af_ctx *ctx, int enable, double *ms, long long *launches);
 
 /* Message of the last error on this context ("" when none). */

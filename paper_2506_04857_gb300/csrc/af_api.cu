@@ -177,9 +177,9 @@ void run_stage(af_ctx *c, double a, double b, int reduce_dt, bool keep_pd = fals
   TIMED(AF_K_POINTS, af_launch_points(c->dev, c->g, a, b, 0, c->stream));
   const bool lists = c->g.pp_on && !c->dev.frz;
   if (lists && !small) {
-    // the point list: only the next stage reads what it writes, so it runs on the
+    // a short point list: only the next stage reads what it writes, so it runs on the
     // second stream beside the face and cell passes and joins at the end of the stage
-    // (a short list would otherwise cost the latency of one thread's slow path)
+    // (it would otherwise cost the latency of one thread's slow path)
     cudaEventRecord(c->ev_fork, c->stream);
     cudaStreamWaitEvent(c->lstream, c->ev_fork, 0);
     TIMED_ON(c->lstream, AF_K_POINTS_SLOW, af_launch_points_slow(c->dev, c->g, a, b, c->lstream));
@@ -187,8 +187,7 @@ void run_stage(af_ctx *c, double a, double b, int reduce_dt, bool keep_pd = fals
   }
   TIMED(AF_K_FACES, af_launch_faces(c->dev, c->g, 0, c->stream));
   TIMED(AF_K_CELLS, af_launch_cells(c->dev, c->g, a, b, 0, c->stream));
-  if (lists && small) TIMED(AF_K_CELLS_SLOW, af_lat_lists(c->dev, c->g, a, b, c->stream));
-  else if (lists) TIMED(AF_K_CELLS_SLOW, af_launch_cells_slow(c->dev, c->g, c->stream));
+  if (lists) TIMED(AF_K_CELLS_SLOW, af_launch_lists(c->dev, c->g, a, b, c->stream));
   if (c->g.pp_on) TIMED(AF_K_FINAL, af_launch_final(c->dev, c->g, a, b, c->stream));
   if (c->g.pp_on && !small) TIMED(AF_K_REPAIR, af_launch_repair(c->dev, c->g, a, b, c->stream));
   if (lists && !small) cudaStreamWaitEvent(c->stream, c->ev_join, 0);

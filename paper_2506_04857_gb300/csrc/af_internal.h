@@ -128,15 +128,16 @@ void af_lat_points(const AfDev &d, const AfGrid &g, double a, double b, int mode
 void af_lat_faces(const AfDev &d, const AfGrid &g, int mode, cudaStream_t s);
 void af_lat_cells(const AfDev &d, const AfGrid &g, double a, double b, int mode, cudaStream_t s);
 void af_lat_final(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s);
-void af_lat_lists(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s);   // both work lists
+void af_lat_lists(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s);
 bool af_small_grid(const AfGrid &g);   // which build the launchers below take
 // levels of the quiet tiles of the stage input; af_quiet_grid: whether a grid's stages use them
 void af_launch_quiet(const AfDev &d, const AfGrid &g, cudaStream_t s);
 bool af_quiet_grid(const AfGrid &g);
 inline size_t af_quiet_tiles(const AfGrid &g) { return (size_t)((g.nxa + 31) / 32) * ((g.nya + 3) / 4); }
-// the limiter slow paths over the work lists the point and cell passes filled
+// the limiter slow paths over the work lists the point and cell passes filled: a short point list
+// of a large grid, and everything else
 void af_launch_points_slow(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s);
-void af_launch_cells_slow(const AfDev &d, const AfGrid &g, cudaStream_t s);
+void af_launch_lists(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s);
 float af_run_fp64_probe(cudaStream_t s, double *flops);
 // point data of the inflow state U (device, 8 doubles) into out (8 + AF_NQP + AF_NQA doubles)
 void af_launch_inflow_pd(const AfGrid &g, const double *U, double *out, cudaStream_t s);

@@ -376,13 +376,13 @@ void af_launch_divb(const AfDev &d, const AfGrid &g, double *partials, double *o
   k_divb<<<b, dim3(32, 4), 0, s>>>(d, g, partials);
   k_divb_sum<<<1, 256, 0, s>>>(partials, (int)(b.x * b.y), out);
 }
-// a fixed grid of 4 blocks per SM walks the list
 void af_launch_points_slow(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s) {
-  if (g.special) pass(k_points_slow<true>, 152 * 4, kListThreads, s, d, g, a, b);
-  else pass(k_points_slow<false>, 152 * 4, kListThreads, s, d, g, a, b);
+  if (g.special) pass(k_points_slow<true>, kShortBlocks, kListThreads, s, d, g, a, b);
+  else pass(k_points_slow<false>, kShortBlocks, kListThreads, s, d, g, a, b);
 }
-void af_launch_cells_slow(const AfDev &d, const AfGrid &g, cudaStream_t s) {
-  pass(k_cells_slow, 152 * 4, kListThreads, s, d, g);
+void af_launch_lists(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s) {
+  if (af_small_grid(g)) af_lat_lists(d, g, a, b, s);
+  else launch_lists(d, g, a, b, s);
 }
 float af_run_fp64_probe(cudaStream_t s, double *flops) {
   int dev = 0, sms = 0;

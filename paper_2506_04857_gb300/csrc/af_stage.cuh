@@ -1822,10 +1822,10 @@ __device__ __forceinline__ bool frame_tile(const AfGrid &g, int nx, Tile &t) {
 // ---- limiter slow paths over the work lists (single runs) -------------------
 // Points whose high-order update left the floors: Sec. 3.3 LLF state, scaling
 // limiter and Remark 4.1 shrink, then the RK combination.
-// A short list (at most one point per four threads of the grid): four lanes per point, each with one
-// neighbour and its LLF flux, so the latency is that of one flux instead of four in a row.  The sums
-// are those of point_llf_state, so the results are too.  A few limited points of a 399 x 401 run:
-// 140 -> 100 us beside the face pass; 160 x 128, both lists in one launch: 50 -> 32 us.
+// A short list: four lanes per point, each with one neighbour and its LLF flux, so the latency is that
+// of one flux instead of four in a row.  The sums are those of point_llf_state, so the results are
+// too.  A few limited points of a 399 x 401 run: 140 -> 100 us beside the face pass; 160 x 128, both
+// lists in one launch: 50 -> 32 us.
 template <bool GB>
 __device__ __forceinline__ void points_short(const AfDev &d, const AfGrid &g, double a, double b, int n, const int bid) {
   const int t = (int)(bid * blockDim.x + threadIdx.x) >> 2, q = threadIdx.x & 3, lane0 = threadIdx.x & 28;
@@ -1915,14 +1915,12 @@ __device__ __forceinline__ void points_long(const AfDev &d, const AfGrid &g, dou
   }
 }
 __device__ __forceinline__ int list_length(const int *count, int cap) { return min(*(const volatile int *)count, cap); }
-// The point list of a run, by block bid of nb
-template <bool GB>
-__device__ __forceinline__ void b_points_slow(const AfDev &d, const AfGrid &g, double a, double b, const int bid,
-                                              const int nb) {
-  const int n = list_length(&d.st->npq, d.pq_cap);
-  if (n <= (int)(nb * blockDim.x) >> 2) points_short<GB>(d, g, a, b, n, bid);
-  else points_long<GB>(d, g, a, b, n, (int)(bid * blockDim.x + threadIdx.x), (int)(nb * blockDim.x));
-}
+// A list is short up to one warp of eight points for each of the 608 schedulers.  On a large grid a
+// short one runs beside the face and cell passes: it is one long latency and few instructions.  A long
+// one is bound by the FP64 pipe, like the passes it would run beside, and delays them by its blocks'
+// registers; it goes with the cell list, after them (a step of a limited 224 x 224 lattice 1.29 ms
+// beside them, 0.92 after; 256 x 256 1.20 and 1.05; 512 x 512 3.52 and 3.17).
+constexpr int kShortBlocks = 152, kShortPoints = kShortBlocks * 32;
 
 // Cells whose box was not certified: Sec. 3.2 step (2) over the list.  A block takes a
 // batch of listed cells.  A (one thread per cell): the rectangle R_rho; Lambda starts at
@@ -2315,26 +2313,31 @@ __global__ void k_repair(const __grid_constant__ AfDev d, const __grid_constant_
   pass_begin();
   if (threadIdx.x == 0 && blockIdx.x == 0) b_repair(d, g, a, b);
 }
-// The list passes: a fixed grid walks the lists.  Large grids run the point list on a
-// second stream beside the face and cell passes; small grids run both lists in one launch.
+// The list passes: a fixed grid walks the lists.  Both run in one launch, but for a short point list
+// of a large grid, which runs on a second stream beside the face and cell passes (k_points_slow).
 template <bool GB>
 __global__ void __launch_bounds__(kListThreads) k_points_slow(const __grid_constant__ AfDev d,
                                                               const __grid_constant__ AfGrid g, double a, double b) {
   pass_begin();
-  b_points_slow<GB>(d, g, a, b, blockIdx.x, gridDim.x);
-}
-__global__ void __launch_bounds__(kListThreads) k_cells_slow(const __grid_constant__ AfDev d,
-                                                             const __grid_constant__ AfGrid g) {
-  pass_begin();
-  b_cells_lists(d, g, blockIdx.x, gridDim.x);
+  const int n = list_length(&d.st->npq, d.pq_cap);
+  if (n <= kShortPoints) points_short<GB>(d, g, a, b, n, blockIdx.x);
 }
 template <bool GB>
 __global__ void __launch_bounds__(kListThreads) k_lists(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                                         double a, double b) {
   pass_begin();
   const int nb = (int)gridDim.x / 2, bid = (int)blockIdx.x;
-  if (bid < nb) b_cells_lists(d, g, bid, nb);
-  else b_points_slow<GB>(d, g, a, b, bid - nb, nb);
+  if (bid < nb) {
+    b_cells_lists(d, g, bid, nb);
+    return;
+  }
+  const int n = list_length(&d.st->npq, d.pq_cap);
+  if (n > kShortPoints)
+    points_long<GB>(d, g, a, b, n, (bid - nb) * kListThreads + (int)threadIdx.x, nb * kListThreads);
+#ifdef AF_LAT
+  else
+    points_short<GB>(d, g, a, b, n, bid - nb);
+#endif
 }
 
 
@@ -2421,10 +2424,15 @@ void launch_final(const AfDev &d, const AfGrid &g, double a, double b, cudaStrea
   const Shape h = shape(g.nx, g.ny, 1);
   pass(k_final, h.g, h.b, s, d, g, a, b);
 }
-// both lists in one launch (a stage of a small grid)
+// the lists, half the blocks each (small grids: a short point list included)
+#ifdef AF_LAT
+constexpr int kListBlocks = kShortBlocks;
+#else
+constexpr int kListBlocks = 152 * 4;
+#endif
 void launch_lists(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s) {
-  if (g.special) pass(k_lists<true>, 152 * 2, kListThreads, s, d, g, a, b);
-  else pass(k_lists<false>, 152 * 2, kListThreads, s, d, g, a, b);
+  if (g.special) pass(k_lists<true>, 2 * kListBlocks, kListThreads, s, d, g, a, b);
+  else pass(k_lists<false>, 2 * kListBlocks, kListThreads, s, d, g, a, b);
 }
 
 }  // namespace

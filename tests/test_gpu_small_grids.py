@@ -81,3 +81,27 @@ def test_timing_counts_every_launch(n):
             "k_points_slow": own, "k_cells_slow": 6}
     assert {k: v[1] for k, v in t.items()} == want
     assert all((v[0] > 0.0) == (v[1] > 0) for v in t.values())
+
+
+# A long point list does not delay the passes: a step of the smaller of two limited grids is the shorter
+# one (about 0.8 by its points).
+def test_a_smaller_limited_grid_is_faster():
+    t = []
+    for n in (224, 256):
+        pb = ai.rarefaction_lattice(n, periods=n // 32, kappa=0.0)
+        s = af.Solver(n, n, pb.gamma, pb.bc, domain=(pb.x0, pb.x1, pb.y0, pb.y1), cfl=pb.cfl, kappa=0.0)
+        s.set_state([torch.from_numpy(u).cuda() for u in ai.dofs(pb)])
+        for _ in range(6):
+            s.step(False)
+        best = 1e9
+        for _ in range(3):
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            e[0].record()
+            for _ in range(5):
+                s.step(False)
+            e[1].record()
+            torch.cuda.synchronize()
+            best = min(best, e[0].elapsed_time(e[1]))
+        t.append(best)
+        s.close()
+    assert t[0] < t[1]
