@@ -614,11 +614,7 @@ __device__ __forceinline__ void adj_point(const AfDev &d, const AfGrid &g, const
 // blockIdx.z: 0 x-faces, 1 y-faces, 2 corners, 3 cell centres
 // A2 compiled for 4 resident blocks of 128 threads (128 registers): 3 % faster than
 // the compiler's 166 registers on the 256x256 adjoint workload
-#ifndef AF_MINB_ADJ2
-#define AF_MINB_ADJ2 4
-#endif
-#define AF_LB_ADJ2 __launch_bounds__(128, AF_MINB_ADJ2)
-__global__ void AF_LB_ADJ2 k_adj2(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
+__global__ void __launch_bounds__(128, 4) k_adj2(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                               const __grid_constant__ Vec4 v, const double *a,
                                               const __grid_constant__ OVec4 tp, double *zc, const double *co) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;

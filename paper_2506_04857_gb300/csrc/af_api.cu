@@ -167,7 +167,7 @@ void run_stage(af_ctx *c, double a, double b, int reduce_dt, bool keep_pd = fals
   c->dev.lev = nullptr;
   if (!keep_pd && af_quiet_grid(c->g) && !c->dev.rec && !c->dev.frz) {
     c->dev.lev = c->dev.quiet + 2 * af_quiet_tiles(c->g);
-    c->dev.ntx = (c->g.nxa + 31) / 32;
+    c->dev.ntx = af_tiles_x(c->g);
   }
   TIMED(AF_K_POINTDATA, {
     if (c->dev.lev) af_launch_quiet(c->dev, c->g, c->stream);

@@ -122,10 +122,6 @@ void bind_stage1(af1d_ctx *c, int s) {
   else bind1(c, n, b2, b1);
 }
 
-// From 2^20 indices on the check for quiet tiles is a small part of a stage
-#ifndef AF_QUIET1_MIN
-#define AF_QUIET1_MIN (1 << 20)
-#endif
 // Stages s0..s1 of a step
 int stages1(af1d_ctx *c, int s0, int s1, int reduce_dt) {
   AfDev d[3];
@@ -146,8 +142,7 @@ int stage1(af1d_ctx *c, int s, int reduce_dt) {
   if (c->cluster && !c->tm.on) return stages1(c, s, s, reduce_dt);
   const int b1 = (c->cur + 1) % 3, b2 = (c->cur + 2) % 3;
   bind_stage1(c, s);
-  // quiet tiles: from 2^20 cells on a stage takes about a millisecond, the check about 10 us
-  c->dev.lev = c->prm.pp_on && c->nf >= AF_QUIET1_MIN ? c->dev.quiet + 2 * af_quiet_tiles1d(c->g) : nullptr;
+  c->dev.lev = c->prm.pp_on && c->nf >= kQuiet1Min ? c->dev.quiet + 2 * af_quiet_tiles1d(c->g) : nullptr;
   af_launch_stage1d(c->dev, c->g, RK1_A[s], RK1_B[s], reduce_dt, c->stream, &c->tm);
   c->dev.lev = nullptr;
   CK1(cudaGetLastError(), "stage launch");

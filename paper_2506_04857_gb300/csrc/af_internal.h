@@ -133,7 +133,10 @@ bool af_small_grid(const AfGrid &g);   // which build the launchers below take
 // levels of the quiet tiles of the stage input; af_quiet_grid: whether a grid's stages use them
 void af_launch_quiet(const AfDev &d, const AfGrid &g, cudaStream_t s);
 bool af_quiet_grid(const AfGrid &g);
-inline size_t af_quiet_tiles(const AfGrid &g) { return (size_t)((g.nxa + 31) / 32) * ((g.nya + 3) / 4); }
+constexpr int kTileW = 32, kTileH = 4;   // index points of a block of the passes of a large grid: a quiet tile
+inline int af_tiles_x(const AfGrid &g) { return (g.nxa + kTileW - 1) / kTileW; }
+inline int af_tiles_y(const AfGrid &g) { return (g.nya + kTileH - 1) / kTileH; }
+inline size_t af_quiet_tiles(const AfGrid &g) { return (size_t)af_tiles_x(g) * af_tiles_y(g); }
 // the limiter slow paths over the work lists the point and cell passes filled: a short point list
 // of a large grid, and everything else
 void af_launch_points_slow(const AfDev &d, const AfGrid &g, double a, double b, cudaStream_t s);
@@ -233,6 +236,9 @@ void af_launch_stage1d(const AfDev &d, const AfGrid &g, double a, double b, int 
 int af_lat_step1d_cluster(int n);
 void af_lat_step1d(const AfDev *d, const AfGrid &g, int s0, int s1, int reduce_dt, int cluster, cudaStream_t s);
 size_t af_quiet_tiles1d(const AfGrid &g);
+constexpr int kTile1 = 128;        // indices of a 1D quiet tile, and of a block of the passes of a long grid
+// From 2^20 indices on the check for quiet tiles (about 10 us) is a small part of a stage (a millisecond)
+constexpr int kQuiet1Min = 1 << 20;
 void af_launch_dt1d(const AfDev &d, const AfGrid &g, cudaStream_t s);
 // divergence measures of Example 4.4 of the state bound in d.us into out[2]
 // (device); partials: 2 * af_divb_nblocks(g) doubles

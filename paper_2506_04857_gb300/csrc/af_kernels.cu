@@ -33,15 +33,7 @@ namespace {
 // Blocks of 256 threads per SM the batch kernels are compiled for: the fastest of a sweep (at
 // most 64 registers for the point pass, 80 for the point data, 128 for the cells: a 32-run ensemble
 // 21.6 -> 20.8 ms with them).
-#ifndef AF_KBPT
-#define AF_KBPT 4
-#endif
-#ifndef AF_KBPD
-#define AF_KBPD 3
-#endif
-#ifndef AF_KBCL
-#define AF_KBCL 2
-#endif
+constexpr int kBatchPt = 4, kBatchPd = 3, kBatchCl = 2;
 // Batches hand limited points and cells to work lists of their own runs, as single runs do: with
 // the slow paths inline the point pass spilled 2.2 kB a thread.
 // the nz parts of the work of a tile (DoF classes, face directions) are items of their own, one part
@@ -55,7 +47,7 @@ namespace {
     call;                                                         \
   }
 
-__global__ void __launch_bounds__(256, AF_KBPD) kb_pointdata(const AfRun *__restrict__ runs, const int4 *__restrict__ items,
+__global__ void __launch_bounds__(256, kBatchPd) kb_pointdata(const AfRun *__restrict__ runs, const int4 *__restrict__ items,
                                                     int nitems, int reduce_dt) {
   AF_BATCH_LOOP(5, b_pointdata(r->d, r->g, i, j, reduce_dt, z + 1));
 }
@@ -64,7 +56,7 @@ __global__ void kb_dt(const AfRun *__restrict__ runs, int nruns) {
   if (t < nruns) b_dt(runs[t].d, runs[t].g);
 }
 template <bool UP>
-__global__ void __launch_bounds__(256, AF_KBPT) kb_points(const AfRun *__restrict__ runs, const int4 *__restrict__ items,
+__global__ void __launch_bounds__(256, kBatchPt) kb_points(const AfRun *__restrict__ runs, const int4 *__restrict__ items,
                                                  int nitems, double a, double b) {
   AF_BATCH_LOOP(4, (b_points<false, UP, kPlain>(r->d, r->g, i, j, a, b, 0, z)));
 }
@@ -72,7 +64,7 @@ __global__ void __launch_bounds__(256) kb_faces(const AfRun *__restrict__ runs, 
                                                 int nitems) {
   AF_BATCH_LOOP(2, b_faces<false>(r->d, r->g, i, j, 0, z));
 }
-__global__ void __launch_bounds__(256, AF_KBCL) kb_cells(const AfRun *__restrict__ runs, const int4 *__restrict__ items,
+__global__ void __launch_bounds__(256, kBatchCl) kb_cells(const AfRun *__restrict__ runs, const int4 *__restrict__ items,
                                                 int nitems, double a, double b) {
   AF_BATCH_LOOP(1, (b_cells<false, true, true>(r->d, r->g, i, j, a, b, 0)));
 }
@@ -324,20 +316,14 @@ inline dim3 grid2(int nx, int ny) { return dim3((nx + 31) / 32, (ny + 3) / 4); }
 
 }  // namespace
 
-#ifndef AF_SMALL
-#define AF_SMALL 1216
-#endif
 // Small grids: up to two warps of a part per scheduler (152 SMs x 4 x 2 row tiles of 32).  There a
 // pass is one chain of dependent operations long and the short chains of AF_LAT pay; above it the
 // FP64 pipe fills and AF_LAT's additional operations cost (10 steps, AF_LAT against the other build:
 // 64 x 64 2036 against 2655 us, 128 x 128 2376 against 2843, 256 x 256 3009 against 2789).
-bool af_small_grid(const AfGrid &g) { return (long long)((g.nxa + 31) / 32) * g.nya <= AF_SMALL; }
+bool af_small_grid(const AfGrid &g) { return (long long)af_tiles_x(g) * g.nya <= 152 * 4 * 2; }
 
-#ifndef AF_QUIET_MIN
-#define AF_QUIET_MIN (1 << 19)
-#endif
 // From 2^19 index points on: a stage then takes over a millisecond, the check about 10 us.
-bool af_quiet_grid(const AfGrid &g) { return !g.special && g.pp_on && !g.upwind && (long long)g.nxa * g.nya >= AF_QUIET_MIN; }
+bool af_quiet_grid(const AfGrid &g) { return !g.special && g.pp_on && !g.upwind && (long long)g.nxa * g.nya >= 1 << 19; }
 void af_launch_quiet(const AfDev &d, const AfGrid &g, cudaStream_t s) { launch_quiet(d, g, s); }
 
 void af_launch_pointdata(const AfDev &d, const AfGrid &g, int reduce_dt, cudaStream_t s) {

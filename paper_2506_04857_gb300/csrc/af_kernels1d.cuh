@@ -1,6 +1,7 @@
 // af_kernels1d.cuh -- the 1D AF scheme (Sec. 4: the 1D tests use the 1D AF
 // scheme with the LLF FVS and without the Godunov-Powell source), included at
-// the end of af_kernels.cu so that it shares the 2D device functions.
+// the end of af_kernels.cu (the passes) and af_kernels_lat.cu (the step of a
+// short grid in one launch) so that it shares the 2D device functions.
 //
 // The 1D problem runs on the 2D data structures with ny = 1: class 0 holds the
 // cell averages (nx), class 1 the interface point values (nxa = nx, or nx + 1
@@ -433,7 +434,6 @@ __global__ void __launch_bounds__(3 * kStepThreads) k1_step(const __grid_constan
 }
 #else
 // Quiet tiles of 128 indices, as in 2D (levels d.lev, one per block)
-constexpr int kTile1 = 128;
 __device__ __forceinline__ int level1(const AfDev &d) { return d.lev ? d.lev[blockIdx.x] : 0; }
 __global__ void __launch_bounds__(kTile1) k1_quiet1(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g) {
   pass_begin();
@@ -598,6 +598,7 @@ void af_lat_step1d(const AfDev *d, const AfGrid &g, int s0, int s1, int reduce_d
 
 // threads per block: a warp until every SM has four of them, which is when the FP64 pipe is full
 static unsigned threads1d(const AfGrid &g) { return g.nxa <= 152 * kTile1 ? 32 : kTile1; }
+static_assert(kQuiet1Min > 152 * kTile1, "the levels of the 1D tiles are indexed by blocks of kTile1 indices");
 
 // One 1D stage: P1 (with the dt pass when reduce_dt), P2..P5 and the repair
 // pass; t (may be NULL) brackets each launch with an event pair.

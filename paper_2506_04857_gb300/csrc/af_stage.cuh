@@ -1803,7 +1803,7 @@ inline __host__ __device__ int frame_rows(const AfGrid &g, int ntx, int threads)
 // blockIdx.y could not hold the frame's rows of a very tall grid): a frame point (true), a point of
 // the inner tiles (false), or nothing to do (t.i < 0)
 __device__ __forceinline__ bool frame_tile(const AfGrid &g, int nx, Tile &t) {
-  const int threads = blockDim.x * blockDim.y, ntx = (nx + 31) / 32, rows = frame_rows(g, ntx, threads);
+  const int threads = blockDim.x * blockDim.y, ntx = (nx + kTileW - 1) / kTileW, rows = frame_rows(g, ntx, threads);
   const int by = blockIdx.x / ntx, bx = blockIdx.x - by * ntx;
   t = {-1, 0, (int)blockIdx.z};
   if (by < rows) {
@@ -2078,7 +2078,7 @@ __device__ __forceinline__ bool same_state(const AfDev &d, const AfGrid &g, int 
   return true;
 }
 __device__ __forceinline__ void b_quiet1(const AfDev &d, const AfGrid &g) {
-  const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 4, i = i0 + threadIdx.x, j = j0 + threadIdx.y;
+  const int i0 = blockIdx.x * kTileW, j0 = blockIdx.y * kTileH, i = i0 + threadIdx.x, j = j0 + threadIdx.y;
   const SV C = sview(d.us[3], g, 3);
   bool ok = true;
   // the energy at the corners first: it ends most tiles of a flow without quiet gas
@@ -2140,7 +2140,7 @@ __global__ void __launch_bounds__(128) k_quiet1(const __grid_constant__ AfDev d,
 __global__ void __launch_bounds__(128) k_quiet23(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                                  int pass) {
   pass_begin();
-  b_quiet23<32, 4, 3>(d, g, pass);
+  b_quiet23<kTileW, kTileH, 3>(d, g, pass);
 }
 // level of the block's tile (0 where no levels are kept)
 __device__ __forceinline__ int tile_level(const AfDev &d) {
@@ -2188,10 +2188,10 @@ __device__ __forceinline__ void quiet_final(const AfDev &d, const AfGrid &g, con
   if (g.bc == 1 && j == g.ny - 1) d.thy[o + g.nxa] = 1.0;
 }
 
-// Launch bounds of the stage kernels (128 threads): a kernel given AF_MINB_x
+// Launch bounds of the stage kernels (128 threads): a kernel given a number of
 // resident blocks per SM is capped at 65536 / (128 x blocks) registers; without
 // it ptxas picks the count.  The kernels keep the FP64 pipe and the integer
-// pipes busy at once; the defaults are the fastest of a sweep (point data and
+// pipes busy at once; the numbers are the fastest of a sweep (point data and
 // point pass at 8 blocks = 64 registers, cell pass at 5 = 96, faces at 9 = 56; the
 // final pass at the compiler's count).  On small grids a pass has fewer warps than the
 // chip has schedulers: one warp a block, and all the registers it asks for.
@@ -2202,30 +2202,13 @@ __device__ __forceinline__ void quiet_final(const AfDev &d, const AfGrid &g, con
 #define AF_LB_CL __launch_bounds__(32)
 #define AF_LB_FN __launch_bounds__(32)
 #else
-#define AF_LB(minb) __launch_bounds__(128, minb)
-#ifndef AF_MINB_PD
-#define AF_MINB_PD 8
-#endif
-#define AF_LB_PD AF_LB(AF_MINB_PD)
-#ifndef AF_MINB_PT
-#define AF_MINB_PT 8
-#endif
-#define AF_LB_PT AF_LB(AF_MINB_PT)
+#define AF_LB_PD __launch_bounds__(128, 8)
+#define AF_LB_PT __launch_bounds__(128, 8)
 // faces: 56 registers (9 blocks) 706 us at 1536 x 1536, 72 (the compiler's count) 738, 64 716; the
 // ghost code of special sides would spill at that
-#ifndef AF_MINB_FC
-#define AF_MINB_FC 9
-#endif
-#define AF_LB_FC AF_LB(GB ? 1 : AF_MINB_FC)
-#ifndef AF_MINB_CL
-#define AF_MINB_CL 5
-#endif
-#define AF_LB_CL AF_LB(AF_MINB_CL)
-#ifdef AF_MINB_FN
-#define AF_LB_FN AF_LB(AF_MINB_FN)
-#else
+#define AF_LB_FC __launch_bounds__(128, GB ? 1 : 9)
+#define AF_LB_CL __launch_bounds__(128, 5)
 #define AF_LB_FN __launch_bounds__(128)
-#endif
 #endif
 __global__ void AF_LB_PD k_pointdata(const __grid_constant__ AfDev d, const __grid_constant__ AfGrid g,
                                                    int reduce_dt) {
@@ -2348,10 +2331,7 @@ struct Shape {
 #ifdef AF_LAT
 constexpr int kRows = 1;
 #else
-#ifndef AF_ROWS
-#define AF_ROWS 4
-#endif
-constexpr int kRows = AF_ROWS;
+constexpr int kRows = kTileH;   // the levels of the quiet tiles are indexed by the blocks of the passes
 #endif
 // One pass, launched programmatically dependent on the pass before it in the stream
 template <class... P, class... A>
@@ -2368,20 +2348,20 @@ void pass(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t s, A... args) {
   cudaLaunchKernelEx(&c, k, P(args)...);
 }
 inline Shape shape(int nx, int ny, int nz) {
-  return {dim3((nx + 31) / 32, (ny + kRows - 1) / kRows, nz), dim3(32, kRows)};
+  return {dim3((nx + kTileW - 1) / kTileW, (ny + kRows - 1) / kRows, nz), dim3(kTileW, kRows)};
 }
 // of a pass that resolves ghosts: with the rows of blocks of the frame
 inline Shape shape(const AfGrid &g, int nx, int ny, int nz) {
   Shape h = shape(nx, ny, nz);
-  if (g.special) h.g = dim3(h.g.x * (h.g.y + frame_rows(g, (int)h.g.x, 32 * kRows)), 1, nz);
+  if (g.special) h.g = dim3(h.g.x * (h.g.y + frame_rows(g, (int)h.g.x, kTileW * kRows)), 1, nz);
   return h;
 }
 
 // levels of the quiet tiles of the stage input (d.quiet: three bytes per tile; the last is d.lev)
 void launch_quiet(const AfDev &d, const AfGrid &g, cudaStream_t s) {
-  const dim3 gr((g.nxa + 31) / 32, (g.nya + 3) / 4);
+  const dim3 gr(af_tiles_x(g), af_tiles_y(g));
   const int nb = (int)((gr.x * gr.y + 127) / 128);
-  pass(k_quiet1, gr, dim3(32, 4), s, d, g);
+  pass(k_quiet1, gr, dim3(kTileW, kTileH), s, d, g);
   pass(k_quiet23, nb, 128, s, d, g, 0);
   pass(k_quiet23, nb, 128, s, d, g, 1);
 }

@@ -33,3 +33,12 @@ def test_dependent_kernels_wait_first():
 
 def test_no_early_start():
     assert "launch_dependents" not in "".join(code(f) for f in FILES)
+
+
+def test_no_build_time_overrides():
+    """Tile sizes, lines between forms and launch bounds stand once: a size that a build could change in
+    one place and not in the others (the quiet tiles and the blocks of the passes) would skip tiles."""
+    for name in sorted(os.listdir(CSRC)):
+        if name == "af_internal.h":   # AF_NCOEF, a public constant af.h defines as well
+            continue
+        assert not re.search(r"#\s*ifn?def\s+AF_(?!LAT\b)", code(name)), name
