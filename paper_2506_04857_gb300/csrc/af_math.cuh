@@ -387,7 +387,10 @@ __device__ __forceinline__ double sub_i(double a, double b) { return add_i(a, ne
 // bits.  The alignment drops less than one unit of 2^-G ulp of the largest term per
 // term, so the error is below sum |c_q| 2^-G ulp (1/4 ulp for the 5-point sum) plus
 // the final rounding, against up to 5 ulp for the chain of FP64 sums it replaces;
-// equal terms whose coefficients cancel give exactly 0.  An alignment costs about 12
+// equal terms whose coefficients cancel give exactly 0.  (Mean error of the 5-point sum on random
+// lines 1.8e-16 of the largest term, of the chain 2.7e-16.  The chain is the more exact one only where
+// the outer terms cancel in pairs, u0 = -u4 and u1 = -u3: it then keeps a small middle value whole,
+// this sum only its bits down to 2^-6 ulp of the largest term.)  An alignment costs about 12
 // integer instructions and the normalisation 18: the 5-point sum keeps the integer ALUs
 // (16 lanes per scheduler) busy for about 180 cycles where its four FP64 instructions
 // kept the FP64 pipe busy for 300, and both run at once.  The sum is that of magnitudes

@@ -555,8 +555,10 @@ __device__ __forceinline__ int upwind_sign(const AfGrid &g, double vl) {
 // into acc (per component), with F^pm = (F +- alpha U)/2.  Writing out D+ and D-:
 // (D+F+ + D-F-) h = ((F0 - F4) + 4 (F3 - F1) + alpha ((U0 + U4) - 4 (U1 + U3) + 6 U2)) / 2.
 // Also returns 2h times the derivative of B_l for the point source in dBl (b_line).
-// RHS: the semi-discrete right-hand side keeps the second difference in FP64 (it serves finite
-// differences, and its rounding is what those see).
+// RHS: the semi-discrete right-hand side keeps the chain of FP64 sums.  Both forms are within rounding;
+// finite differences of the right-hand side with small steps see which one it is, and those in use
+// were set with the chain.  U + dt rhs(U) therefore agrees with a forward-Euler stage to rounding,
+// not bit for bit.
 // The second difference of U runs on the integer pipes (up5): the point pass is bound by
 // the FP64 pipe (84 % busy, integer ALUs 14 %).  Orszag-Tang 1536^2: the pass 1813 -> 1555 us;
 // blast 1024^2: 838 -> 694 us.  The flux difference stays on the FP64 pipe: moved too, the

@@ -1,6 +1,9 @@
 """The second difference of a 5-point FVS line in fixed point (af_math.cuh up5): components over
 the whole exponent range, exact zeros, mixed signs and jumps, through unlimited stages against the
 oracle (dt of order 1: the update is as large as the state)."""
+import math
+from fractions import Fraction as F
+
 import numpy as np
 import pytest
 
@@ -77,3 +80,51 @@ def test_jumps(bits):
     a, b = stage(pb, U)[3], oracle_stage(pb, U)[3]
     for k in range(8):
         assert np.abs(a[k] - b[k]).max() <= 1e-12 * np.abs(b[k]).max(), (k, bits)
+
+
+# The sum itself to its own error bound.  Gas at rest under one pressure without a field: every flux
+# difference is 0 and a corner's density becomes rho - c alpha up, up = u0 + u4 - 4 (u1 + u3) + 6 u2 of
+# its x line (its y line is constant), c a power of two.  up may be off by a quarter of a unit of
+# the largest term's last place (the bits dropped in the alignment) and half of one of its own
+# (rounding); alpha (two square roots, a reciprocal, three products), its product with up and the
+# update add at most 8 half units of the result's.  Lines: ordinary values, jumps of 2^bits, and
+# lines of equal or exactly cancelling values, where up is 0 and the density must not change.
+@pytest.mark.parametrize("kind", ["smooth", "cancel", 0, 1, 5, 6, 7, 31, 52, 58, 59, 64, 70])
+def test_error_bound(kind):
+    nx, ny, p, gamma = 64, 4, 1.0, 1.5
+    rng = np.random.default_rng(11)
+    x = np.arange(2 * nx) / (2 * nx)   # corners at the even places, y-faces at the odd ones
+    if kind == "smooth":
+        rho = 1.0 + 0.3 * np.sin(2 * np.pi * x) + 0.1 * np.cos(6 * np.pi * x)
+    elif kind == "cancel":   # cubics with coefficients of a few bits, and constant stretches
+        k = np.arange(2 * nx)
+        rho = np.where(k % 32 < 16, 1.0 + ((k % 16) - 8.0) ** 3 / 4096.0, 1.375)
+    else:
+        rho = (1.0 + rng.random(2 * nx)) * np.where(rng.random(2 * nx) < 0.3, 2.0 ** kind, 1.0)
+    C, Y = rho[0::2], rho[1::2]
+    U = []
+    for r in (Y, C, Y, C):   # averages and x-faces lie on other lines; x-faces as the corners above and below
+        u = np.zeros((8, ny, nx))
+        u[0], u[7] = r, p / (gamma - 1.0)
+        U.append(u)
+    s = af.Solver(nx, ny, gamma, ai.PERIODIC, domain=(0.0, 1.0, 0.0, 1.0), kappa=0.0, pp_on=False)
+    s.set_state([torch.from_numpy(u).cuda() for u in U])
+    s.stage(0, 2.0 ** 20)
+    got = s.get_stage(device=False)[3][0]
+    s.close()
+    c = F(2) ** 25
+    zeros = 0
+    for i in range(nx):
+        u = [C[i - 1], Y[i - 1], C[i], Y[i], C[(i + 1) % nx]]
+        up = F(u[0]) + F(u[4]) - 4 * (F(u[1]) + F(u[3])) + 6 * F(u[2])
+        al = F(math.sqrt(gamma * p / min(u)))
+        want = F(u[2]) - c * al * up
+        bound = c * al * (F(1, 4) * F(np.spacing(max(u))) + F(1, 2) * F(np.spacing(abs(float(up)))))
+        bound += 8 * F(1, 2) * F(np.spacing(abs(float(want))))
+        for j in range(ny):
+            if up == 0:
+                zeros += 1
+                assert got[j, i] == u[2]
+            else:
+                assert abs(F(got[j, i]) - want) <= bound, (i, j, float(up))
+    assert kind != "cancel" or zeros > nx
