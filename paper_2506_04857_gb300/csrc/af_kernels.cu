@@ -20,8 +20,9 @@
 //                    of the parametrized flux limiter (Sec. 3.2) -> Lambda.
 //   P5 k_final     : per cell: unique face coefficients (step (3)), limited
 //                    update, round-off check, RK combination.
-// A one-thread repair kernel applies the round-off shrink of Remark 4.1 to
-// the (rare) cell averages that leave the admissible set.
+// Points and cells whose limiters may act go to work lists (k_points_slow,
+// k_lists).  A one-thread repair kernel applies the round-off shrink of Remark
+// 4.1 to the (rare) cell averages that leave the admissible set.
 //
 // Limiter fast paths: where the paper's limiter provably returns theta = 1
 // (all tested quantities clear 1e-13 by a wide margin) the blend is skipped;
@@ -318,11 +319,13 @@ inline dim3 grid2(int nx, int ny) { return dim3((nx + 31) / 32, (ny + 3) / 4); }
 
 // Small grids: up to two warps of a part per scheduler (152 SMs x 4 x 2 row tiles of 32).  There a
 // pass is one chain of dependent operations long and the short chains of AF_LAT pay; above it the
-// FP64 pipe fills and AF_LAT's additional operations cost (10 steps, AF_LAT against the other build:
-// 64 x 64 2036 against 2655 us, 128 x 128 2376 against 2843, 256 x 256 3009 against 2789).
+// FP64 pipe fills and AF_LAT's additional operations cost (a step of Orszag-Tang, AF_LAT against the
+// other build: 96 x 96 162 against 238 us, 128 x 128 203 and 262, 192 x 192 344 and 399, 256 x 256 592
+// and 542).
 bool af_small_grid(const AfGrid &g) { return (long long)af_tiles_x(g) * g.nya <= 152 * 4 * 2; }
 
-// From 2^19 index points on: a stage then takes over a millisecond, the check about 10 us.
+// From 2^19 index points on: a stage then takes over a millisecond, the check about 10 us (46 us of
+// 8 ms at 2048 x 2048).
 bool af_quiet_grid(const AfGrid &g) { return !g.special && g.pp_on && !g.upwind && (long long)g.nxa * g.nya >= 1 << 19; }
 void af_launch_quiet(const AfDev &d, const AfGrid &g, cudaStream_t s) { launch_quiet(d, g, s); }
 

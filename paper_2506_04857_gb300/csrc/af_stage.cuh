@@ -936,7 +936,7 @@ __device__ __forceinline__ void b_point(const AfDev &d, const AfGrid &g, const i
         for (int k = 0; k < 8; ++k) acc[k] = out[k];
       }
     } else if (!clear_of_floor(acc, g)) {
-      // slow path in k_points_slow, over a dense list (the warp does not wait here); the high-order
+      // slow path in the list passes, over a dense list (the warp does not wait here); the high-order
       // update waits there in the point's own place of the output
       const int slot = enqueue(d.st, &d.st->npq, d.pq_cap);
       if (slot >= 0) d.pq[slot] = (cls << 28) | (int)op;
@@ -1505,7 +1505,7 @@ __device__ __forceinline__ void b_cells(const AfDev &d, const AfGrid &g, const i
         if (!PL && d.frz) {
         } else if (fast) {
           Lam[0] = Lam[1] = Lam[2] = Lam[3] = 1.0;
-        } else {   // step (1) here, the box of step (2) in k_cells_slow over a dense list
+        } else {   // step (1) here, the box of step (2) in k_lists over a dense list
           int sl = 0;
           double eps_rho, eps_p;
           cell_source_limit(Ullf, dS, dtts, g, L1, sl, th_src, eps_rho, eps_p);
@@ -2068,10 +2068,13 @@ __device__ __forceinline__ void b_cells_lists(const AfDev &d, const AfGrid &g, c
 // sensor values up to 3, point data up to 4; each pass reaches one index, so one tile per pass
 // (a last tile may hold a single row or column).  The rest is not touched, but for the
 // Runge-Kutta combination.  Grids with reflective or inflow sides, recorded or frozen stages
-// and small grids (whose passes are as short as a launch) do not take it.  Without quiet
-// tiles the check costs one load per point and class and three launches (Orszag-Tang 1536 x 1536:
-// 14.12 -> 14.3 ms for a step with its copies); the 2048 x 2048 blast, 1/6 of it disturbed, takes
-// 19.7 ms for two steps instead of 45.4.
+// and small grids (whose passes are as short as a launch) do not take it.
+// Averages and points have to be equal: data whose averages come from a quadrature that leaves them
+// a rounding off the points, like the benchmark's blast, hold no such tile, and pay for the check:
+// one load per point and class and three launches, 46 us of a stage of 8 ms at 2048 x 2048.  A
+// 2048 x 2048 blast that is uniform outside its disturbed sixth takes 17.2 ms for its first two
+// steps with the copies of the state, 45.4 without the levels; the gain shrinks as the
+// disturbance grows.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ bool same_state(const AfDev &d, const AfGrid &g, int cls, int ia, int ja, int ib, int jb) {
   const SV C = sview(d.us[cls], g, cls);
