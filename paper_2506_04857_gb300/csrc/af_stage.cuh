@@ -2209,9 +2209,10 @@ __device__ __forceinline__ void quiet_final(const AfDev &d, const AfGrid &g, con
 #else
 #define AF_LB_PD __launch_bounds__(128, 8)
 #define AF_LB_PT __launch_bounds__(128, 8)
-// faces: 56 registers (9 blocks) 706 us at 1536 x 1536, 72 (the compiler's count) 738, 64 716; the
-// ghost code of special sides would spill at that
-#define AF_LB_FC __launch_bounds__(128, GB ? 1 : 9)
+// faces: 56 registers (9 blocks) 706 us at 1536 x 1536, 72 (the compiler's count) 738, 64 716; with
+// special sides, whose frame's ghost code spills at that, jets 512 x 1536 235 us, 64 243, 94 (the
+// compiler's count) 357
+#define AF_LB_FC __launch_bounds__(128, 9)
 #define AF_LB_CL __launch_bounds__(128, 5)
 #define AF_LB_FN __launch_bounds__(128)
 #endif
