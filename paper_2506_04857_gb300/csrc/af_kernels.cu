@@ -324,7 +324,7 @@ inline dim3 grid2(int nx, int ny) { return dim3((nx + 31) / 32, (ny + 3) / 4); }
 // and 542).
 bool af_small_grid(const AfGrid &g) { return (long long)af_tiles_x(g) * g.nya <= 152 * 4 * 2; }
 
-// From 2^19 index points on: a stage then takes over a millisecond, the check about 10 us (46 us of
+// From 2^19 index points on: a stage then takes over a millisecond, the check about 10 us (40 us of
 // 8 ms at 2048 x 2048).
 bool af_quiet_grid(const AfGrid &g) { return !g.special && g.pp_on && !g.upwind && (long long)g.nxa * g.nya >= 1 << 19; }
 void af_launch_quiet(const AfDev &d, const AfGrid &g, cudaStream_t s) { launch_quiet(d, g, s); }

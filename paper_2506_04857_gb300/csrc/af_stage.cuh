@@ -2071,7 +2071,7 @@ __device__ __forceinline__ void b_cells_lists(const AfDev &d, const AfGrid &g, c
 // and small grids (whose passes are as short as a launch) do not take it.
 // Averages and points have to be equal: data whose averages come from a quadrature that leaves them
 // a rounding off the points, like the benchmark's blast, hold no such tile, and pay for the check:
-// one load per point and class and three launches, 46 us of a stage of 8 ms at 2048 x 2048.  A
+// one load per point and class and three launches, 40 us of a stage of 8 ms at 2048 x 2048.  A
 // 2048 x 2048 blast that is uniform outside its disturbed sixth takes 17.2 ms for its first two
 // steps with the copies of the state, 45.4 without the levels; the gain shrinks as the
 // disturbance grows.
