@@ -101,7 +101,7 @@ EXEC_FP64_DIVB = {}
 # (the kernel k_lists: the cell list, and a long point list), the names af_timing reports them
 # under.
 EXEC_FP64 = {
-    "blast_low_beta": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "1d1c64652d4575d4407fc99d1a7f6536cb27b2c1", "kernels": {
+    "blast_low_beta": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "bda2d9120f983209357f69cd3b2aeb590d6ca96f", "kernels": {
         "k_pointdata": {"dadd": 98.04, "dmul": 0.01, "dfma": 188.15, "pipe": 286.19, "dram_bytes": 1362.2, "int_mul": 124.09, "int_add": 0.00},
         "k_points": {"dadd": 95.13, "dmul": 6.01, "dfma": 160.29, "pipe": 261.42, "dram_bytes": 1630.5, "int_mul": 40.06, "int_add": 184.28},
         "k_points_slow": {"dadd": 0.24, "dmul": 0.29, "dfma": 0.51, "pipe": 1.07, "dram_bytes": 2.7, "int_mul": 0.02, "int_add": 0.00},
@@ -110,7 +110,7 @@ EXEC_FP64 = {
         "k_cells_slow": {"dadd": 0.06, "dmul": 0.18, "dfma": 0.20, "pipe": 0.54, "dram_bytes": 0.8, "int_mul": 0.00, "int_add": 0.00},
         "k_final": {"dadd": 0.00, "dmul": 0.00, "dfma": 21.33, "pipe": 21.33, "dram_bytes": 327.3, "int_mul": 8.33, "int_add": 16.00},
     }},
-    "orszag_tang": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "1d1c64652d4575d4407fc99d1a7f6536cb27b2c1", "kernels": {
+    "orszag_tang": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "bda2d9120f983209357f69cd3b2aeb590d6ca96f", "kernels": {
         "k_pointdata": {"dadd": 98.00, "dmul": 0.00, "dfma": 188.00, "pipe": 286.00, "dram_bytes": 1179.0, "int_mul": 124.00, "int_add": 0.00},
         "k_points": {"dadd": 96.00, "dmul": 6.00, "dfma": 166.00, "pipe": 268.00, "dram_bytes": 1570.4, "int_mul": 42.00, "int_add": 184.00},
         "k_points_slow": {"dadd": 0.00, "dmul": 0.00, "dfma": 0.00, "pipe": 0.00, "dram_bytes": 0.2, "int_mul": 0.00, "int_add": 0.00},
@@ -119,7 +119,7 @@ EXEC_FP64 = {
         "k_cells_slow": {"dadd": 0.00, "dmul": 0.00, "dfma": 0.00, "pipe": 0.00, "dram_bytes": 0.3, "int_mul": 0.00, "int_add": 0.00},
         "k_final": {"dadd": 0.00, "dmul": 0.00, "dfma": 21.33, "pipe": 21.33, "dram_bytes": 274.9, "int_mul": 8.33, "int_add": 16.00},
     }},
-    "jets": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "1d1c64652d4575d4407fc99d1a7f6536cb27b2c1", "kernels": {
+    "jets": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "bda2d9120f983209357f69cd3b2aeb590d6ca96f", "kernels": {
         "k_pointdata": {"dadd": 98.05, "dmul": 0.00, "dfma": 188.18, "pipe": 286.22, "dram_bytes": 1345.6, "int_mul": 124.13, "int_add": 0.00},
         "k_points": {"dadd": 100.90, "dmul": 6.10, "dfma": 160.23, "pipe": 267.24, "dram_bytes": 1739.3, "int_mul": 39.14, "int_add": 212.74},
         "k_points_slow": {"dadd": 0.03, "dmul": 0.04, "dfma": 0.06, "pipe": 0.14, "dram_bytes": 0.2, "int_mul": 0.00, "int_add": 0.00},
@@ -128,7 +128,7 @@ EXEC_FP64 = {
         "k_cells_slow": {"dadd": 0.03, "dmul": 0.09, "dfma": 0.10, "pipe": 0.27, "dram_bytes": 0.1, "int_mul": 0.00, "int_add": 0.00},
         "k_final": {"dadd": 0.00, "dmul": 0.00, "dfma": 21.33, "pipe": 21.33, "dram_bytes": 319.7, "int_mul": 8.33, "int_add": 16.00},
     }},
-    "rarefaction_lattice": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "1d1c64652d4575d4407fc99d1a7f6536cb27b2c1", "kernels": {
+    "rarefaction_lattice": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "bda2d9120f983209357f69cd3b2aeb590d6ca96f", "kernels": {
         "k_pointdata": {"dadd": 98.50, "dmul": 1.87, "dfma": 192.23, "pipe": 293.05, "dram_bytes": 1176.1, "int_mul": 124.00, "int_add": 0.00},
         "k_points": {"dadd": 96.00, "dmul": 6.00, "dfma": 166.80, "pipe": 268.77, "dram_bytes": 1558.6, "int_mul": 39.81, "int_add": 183.99},
         "k_points_slow": {"dadd": 0.00, "dmul": 0.00, "dfma": 0.00, "pipe": 0.00, "dram_bytes": 0.2, "int_mul": 6.84, "int_add": 0.00},
@@ -137,7 +137,7 @@ EXEC_FP64 = {
         "k_cells_slow": {"dadd": 100.40, "dmul": 127.62, "dfma": 368.50, "pipe": 622.45, "dram_bytes": 855.2, "int_mul": 0.00, "int_add": 0.00},
         "k_final": {"dadd": 0.00, "dmul": 2.86, "dfma": 24.20, "pipe": 27.05, "dram_bytes": 275.0, "int_mul": 8.33, "int_add": 13.14},
     }},
-    "blast1d": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "0c6d616c6256672b6680478156df2e0d43e45fcc", "kernels": {
+    "blast1d": {"source": "profiles/fp64ops_stage_kernels.md", "digest": "fe36faa10ce2513e904607a8fb56912d942674ba", "kernels": {
         "k1_pointdata": {"dadd": 0.69, "dmul": 0.01, "dfma": 2.75, "pipe": 3.45, "dram_bytes": 21.6, "int_mul": 0.00, "int_add": 0.00},
         "k1_points": {"dadd": 0.01, "dmul": 0.00, "dfma": 5.35, "pipe": 5.36, "dram_bytes": 162.5, "int_mul": 0.00, "int_add": 0.00},
         "k1_faces": {"dadd": 0.02, "dmul": 0.01, "dfma": 0.01, "pipe": 0.04, "dram_bytes": 0.2, "int_mul": 0.00, "int_add": 0.00},
@@ -145,7 +145,7 @@ EXEC_FP64 = {
         "k1_final": {"dadd": 0.00, "dmul": 0.00, "dfma": 5.34, "pipe": 5.34, "dram_bytes": 161.2, "int_mul": 0.00, "int_add": 0.00},
     }},
 }
-EXEC_FP64_DIVB["blast_low_beta"] = {"source": "profiles/divb_blast512.md", "digest": "1d1c64652d4575d4407fc99d1a7f6536cb27b2c1",
+EXEC_FP64_DIVB["blast_low_beta"] = {"source": "profiles/divb_blast512.md", "digest": "bda2d9120f983209357f69cd3b2aeb590d6ca96f",
                                      "dadd": 67.99, "dmul": 19.01, "dfma": 57.03, "pipe": 143.98}
 # FP64 roofline from unit counts and clock: the GB300 SM retires 2 DFMA thread
 # instructions per cycle (ncu: sm__sass_thread_inst_executed_op_dfma_pred_on

@@ -81,7 +81,7 @@ struct AfStatus {
 struct AfDev {
   const double *un[4];    // U^n
   const double *us[4];    // stage input U^(s)
-  double *uo[4];          // stage output
+  double *uo[4];          // stage output, a buffer that overlaps neither: listed points wait in it
   double *pd[5];          // point data, classes 0..3 and cell centres (4)
   double *uc;             // limited cell-centre values
   double *phi;            // phi_1x, phi_1y, phi_2, phi_3
